@@ -29,6 +29,22 @@
 
 namespace lbe {
 
+template <int S>
+struct ColTable {
+    static constexpr auto cols = make_columns<S>();
+    static constexpr int count = column_count(S);
+};
+
+template <int S, int TZ>
+__host__ __device__ constexpr bool col_needs(unsigned mask, int k) {
+    // plane offset k (relative to the first output) is read by some output t
+    for (int t = 0; t < TZ; ++t) {
+        int ez = k - t;
+        if (ez >= -S && ez <= S && (mask >> (ez + S)) & 1u) return true;
+    }
+    return false;
+}
+
 // e_CC of the point (ex, ey, ez)
 template <int CC>
 __host__ __device__ constexpr int comp(int ex, int ey, int ez) {

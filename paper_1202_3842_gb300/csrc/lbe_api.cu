@@ -3,6 +3,7 @@
 // runs in the kernels of lbe_kernels.cu and lbe_shell.cu on the context stream.
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -14,6 +15,7 @@
 #include "lbe_device.cuh"
 #include "lbe_launch.h"
 #include "lbe_shell.cuh"
+#include "lbe_shell_march.cuh"
 
 using namespace lbe;
 
@@ -43,10 +45,6 @@ struct PairShell {
 
 }  // namespace
 
-#ifndef LBE_SHELL_STREAMS
-#define LBE_SHELL_STREAMS 2
-#endif
-
 struct lbe_ctx {
     lbe_config cfg{};
     Prec prec = Prec::F32;
@@ -70,6 +68,10 @@ struct lbe_ctx {
     int cur = 0;
     Buf solid, mask, V, phi, amp, F;
     Buf npad, gab, gnpad, C;
+    Buf npad2;  // FP32 direct shell force: padded deviations n_b - ref_n [M][P]; gnpad then holds g_ab n_b - ref_g
+    double ref_n[MAXS] = {0}, ref_g[MAXS][MAXS] = {{0}};
+    bool ref_dirty = true;
+    ShellMarchMaps *march_maps = nullptr;
     Buf flux_buf, flux_acc, flux_last;
     Buf err;
     Buf scratch64;  // FP64 scratch for getters: n [M][N] + J [M][3][N] (+ more)
@@ -112,10 +114,6 @@ struct lbe_ctx {
     long long launches = 0;
     long long steps_since_check = 0;
     std::string last_error;
-
-    // second stream of the shell stage: the pair launches of odd species run there (created on first use)
-    cudaStream_t side = nullptr;
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
 
     // stage timing
     bool timing = false;
@@ -325,13 +323,13 @@ int shell_count(int S) {
     return k;
 }
 
-// Cost rule of LBE_SHELL_AUTO, from measurements on GB300 (512x128x128 two-species channel, pair
-// diameters 4, 5, 5, 6; 256^3 one-species well, diameter 6).  The spectral form replaces the contact
-// kernel and the shell stencil; the stencil costs a fixed time per node and shell point, the spectral
-// form a fixed time per grid point and pair.  Counting the contact kernel's time on the direct side,
-// the two break even at a mean shell of about 280 (well) to 323 (channel) points per pair in FP32,
-// scaled by the lattice over the grid, and about 100 in FP64, where the stencil is bound by the FP64
-// rate.  The constants lean to the stencil.
+// Cost rule between the spectral form and the point-by-point stencil, from measurements on GB300 (512x128x128
+// two-species channel, pair diameters 4, 5, 5, 6; 256^3 one-species well, diameter 6): the stencil costs a
+// fixed time per node and shell point, the spectral form a fixed time per grid point and pair, and they break
+// even at a mean shell of about 320 points per pair in FP32 and 110 in FP64, scaled by the lattice over the
+// grid.  The shell transpose of the adjoint follows it (its stencil is 2.6 times the cost), and so does the
+// forward form of lattices of fewer than DIRECT_NODES nodes, FP64 and the rest of what direct_cheaper
+// leaves.
 bool spectral_cheaper(const lbe_ctx *c, bool f64, double stencil_factor = 1.0) {
     long long pts = 0;
     int Smax = 0;
@@ -346,6 +344,15 @@ bool spectral_cheaper(const lbe_ctx *c, bool f64, double stencil_factor = 1.0) {
     const double even = (f64 ? 110.0 : 320.0) / stencil_factor;
     return spectral_shape_ok(c, Smax) && (double)pts * (double)g.N > even * (double)c->pairs.size() * Nr;
 }
+
+// Whether the marching kernels (lbe_shell_march.cuh, lbe_contact.cuh) take the forward force under
+// LBE_SHELL_AUTO.  FP32, K2 + K3 on GB300: 738 against 1146 us on the 256^3 well of diameter 6, 533 against 602 us
+// on a 192^3 well of diameter 8 (the widest they take), 1100 against 2390 us on the 512x128x128 channel of
+// diameters 4 and 6, 51 against 95 us on a 64^3 well of diameter 6: direct wherever a stencil is compiled.
+// Lattices below DIRECT_NODES nodes are bound by launches in either form and keep the rule above, which
+// programs that record the method of a small lattice rely on.
+constexpr long long DIRECT_NODES = 16384;
+bool direct_cheaper(const lbe_ctx *c, bool f64) { return !f64 && c->g.N >= DIRECT_NODES; }
 
 // The pairs as the spectral kernels see them (shell index into the table of distinct shells), the
 // distinct shells, and the grid: the lattice along periodic axes, at least Smax zero planes beyond it
@@ -593,15 +600,16 @@ lbe_status prepare(lbe_ctx *c) {
                 c->pairs.push_back(ps);
                 H = std::max(H, S);
             }
-        // K3 method: the direct stencil, or the spectral form for FP64 (bound by the FP64 rate) and
-        // for diameters without a compiled stencil
+        // K3 method: the direct stencil, or the spectral form where the rules above find it cheaper and for
+        // diameters without a compiled stencil
         c->spectral = false;
         if (!c->pairs.empty()) {
             if (c->shell_method == LBE_SHELL_DIRECT && !direct_ok)
                 return fail(c, LBE_ERR_UNSUPPORTED,
                             "a pair diameter has no compiled direct shell stencil (the spectral method takes it)");
             c->spectral = c->shell_method == LBE_SHELL_SPECTRAL ||
-                          (c->shell_method == LBE_SHELL_AUTO && (!direct_ok || spectral_cheaper(c, f64)));
+                          (c->shell_method == LBE_SHELL_AUTO &&
+                           (!direct_ok || (!direct_cheaper(c, f64) && spectral_cheaper(c, f64))));
         }
         // ball radii
         ContactParams cp{};
@@ -617,6 +625,8 @@ lbe_status prepare(lbe_ctx *c) {
         }
         if (RB > 4) return fail(c, LBE_ERR_UNSUPPORTED, "ball radius sigma/2 above 4 lattice units");
         H = std::max(H, RB);
+        // the marching kernels' tiles start on 16-byte boundaries of the padded rows
+        if (!c->pairs.empty()) H = (H + 3) / 4 * 4;
         c->RB = RB;
         c->H = H;
         Grid &g = c->g;
@@ -657,23 +667,30 @@ lbe_status prepare(lbe_ctx *c) {
         c->cparams = cp;
         const size_t rb = real_bytes(c);
         TRY(dev_alloc(c, c->npad, rb * c->M * g.P));
-        // g_ab n_b of every ordered pair for the direct shell stencil: FP32 stores the interleaved pair
-        // (n_b, g_ab n_b), 8 bytes per node (the spectral form keeps its own grid fields instead)
-        const size_t gnb = (f64 ? rb : 2 * rb) * c->M * c->M * g.P;
+        // g_ab n_b of every ordered pair for the direct shell stencil (the spectral form keeps its own grid
+        // fields instead); FP32 keeps deviations of n_b and g_ab n_b from reference values
+        const size_t gnb = rb * c->M * c->M * g.P;
         if (!c->spectral) TRY(dev_alloc(c, c->gnpad, gnb));
+        if (!c->spectral && !f64) TRY(dev_alloc(c, c->npad2, rb * c->M * g.P));
+        c->ref_dirty = true;
         TRY(dev_alloc(c, c->gab, rb * c->M * c->M * g.N));
         TRY(dev_alloc(c, c->C, rb * c->M * 3 * g.N));
         CK(cudaMemsetAsync(c->npad.p, 0, rb * c->M * g.P, c->stream), "memset npad");
-        if (!c->spectral) CK(cudaMemsetAsync(c->gnpad.p, 0, gnb, c->stream), "memset gnpad");
+        if (!c->spectral && f64) CK(cudaMemsetAsync(c->gnpad.p, 0, gnb, c->stream), "memset gnpad");
+        if (!c->march_maps && !f64) {
+            c->march_maps = new (std::nothrow) ShellMarchMaps;
+            if (!c->march_maps) return fail(c, LBE_ERR_OOM, "host allocation failed");
+        }
         CK(cudaMemsetAsync(c->C.p, 0, rb * c->M * 3 * g.N, c->stream), "memset C");
         for (auto &ps : c->pairs) {
             if (c->spectral) break;
-            char *nb = (char *)c->npad.p + rb * ps.b * g.P;
-            char *gn = (char *)c->gnpad.p + (f64 ? rb : 2 * rb) * (ps.a * c->M + ps.b) * g.P;
+            const int ab = ps.a * c->M + ps.b;
+            char *nb = (char *)(f64 ? c->npad.p : c->npad2.p) + rb * ps.b * g.P;
+            char *gn = (char *)c->gnpad.p + rb * ab * g.P;
             int bx = 0, by = 0;
             shell_box(f64, ps.S, &bx, &by);
-            if (f64) TRY(make_map(c, &ps.map_n, nb, bx, by));
-            TRY(make_map(c, &ps.map_gn, gn, bx, by, !f64));
+            TRY(make_map(c, f64 ? &ps.map_n : &c->march_maps->n[ab], nb, bx, by));
+            TRY(make_map(c, f64 ? &ps.map_gn : &c->march_maps->gn[ab], gn, bx, by));
         }
         {
             int bx = 0, by = 0;
@@ -717,6 +734,44 @@ StepParams step_params(const lbe_ctx *c) {
     return sp;
 }
 
+// Reference values of the FP32 shell fields: the species' mean densities n0 and the contact values of a uniform
+// fluid at those densities.  They only set where the sums round (an odd kernel takes no constant), so a
+// context without a mean density uses 0.  A change refills the fields, whose ghosts beyond closed axes
+// stand for density 0.
+lbe_status update_refs(lbe_ctx *c) {
+    double rn[MAXS] = {0}, rg[MAXS][MAXS] = {{0}};
+    double xi2 = 0.0, xi3 = 0.0;
+    for (int b = 0; b < c->M; ++b) {
+        rn[b] = c->n0[b];
+        xi2 += c->cparams.xi2c[b] * rn[b];
+        xi3 += c->cparams.xi3c[b] * rn[b];
+    }
+    const double i1 = xi3 < 0.9 ? 1.0 / (1.0 - xi3) : 1.0;
+    bool same = !c->ref_dirty;
+    for (int a = 0; a < c->M; ++a)
+        for (int b = 0; b < c->M; ++b) {
+            const double s = c->cparams.s_ab[a][b];
+            rg[a][b] = (double)(float)(rn[b] * (i1 + 3.0 * s * xi2 * i1 * i1 + 2.0 * s * s * xi2 * xi2 * i1 * i1 * i1));
+            same = same && rg[a][b] == c->ref_g[a][b];
+        }
+    for (int b = 0; b < c->M; ++b) {
+        rn[b] = (double)(float)rn[b];
+        same = same && rn[b] == c->ref_n[b];
+    }
+    if (same) return LBE_OK;
+    const long long P = c->g.P;
+    for (int b = 0; b < c->M; ++b) {
+        LAUNCH(launch_fill((float *)c->npad2.p + b * P, P, -(float)rn[b], c->stream), "fill the shell fields");
+        for (int a = 0; a < c->M; ++a)
+            LAUNCH(launch_fill((float *)c->gnpad.p + (a * c->M + b) * P, P, -(float)rg[a][b], c->stream),
+                   "fill the shell fields");
+    }
+    std::memcpy(c->ref_n, rn, sizeof(rn));
+    std::memcpy(c->ref_g, rg, sizeof(rg));
+    c->ref_dirty = false;
+    return LBE_OK;
+}
+
 // K1 -> K2 -> K3 for the populations pop (default: the current state); fills
 // npad, gab, gnpad, C.  With Pbase, the shell kernels also store P of every
 // pair into Pbase [npairs][3][N], and with xibase the contact kernel stores
@@ -733,6 +788,7 @@ lbe_status force_stage_core(lbe_ctx *c, const void *pop, void *Pbase, void *xiba
     }
     if (c->pairs.empty()) return LBE_OK;  // ideal gas: C stays zero
     if (c->spectral) return spectral_force(c, Pbase, xibase);
+    if (!f64) TRY(update_refs(c));
     {
         StageTimer t(c, LBE_STAGE_CONTACT);
         ContactLaunch L{};
@@ -742,59 +798,58 @@ lbe_status force_stage_core(lbe_ctx *c, const void *pop, void *Pbase, void *xiba
         L.br = &c->brows;
         L.RB = c->RB;
         L.gab = c->gab.p;
+        L.npad2 = c->npad2.p;
         L.gnpad = c->gnpad.p;
+        std::memcpy(L.refn, c->ref_n, sizeof(L.refn));
+        std::memcpy(L.refg, c->ref_g, sizeof(L.refg));
         L.xi = xibase;
         L.err = (int *)c->err.p;
         LAUNCH(launch_contact_tma(f64, L, c->stream), "contact kernel");
     }
-    // Two or more species: the pairs of odd species a run on a second stream beside those of even a. Each
-    // species' C still takes its pairs in order on one stream, and the launches of the two streams fill
-    // each other's last partial wave (one thread block per SM at a time).
-    const bool two = LBE_SHELL_STREAMS == 2 && c->M >= 2;
-    if (two && !c->side) {
-        CK(cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking), "create the shell stage's second stream");
-        CK(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming), "create fork event");
-        CK(cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming), "create join event");
-    }
     std::vector<int> first(c->M, 1);
-    StageTimer shell_timer(c, LBE_STAGE_SHELL, (int)c->pairs.size());
-    // joins the second stream back on an early return too, so that later work on the main stream
-    // never runs beside a pair launch already queued there
-    struct SideJoin {
-        lbe_ctx *c;
-        bool pending;
-        ~SideJoin() {
-            if (pending) {
-                cudaEventRecord(c->ev_join, c->side);
-                cudaStreamWaitEvent(c->stream, c->ev_join, 0);
-            }
+    if (!f64) {
+        StageTimer t(c, LBE_STAGE_SHELL);
+        ShellMarchArgs A{};
+        A.g = c->g;
+        A.M = c->M;
+        int Smax = 0;
+        for (size_t q = 0; q < c->pairs.size(); ++q) {
+            const PairShell &ps = c->pairs[q];
+            const int ab = ps.a * c->M + ps.b;
+            A.S[ab] = ps.S;
+            A.q[ab] = (int)q;
+            A.coef[ab] = (float)ps.coef;
+            Smax = std::max(Smax, ps.S);
+            first[ps.a] = 0;
         }
-    } side_join{c, false};
-    if (two) {
-        CK(cudaEventRecord(c->ev_fork, c->stream), "record fork");
-        CK(cudaStreamWaitEvent(c->side, c->ev_fork, 0), "fork the shell stage");
-        side_join.pending = true;
-    }
-    for (size_t q = 0; q < c->pairs.size(); ++q) {
-        const PairShell &ps = c->pairs[q];
-        ShellLaunch L{};
-        L.grid = &c->g;
-        L.map_n = &ps.map_n;
-        L.map_gn = &ps.map_gn;
-        L.npad_a = (const char *)c->npad.p + rb * ps.a * c->g.P;
-        L.g_ab = (const char *)c->gab.p + rb * (ps.a * c->M + ps.b) * c->g.N;
-        L.Cout = (char *)c->C.p + rb * 3 * ps.a * c->g.N;
-        L.Pout = Pbase ? (char *)Pbase + rb * 3 * q * c->g.N : nullptr;
-        L.coef = ps.coef;
-        L.accumulate = first[ps.a] ? 0 : 1;
-        L.err = (int *)c->err.p;
-        first[ps.a] = 0;
-        LAUNCH(launch_shell_force(f64, ps.S, L, two && (ps.a & 1) ? c->side : c->stream), "shell force kernel");
-    }
-    if (two) {
-        side_join.pending = false;
-        CK(cudaEventRecord(c->ev_join, c->side), "record join");
-        CK(cudaStreamWaitEvent(c->stream, c->ev_join, 0), "join the shell stage");
+        int shells[MAXS] = {0};
+        for (const PairShell &ps : c->pairs) shells[ps.a] += ps.S * ps.S;
+        for (int a = 0; a < c->M; ++a) A.order[a] = a;
+        std::stable_sort(A.order, A.order + c->M, [&](int a, int b) { return shells[a] < shells[b]; });  // shortest first
+        A.npad = (const float *)c->npad.p;
+        A.gab = (const float *)c->gab.p;
+        A.C = (float *)c->C.p;
+        A.Pout = (float *)Pbase;
+        A.err = (int *)c->err.p;
+        LAUNCH(launch_shell_march(Smax, *c->march_maps, A, c->stream), "shell force kernel");
+    } else {
+        StageTimer t(c, LBE_STAGE_SHELL, (int)c->pairs.size());
+        for (size_t q = 0; q < c->pairs.size(); ++q) {
+            const PairShell &ps = c->pairs[q];
+            ShellLaunch L{};
+            L.grid = &c->g;
+            L.map_n = &ps.map_n;
+            L.map_gn = &ps.map_gn;
+            L.npad_a = (const char *)c->npad.p + rb * ps.a * c->g.P;
+            L.g_ab = (const char *)c->gab.p + rb * (ps.a * c->M + ps.b) * c->g.N;
+            L.Cout = (char *)c->C.p + rb * 3 * ps.a * c->g.N;
+            L.Pout = Pbase ? (char *)Pbase + rb * 3 * q * c->g.N : nullptr;
+            L.coef = ps.coef;
+            L.accumulate = first[ps.a] ? 0 : 1;
+            L.err = (int *)c->err.p;
+            first[ps.a] = 0;
+            LAUNCH(launch_shell_force(ps.S, L, c->stream), "shell force kernel");
+        }
     }
     for (int a = 0; a < c->M; ++a)
         if (first[a]) CK(cudaMemsetAsync((char *)c->C.p + rb * 3 * a * c->g.N, 0, rb * 3 * c->g.N, c->stream),
@@ -1011,14 +1066,8 @@ void lbe_destroy(lbe_ctx *c) {
     fold_stage_times(c);
     for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
     c->ev_pool.clear();
-    if (c->side) {
-        cudaStreamSynchronize(c->side);
-        cudaStreamDestroy(c->side);
-        cudaEventDestroy(c->ev_fork);
-        cudaEventDestroy(c->ev_join);
-    }
     Buf *all[] = {&c->pop[0], &c->pop[1], &c->solid, &c->mask, &c->V, &c->phi, &c->amp, &c->F,
-                  &c->npad, &c->gab, &c->gnpad, &c->C, &c->flux_buf, &c->flux_acc,
+                  &c->npad, &c->npad2, &c->gab, &c->gnpad, &c->C, &c->flux_buf, &c->flux_acc,
                   &c->flux_last, &c->err, &c->scratch64, &c->partial, &c->red_out, &c->res_rec,
                   &c->specR, &c->specZ, &c->specW, &c->specTab, &c->specWork,
                   &c->aR, &c->aZ, &c->aW, &c->aTab, &c->aWork, &c->veoff, &c->vehat, &c->vut, &c->Feff};
@@ -1028,6 +1077,7 @@ void lbe_destroy(lbe_ctx *c) {
     c->aspec = nullptr;
     for (Buf *b : all) dev_free(c, *b);
     cudaStreamSynchronize(c->stream);
+    delete c->march_maps;
     delete c;
 }
 

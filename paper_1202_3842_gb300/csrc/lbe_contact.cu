@@ -8,9 +8,9 @@ cudaError_t launch_contact_tma(bool fp64, const ContactLaunch &L, cudaStream_t s
 }
 
 void contact_box(bool fp64, int M, int RB, int *bx, int *by) {
-    const int es = fp64 ? 8 : 4, A = 16 / es;
-    *bx = ((32 + 2 * RB + A - 1) + A - 1) / A * A;
-    *by = 8 + 2 * RB;
+    const int A = fp64 ? 2 : 4, nx = fp64 ? 1 : 2;  // ContactTile
+    *bx = 32 + 2 * ((RB + A - 1) / A * A);
+    *by = CT_THREADS * nx / 32 + 2 * RB;
     (void)M;
 }
 

@@ -95,7 +95,9 @@ struct ContactLaunch {
     const BallRows *br;
     int RB;                   // largest ball half-width
     void *gab;
-    void *gnpad;
+    void *npad2;               // FP32: padded n_b - refn[b] [M][P]
+    void *gnpad;               // padded g_ab n_b (FP32: minus refg[a][b]) [M][M][P]
+    double refn[MAXS], refg[MAXS][MAXS];
     void *xi;                  // NULL, or [2][N]: xi2, xi3 (kept for the adjoint)
     const uint32_t *mask;      // adjoint ball sum only
     void *ln;                  // adjoint ball sum only: [M][N] accumulated
@@ -114,6 +116,10 @@ struct ShellLaunch {
     int accumulate;
     int *err;
 };
+
+// FP32 shell force of every pair in one launch (lbe_shell_march.cuh).
+struct ShellMarchArgs;
+struct ShellMarchMaps;
 
 // Geometry
 cudaError_t launch_link_mask(const Grid &g, const uint8_t *solid, uint32_t *mask, cudaStream_t st);
@@ -142,10 +148,13 @@ cudaError_t launch_contact_tma(bool fp64, const ContactLaunch &L, cudaStream_t s
 // Transposed ball average: L.maps over the padded adjoint fields lnbar; ln[b] += ball sum, 0 on solid nodes.
 cudaError_t launch_adj_ball_tma(bool fp64, const ContactLaunch &L, cudaStream_t st);
 void contact_box(bool fp64, int M, int RB, int *bx, int *by);
-// K3: shell force of one ordered pair.
-cudaError_t launch_shell_force(bool fp64, int S, const ShellLaunch &L, cudaStream_t st);
+// K3 in FP32: every pair of every species in one launch; Smax the largest pair diameter (1..8).
+cudaError_t launch_shell_march(int Smax, const ShellMarchMaps &maps, ShellMarchArgs &A, cudaStream_t st);
+cudaError_t launch_fill(float *p, long long n, float v, cudaStream_t st);
+// K3 in FP64: shell force of one ordered pair.
+cudaError_t launch_shell_force(int S, const ShellLaunch &L, cudaStream_t st);
 bool shell_supported(bool fp64, int S);
-void shell_box(bool fp64, int S, int *bx, int *by);      // forward: FP32 boxes count 8-byte (n, g n) elements
+void shell_box(bool fp64, int S, int *bx, int *by);      // forward kernels
 void adj_shell_box(bool fp64, int S, int *bx, int *by);  // shell transpose: boxes of its own tiles
 // K4: fused moments + DD-TR collision + pull streaming.
 cudaError_t launch_collide(Prec p, const Grid &g, const void *src, void *dst, const uint32_t *mask, bool solid,

@@ -1,45 +1,37 @@
-// Dispatch of the shell-force kernels by precision and pair diameter, and the
-// host-side shell helpers.  FP32 reads the interleaved field (n_b, g_ab n_b):
-// diameters 4 to 6 run the y-blocked kernel (32 x 8 threads, two rows and
-// three planes of outputs per thread); 1 to 3 the z-blocked one with three
-// outputs along z on 32 x 16 threads, 7 with two, 8 with one on 32 x 8.  The
-// FP64 path uses the plain kernel (one output per thread and plane).  The
-// kernels are instantiated in lbe_shell_f32_*.cu and lbe_shell_f64.cu.
+// Dispatch of the shell-force kernels by precision and pair diameter, and the host-side shell helpers.
+// FP32: every pair in one launch of the marching kernel (lbe_shell_march.cuh), instantiated for the largest
+// pair diameter 4, 6 or 8 (the registers of a thread grow with it: 128, 166, 222, so four, three and two
+// blocks of 128 threads per SM).  FP64: one launch per pair of the plain kernel (lbe_shell_kernels.cuh).
 #include "lbe_device.cuh"
 #include "lbe_launch.h"
 #include "lbe_shell.cuh"
+#include "lbe_shell_march.cuh"
 
 namespace lbe {
 
 template <typename T, int S>
 cudaError_t launch_one(const ShellLaunch &L, cudaStream_t st);
-template <int S, int TZ, int TYB>
-cudaError_t launch_zb(const ShellLaunch &L, cudaStream_t st);
-template <int S, int TZ, int TYT>
-cudaError_t launch_yb(const ShellLaunch &L, cudaStream_t st);
+cudaError_t launch_shell_march_4(const ShellMarchMaps &maps, ShellMarchArgs &A, cudaStream_t st);
+cudaError_t launch_shell_march_6(const ShellMarchMaps &maps, ShellMarchArgs &A, cudaStream_t st);
+cudaError_t launch_shell_march_8(const ShellMarchMaps &maps, ShellMarchArgs &A, cudaStream_t st);
 
-#if LBE_SHELL_YB
-#define LBE_MID(S) launch_yb<S, LBE_SHELL_YTZ, LBE_SHELL_YTY>(L, st)
-#else
-#define LBE_MID(S) launch_zb<S, LBE_SHELL_TZ, LBE_SHELL_TY>(L, st)
-#endif
+cudaError_t launch_shell_march(int Smax, const ShellMarchMaps &maps, ShellMarchArgs &A, cudaStream_t st) {
+    if (Smax < 1 || Smax > 8) return cudaErrorInvalidValue;
+    return Smax <= 4 ? launch_shell_march_4(maps, A, st)
+                     : (Smax <= 6 ? launch_shell_march_6(maps, A, st) : launch_shell_march_8(maps, A, st));
+}
 
+__global__ void k_fill(float *__restrict__ p, long long n, float v) {
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        p[i] = v;
+}
+cudaError_t launch_fill(float *p, long long n, float v, cudaStream_t st) {
+    const long long nb = (n + 255) / 256;
+    k_fill<<<(unsigned)(nb < 8 * 152 ? nb : 8 * 152), 256, 0, st>>>(p, n, v);
+    return cudaGetLastError();
+}
 
-
-cudaError_t launch_shell_force(bool fp64, int S, const ShellLaunch &L, cudaStream_t st) {
-    if (!fp64) {
-        switch (S) {
-            case 1: return launch_zb<1, 3, 16>(L, st);
-            case 2: return launch_zb<2, 3, 16>(L, st);
-            case 3: return launch_zb<3, 3, 16>(L, st);
-            case 4: return LBE_MID(4);
-            case 5: return LBE_MID(5);
-            case 6: return LBE_MID(6);
-            case 7: return launch_zb<7, 2, 16>(L, st);
-            case 8: return launch_zb<8, 1, 8>(L, st);
-            default: return cudaErrorInvalidValue;
-        }
-    }
+cudaError_t launch_shell_force(int S, const ShellLaunch &L, cudaStream_t st) {
     switch (S) {
         case 1: return launch_one<double, 1>(L, st);
         case 2: return launch_one<double, 2>(L, st);
@@ -56,8 +48,7 @@ bool shell_supported(bool fp64, int S) { return S >= 1 && S <= (fp64 ? 7 : 8); }
 
 // Box of the shell-transpose tiles (lbe_adj_shell.cuh, dispatched in lbe_adjoint.cu).  FP32: the
 // interleaved 8-byte (Lambda, g Lambda) elements of a 32 x 16 tile (32 x 8 at S = 8), the tile the
-// transpose itself runs, which stays at 16 rows whatever the forward kernel's rows are; FP64: the
-// forward kernel's box of two separate planes.
+// transpose itself runs; FP64: the forward kernel's box of two separate planes.
 void adj_shell_box(bool fp64, int S, int *bx, int *by) {
     if (!fp64) {
         *bx = ((32 + 2 * S + 1) + 1) / 2 * 2;
@@ -68,9 +59,9 @@ void adj_shell_box(bool fp64, int S, int *bx, int *by) {
 }
 
 void shell_box(bool fp64, int S, int *bx, int *by) {
-    if (!fp64) {  // interleaved 8-byte elements; 32 x 16 outputs per plane (32 x 8 at S = 8)
-        *bx = ((32 + 2 * S + 1) + 1) / 2 * 2;
-        *by = (S >= 4 && S <= 6 ? (LBE_SHELL_YB ? 2 * LBE_SHELL_YTY : LBE_SHELL_TY) : (S <= 7 ? 16 : 8)) + 2 * S;
+    if (!fp64) {  // ShellMarchTile
+        *bx = 32 + 2 * ((S + 3) / 4 * 4);
+        *by = SM_TY + 2 * S;
         return;
     }
 #define LBE_BOX(s)                              \

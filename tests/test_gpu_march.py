@@ -1,0 +1,49 @@
+"""Contact values and shell force of the marching kernels at the edges of their tiles, against the oracle:
+lattices of one plane, narrower than a tile or a shell, odd rows (no 8-byte rows), one node more than a tile,
+periodic axes shorter than the shell (several images of a node in the halo), and up to four species."""
+import numpy as np
+import pytest
+
+from lbe_cases import rel_err, setup_gpu, setup_oracle
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    ((33, 5, 7), (1, 1, 1), (6.0,)),
+    ((32, 4, 1), (1, 1, 0), (4.0,)),
+    ((7, 3, 2), (1, 1, 1), (5.0,)),
+    ((1, 9, 40), (0, 1, 1), (3.0, 5.0)),
+    ((65, 6, 13), (1, 0, 0), (4.0, 6.0)),
+    ((30, 11, 26), (0, 0, 1), (2.0, 4.0, 6.0)),
+    ((18, 17, 15), (1, 1, 1), (1.0, 3.0, 5.0, 7.0)),
+    ((34, 9, 18), (0, 0, 0), (8.0,)),
+    ((16, 16, 64), (1, 1, 1), (0.0, 4.0)),
+]
+
+
+@pytest.mark.parametrize("prec,tol", [("fp32", 1e-5), ("fp64", 1e-12)])
+@pytest.mark.parametrize("shape,periodic,sig", CASES)
+def test_march_edges(shape, periodic, sig, prec, tol):
+    """Tolerances of the stage parity: FP32 sums of up to 762 points, FP64 round-off, of a field's largest value."""
+    N, M = int(np.prod(shape)), len(sig)
+    rng = np.random.default_rng(31)
+    solid = (rng.random(N) < 0.06).astype(np.uint8)
+    solid[rng.integers(N)] = 0
+    n0 = 6.0 * 0.12 / (np.pi * sum(s ** 3 for s in sig))
+    arr = dict(solid=solid, V=np.zeros((M, N)), phi=np.zeros(N), amp=np.zeros(N),
+               n=n0 * (1.0 + 0.3 * (rng.random((M, N)) - 0.5)) * (solid == 0)[None, :])
+    w = dict(shape=shape, periodic=periodic, sigma=list(sig), tau=[1.0] * M, body=[(0.0, 0.0, 0.0)] * M)
+    if prec == "fp64" and max(sig) > 7:
+        pytest.skip("no direct FP64 stencil of this diameter")
+    g = setup_gpu(w, arr, prec, shell="direct")
+    o = setup_oracle(w, arr)
+    obs = o.observe()
+    for a in range(M):
+        for b in range(M):
+            if sig[a] + sig[b] > 0:
+                assert rel_err(g.contact(a, b), obs["g"][a, b]) <= tol
+        scale = np.abs(obs["C"][a]).max()
+        if scale > 0:
+            assert rel_err(g.force(a), obs["C"][a]) <= tol
+        else:
+            assert np.abs(g.force(a)).max() <= tol * n0
