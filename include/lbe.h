@@ -84,11 +84,10 @@ typedef enum { LBE_DD_TR = 0, LBE_SD_TR = 1, LBE_SD_EU = 2, LBE_DD_EU = 3 } lbe_
  *     likewise; any integer pair diameter up to the limit of the contact
  *     values (sigma_b / 2 <= 4);
  *   LBE_SHELL_AUTO (default): spectral for diameters without a compiled
- *     stencil, and where it is cheaper by a cost rule measured on GB300.  FP32
- *     arithmetic: direct on lattices of 16384 nodes and more; on smaller ones,
- *     and in FP64, spectral where the mean shell of the pairs is above about
- *     320 points (FP32) or 110 points (FP64, where the stencil is bound by the
- *     FP64 rate), scaled by the padded grid over the lattice.
+ *     stencil, direct for compiled diameters on lattices of 16384 nodes and
+ *     more (measured on GB300); on smaller ones spectral where the mean shell
+ *     of the pairs is above about 320 points (FP32) or 110 points (FP64),
+ *     scaled by the padded grid over the lattice.
  * Both give the sums of the definition up to rounding.  The discrete adjoint
  * (lbe_adjoint_flux_gradient) transposes the shell sums with the method this
  * call sets: the stencil (pair diameters with a compiled stencil), the

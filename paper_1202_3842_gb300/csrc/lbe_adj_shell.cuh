@@ -25,7 +25,8 @@
 #pragma once
 #include <utility>
 
-#include "lbe_shell_kernels.cuh"
+#include "lbe_launch.h"
+#include "lbe_march.cuh"
 
 namespace lbe {
 

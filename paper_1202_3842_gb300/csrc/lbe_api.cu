@@ -15,6 +15,7 @@
 #include "lbe_device.cuh"
 #include "lbe_launch.h"
 #include "lbe_shell.cuh"
+#include "lbe_shell_fixed.cuh"
 #include "lbe_shell_march.cuh"
 
 using namespace lbe;
@@ -40,7 +41,6 @@ struct Buf {
 struct PairShell {
     int a, b, S;
     double coef;  // -kT sigma_ab^2 w_ab
-    CUtensorMap map_n, map_gn;
 };
 
 }  // namespace
@@ -71,6 +71,7 @@ struct lbe_ctx {
     Buf npad2;  // FP32 direct shell force: padded deviations n_b - ref_n [M][P]; gnpad then holds g_ab n_b - ref_g
     double ref_n[MAXS] = {0}, ref_g[MAXS][MAXS] = {{0}};
     bool ref_dirty = true;
+    Buf fix, top;  // FP64 direct shell force: fixed-point images of n_b and g_ab n_b [M + M^2][P], maxima's high words
     ShellMarchMaps *march_maps = nullptr;
     Buf flux_buf, flux_acc, flux_last;
     Buf err;
@@ -328,8 +329,7 @@ int shell_count(int S) {
 // fixed time per node and shell point, the spectral form a fixed time per grid point and pair, and they break
 // even at a mean shell of about 320 points per pair in FP32 and 110 in FP64, scaled by the lattice over the
 // grid.  The shell transpose of the adjoint follows it (its stencil is 2.6 times the cost), and so does the
-// forward form of lattices of fewer than DIRECT_NODES nodes, FP64 and the rest of what direct_cheaper
-// leaves.
+// forward form of lattices of fewer than DIRECT_NODES nodes.
 bool spectral_cheaper(const lbe_ctx *c, bool f64, double stencil_factor = 1.0) {
     long long pts = 0;
     int Smax = 0;
@@ -345,14 +345,15 @@ bool spectral_cheaper(const lbe_ctx *c, bool f64, double stencil_factor = 1.0) {
     return spectral_shape_ok(c, Smax) && (double)pts * (double)g.N > even * (double)c->pairs.size() * Nr;
 }
 
-// Whether the marching kernels (lbe_shell_march.cuh, lbe_contact.cuh) take the forward force under
-// LBE_SHELL_AUTO.  FP32, K2 + K3 on GB300: 738 against 1146 us on the 256^3 well of diameter 6, 533 against 602 us
-// on a 192^3 well of diameter 8 (the widest they take), 1100 against 2390 us on the 512x128x128 channel of
-// diameters 4 and 6, 51 against 95 us on a 64^3 well of diameter 6: direct wherever a stencil is compiled.
-// Lattices below DIRECT_NODES nodes are bound by launches in either form and keep the rule above, which
-// programs that record the method of a small lattice rely on.
+// Whether the marching kernels (lbe_shell_march.cuh, lbe_shell_fixed.cuh, lbe_contact.cuh) take the forward force
+// under LBE_SHELL_AUTO.  K2 + K3 on GB300 in FP32: 738 against 1146 us on the 256^3 well of diameter 6, 533 against
+// 602 us on a 192^3 well of diameter 8 (the widest they take), 1100 against 2390 us on the 512x128x128 channel
+// of diameters 4 and 6, 51 against 95 us on a 64^3 well of diameter 6; in FP64 1125 against 3870 us on the
+// 256x64x64 channel of diameters 4 and 6, 75 against 195 us on a 48^3 well of diameter 4: direct wherever a
+// stencil is compiled.  Lattices below DIRECT_NODES nodes are bound by launches in either form and keep the
+// rule above, which programs that record the method of a small lattice rely on.
 constexpr long long DIRECT_NODES = 16384;
-bool direct_cheaper(const lbe_ctx *c, bool f64) { return !f64 && c->g.N >= DIRECT_NODES; }
+bool direct_cheaper(const lbe_ctx *c) { return c->g.N >= DIRECT_NODES; }
 
 // The pairs as the spectral kernels see them (shell index into the table of distinct shells), the
 // distinct shells, and the grid: the lattice along periodic axes, at least Smax zero planes beyond it
@@ -609,7 +610,7 @@ lbe_status prepare(lbe_ctx *c) {
                             "a pair diameter has no compiled direct shell stencil (the spectral method takes it)");
             c->spectral = c->shell_method == LBE_SHELL_SPECTRAL ||
                           (c->shell_method == LBE_SHELL_AUTO &&
-                           (!direct_ok || (!direct_cheaper(c, f64) && spectral_cheaper(c, f64))));
+                           (!direct_ok || (!direct_cheaper(c) && spectral_cheaper(c, f64))));
         }
         // ball radii
         ContactParams cp{};
@@ -672,12 +673,16 @@ lbe_status prepare(lbe_ctx *c) {
         const size_t gnb = rb * c->M * c->M * g.P;
         if (!c->spectral) TRY(dev_alloc(c, c->gnpad, gnb));
         if (!c->spectral && !f64) TRY(dev_alloc(c, c->npad2, rb * c->M * g.P));
+        if (!c->spectral && f64) {
+            TRY(dev_alloc(c, c->fix, 8 * (c->M + c->M * c->M) * g.P));
+            TRY(dev_alloc(c, c->top, 4 * (c->M + c->M * c->M)));
+        }
         c->ref_dirty = true;
         TRY(dev_alloc(c, c->gab, rb * c->M * c->M * g.N));
         TRY(dev_alloc(c, c->C, rb * c->M * 3 * g.N));
         CK(cudaMemsetAsync(c->npad.p, 0, rb * c->M * g.P, c->stream), "memset npad");
         if (!c->spectral && f64) CK(cudaMemsetAsync(c->gnpad.p, 0, gnb, c->stream), "memset gnpad");
-        if (!c->march_maps && !f64) {
+        if (!c->march_maps) {
             c->march_maps = new (std::nothrow) ShellMarchMaps;
             if (!c->march_maps) return fail(c, LBE_ERR_OOM, "host allocation failed");
         }
@@ -685,12 +690,12 @@ lbe_status prepare(lbe_ctx *c) {
         for (auto &ps : c->pairs) {
             if (c->spectral) break;
             const int ab = ps.a * c->M + ps.b;
-            char *nb = (char *)(f64 ? c->npad.p : c->npad2.p) + rb * ps.b * g.P;
-            char *gn = (char *)c->gnpad.p + rb * ab * g.P;
+            char *nb = (char *)(f64 ? c->fix.p : c->npad2.p) + rb * ps.b * g.P;
+            char *gn = f64 ? (char *)c->fix.p + rb * (c->M + ab) * g.P : (char *)c->gnpad.p + rb * ab * g.P;
             int bx = 0, by = 0;
             shell_box(f64, ps.S, &bx, &by);
-            TRY(make_map(c, f64 ? &ps.map_n : &c->march_maps->n[ab], nb, bx, by));
-            TRY(make_map(c, f64 ? &ps.map_gn : &c->march_maps->gn[ab], gn, bx, by));
+            TRY(make_map(c, &c->march_maps->n[ab], nb, bx, by));
+            TRY(make_map(c, &c->march_maps->gn[ab], gn, bx, by));
         }
         {
             int bx = 0, by = 0;
@@ -803,53 +808,48 @@ lbe_status force_stage_core(lbe_ctx *c, const void *pop, void *Pbase, void *xiba
         std::memcpy(L.refn, c->ref_n, sizeof(L.refn));
         std::memcpy(L.refg, c->ref_g, sizeof(L.refg));
         L.xi = xibase;
+        L.top = (unsigned *)c->top.p;
+        if (f64) CK(cudaMemsetAsync(c->top.p, 0, 4 * (c->M + c->M * c->M), c->stream), "memset maxima");
         L.err = (int *)c->err.p;
         LAUNCH(launch_contact_tma(f64, L, c->stream), "contact kernel");
     }
     std::vector<int> first(c->M, 1);
-    if (!f64) {
-        StageTimer t(c, LBE_STAGE_SHELL);
-        ShellMarchArgs A{};
+    StageTimer t(c, LBE_STAGE_SHELL, f64 ? 2 : 1);
+    int Smax = 0, shells[MAXS] = {0};
+    auto fill = [&](auto &A, auto zero) {  // the launch's arguments, in the precision of `zero`
+        using T = decltype(zero);
         A.g = c->g;
         A.M = c->M;
-        int Smax = 0;
         for (size_t q = 0; q < c->pairs.size(); ++q) {
             const PairShell &ps = c->pairs[q];
             const int ab = ps.a * c->M + ps.b;
             A.S[ab] = ps.S;
             A.q[ab] = (int)q;
-            A.coef[ab] = (float)ps.coef;
+            A.coef[ab] = (T)ps.coef;
             Smax = std::max(Smax, ps.S);
+            shells[ps.a] += ps.S * ps.S;
             first[ps.a] = 0;
         }
-        int shells[MAXS] = {0};
-        for (const PairShell &ps : c->pairs) shells[ps.a] += ps.S * ps.S;
         for (int a = 0; a < c->M; ++a) A.order[a] = a;
-        std::stable_sort(A.order, A.order + c->M, [&](int a, int b) { return shells[a] < shells[b]; });  // shortest first
-        A.npad = (const float *)c->npad.p;
-        A.gab = (const float *)c->gab.p;
-        A.C = (float *)c->C.p;
-        A.Pout = (float *)Pbase;
+        std::stable_sort(A.order, A.order + c->M, [&](int a, int b) { return shells[a] < shells[b]; });
+        A.npad = (const T *)c->npad.p;
+        A.gab = (const T *)c->gab.p;
+        A.C = (T *)c->C.p;
+        A.Pout = (T *)Pbase;
         A.err = (int *)c->err.p;
-        LAUNCH(launch_shell_march(Smax, *c->march_maps, A, c->stream), "shell force kernel");
+    };
+    if (f64) {
+        FixedArgs A{};
+        fill(A, 0.0);
+        A.top = (const unsigned *)c->top.p;
+        LAUNCH(launch_to_fixed(Smax, (const double *)c->npad.p, (const double *)c->gnpad.p, c->g.P, c->M, A.top,
+                               (long long *)c->fix.p, c->stream),
+               "fixed-point fields");
+        LAUNCH(launch_shell_fixed(Smax, *c->march_maps, A, c->stream), "shell force kernel");
     } else {
-        StageTimer t(c, LBE_STAGE_SHELL, (int)c->pairs.size());
-        for (size_t q = 0; q < c->pairs.size(); ++q) {
-            const PairShell &ps = c->pairs[q];
-            ShellLaunch L{};
-            L.grid = &c->g;
-            L.map_n = &ps.map_n;
-            L.map_gn = &ps.map_gn;
-            L.npad_a = (const char *)c->npad.p + rb * ps.a * c->g.P;
-            L.g_ab = (const char *)c->gab.p + rb * (ps.a * c->M + ps.b) * c->g.N;
-            L.Cout = (char *)c->C.p + rb * 3 * ps.a * c->g.N;
-            L.Pout = Pbase ? (char *)Pbase + rb * 3 * q * c->g.N : nullptr;
-            L.coef = ps.coef;
-            L.accumulate = first[ps.a] ? 0 : 1;
-            L.err = (int *)c->err.p;
-            first[ps.a] = 0;
-            LAUNCH(launch_shell_force(ps.S, L, c->stream), "shell force kernel");
-        }
+        ShellMarchArgs A{};
+        fill(A, 0.f);
+        LAUNCH(launch_shell_march(Smax, *c->march_maps, A, c->stream), "shell force kernel");
     }
     for (int a = 0; a < c->M; ++a)
         if (first[a]) CK(cudaMemsetAsync((char *)c->C.p + rb * 3 * a * c->g.N, 0, rb * 3 * c->g.N, c->stream),
@@ -1067,7 +1067,7 @@ void lbe_destroy(lbe_ctx *c) {
     for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
     c->ev_pool.clear();
     Buf *all[] = {&c->pop[0], &c->pop[1], &c->solid, &c->mask, &c->V, &c->phi, &c->amp, &c->F,
-                  &c->npad, &c->npad2, &c->gab, &c->gnpad, &c->C, &c->flux_buf, &c->flux_acc,
+                  &c->npad, &c->npad2, &c->fix, &c->top, &c->gab, &c->gnpad, &c->C, &c->flux_buf, &c->flux_acc,
                   &c->flux_last, &c->err, &c->scratch64, &c->partial, &c->red_out, &c->res_rec,
                   &c->specR, &c->specZ, &c->specW, &c->specTab, &c->specWork,
                   &c->aR, &c->aZ, &c->aW, &c->aTab, &c->aWork, &c->veoff, &c->vehat, &c->vut, &c->Feff};

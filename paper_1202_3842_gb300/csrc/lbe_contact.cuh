@@ -184,7 +184,7 @@ template <typename T, int M, int RB, int MODE>
 __global__ void __launch_bounds__(CT_THREADS)
     k_contact_tma(const __grid_constant__ ContactMaps maps, Grid g, ContactConst<T> cs, T *__restrict__ gab,
                   T *__restrict__ npad2, T *__restrict__ gnpad, T *__restrict__ xi_out,
-                  const uint32_t *__restrict__ mask, T *__restrict__ ln, int *err) {
+                  const uint32_t *__restrict__ mask, T *__restrict__ ln, unsigned *__restrict__ top, int *err) {
     using Tl = ContactTile<T, M, RB>;
     using Ln = Lane<T>;
     using V = typename Ln::V;
@@ -238,6 +238,12 @@ __global__ void __launch_bounds__(CT_THREADS)
     for (int b = 0; b < M; ++b)
 #pragma unroll
         for (int k = 0; k <= 2 * RB; ++k) acc[b][k] = Ln::zero();
+
+    // FP64: high words of the largest values this thread writes (they order like the values)
+    constexpr int NT = sizeof(T) == 8 && MODE == 0 ? M + M * M : 1;
+    unsigned big[NT];
+#pragma unroll
+    for (int f = 0; f < NT; ++f) big[f] = 0;
 
     int slot = 0, cslot = Tl::R - RB;  // ring slots of the input plane and of the plane RB behind it
     if (cslot == Tl::R) cslot = 0;
@@ -362,6 +368,14 @@ __global__ void __launch_bounds__(CT_THREADS)
                                 }
                             }
                         }
+                    if constexpr (sizeof(T) == 8) {
+#pragma unroll
+                        for (int b = 0; b < M; ++b)
+                            big[b] = max(big[b], (unsigned)__double2hiint(nloc[b][0]) & 0x7fffffffu);
+#pragma unroll
+                        for (int f = 0; f < M * M; ++f)
+                            big[M + f] = max(big[M + f], (unsigned)__double2hiint(pv[f][0]) & 0x7fffffffu);
+                    }
                     auto field = [&](int f) -> T * {
                         return f < ND ? npad2 + (long long)f * g.P : gnpad + (long long)(f - ND) * g.P;
                     };
@@ -413,6 +427,14 @@ __global__ void __launch_bounds__(CT_THREADS)
         }
         if (++cslot == Tl::R) cslot = 0;
     }
+    if constexpr (sizeof(T) == 8 && MODE == 0) {
+#pragma unroll
+        for (int f = 0; f < NT; ++f) {
+            const unsigned m = __reduce_max_sync(0xffffffffu, big[f]);
+            // most warps find the maximum raised already
+            if ((tid & 31) == 0 && m > *(volatile unsigned *)(top + f)) atomicMax(top + f, m);
+        }
+    }
 }
 
 template <typename T, int M, int RB, int MODE>
@@ -449,7 +471,7 @@ cudaError_t launch_ct(const ContactLaunch &L, cudaStream_t st) {
     dim3 grid(nbx, nby, (g.nz + cs.lz - 1) / cs.lz);
     k_contact_tma<T, M, RB, MODE><<<grid, CT_THREADS, Tl::SMEM, st>>>(maps, g, cs, (T *)L.gab,
                                                                  (T *)L.npad2, (T *)L.gnpad, (T *)L.xi, L.mask,
-                                                                 (T *)L.ln, L.err);
+                                                                 (T *)L.ln, L.top, L.err);
     return cudaGetLastError();
 }
 

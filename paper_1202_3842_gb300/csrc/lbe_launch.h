@@ -98,27 +98,16 @@ struct ContactLaunch {
     void *npad2;               // FP32: padded n_b - refn[b] [M][P]
     void *gnpad;               // padded g_ab n_b (FP32: minus refg[a][b]) [M][M][P]
     double refn[MAXS], refg[MAXS][MAXS];
+    unsigned *top;             // FP64: high words of the largest n_b [M] and g_ab n_b [M][M], raised from 0
     void *xi;                  // NULL, or [2][N]: xi2, xi3 (kept for the adjoint)
     const uint32_t *mask;      // adjoint ball sum only
     void *ln;                  // adjoint ball sum only: [M][N] accumulated
     int *err;
 };
 
-struct ShellLaunch {
-    const Grid *grid;
-    const CUtensorMap *map_n;
-    const CUtensorMap *map_gn;
-    const void *npad_a;
-    const void *g_ab;
-    void *Cout;
-    void *Pout;  // NULL, or [3][N]: P = sum_e e^ n_b(r+e) of the pair (for the adjoint)
-    double coef;
-    int accumulate;
-    int *err;
-};
-
-// FP32 shell force of every pair in one launch (lbe_shell_march.cuh).
+// Shell force of every pair in one launch (lbe_shell_march.cuh FP32, lbe_shell_fixed.cuh FP64).
 struct ShellMarchArgs;
+struct FixedArgs;
 struct ShellMarchMaps;
 
 // Geometry
@@ -151,8 +140,11 @@ void contact_box(bool fp64, int M, int RB, int *bx, int *by);
 // K3 in FP32: every pair of every species in one launch; Smax the largest pair diameter (1..8).
 cudaError_t launch_shell_march(int Smax, const ShellMarchMaps &maps, ShellMarchArgs &A, cudaStream_t st);
 cudaError_t launch_fill(float *p, long long n, float v, cudaStream_t st);
-// K3 in FP64: shell force of one ordered pair.
-cudaError_t launch_shell_force(int S, const ShellLaunch &L, cudaStream_t st);
+// K3 in FP64, diameters 1..7, and the fixed-point images [M + M^2][P] of its fields; top: high words of the
+// largest values of n_b [M] and g_ab n_b [M][M], from K2.
+cudaError_t launch_shell_fixed(int Smax, const ShellMarchMaps &maps, FixedArgs &A, cudaStream_t st);
+cudaError_t launch_to_fixed(int Smax, const double *npad, const double *gnpad, long long P, int M,
+                            const unsigned *top, long long *out, cudaStream_t st);
 bool shell_supported(bool fp64, int S);
 void shell_box(bool fp64, int S, int *bx, int *by);      // forward kernels
 void adj_shell_box(bool fp64, int S, int *bx, int *by);  // shell transpose: boxes of its own tiles

@@ -104,4 +104,24 @@ inline int march_planes(long long tiles, int nz, int r, int per_sm, double halo,
     return best;
 }
 
+// Tensor maps of the shell fields of every ordered pair [a][b]: n_b and g_ab n_b (FP32: their deviations), boxes
+// of the pair's diameter.
+struct ShellMarchMaps {
+    CUtensorMap n[MAXS * MAXS], gn[MAXS * MAXS];
+};
+
+// A mixture's blocks differ in length.  A.order lists the species with the smaller shells first; with few blocks
+// the largest go first, so that the last to start are the short ones (128x32x32 channel, diameters 4 and 6: 46
+// against 53 us; 90x75x66, diameters 2, 4, 6: 166 against 188 us).  Where many waves follow each other the order
+// stays (512x128x128 channel: 1007 against 1029 us).
+template <typename Args>
+inline void march_order(Args &A, long long blocks, int per_sm) {
+    if (blocks > 152ll * 2 * per_sm) return;
+    for (int k = 0; 2 * k < A.M - 1; ++k) {
+        const int t = A.order[k];
+        A.order[k] = A.order[A.M - 1 - k];
+        A.order[A.M - 1 - k] = t;
+    }
+}
+
 }  // namespace lbe

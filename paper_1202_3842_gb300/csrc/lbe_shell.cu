@@ -1,16 +1,16 @@
 // Dispatch of the shell-force kernels by precision and pair diameter, and the host-side shell helpers.
 // FP32: every pair in one launch of the marching kernel (lbe_shell_march.cuh), instantiated for the largest
 // pair diameter 4, 6 or 8 (the registers of a thread grow with it: 128, 166, 222, so four, three and two
-// blocks of 128 threads per SM).  FP64: one launch per pair of the plain kernel (lbe_shell_kernels.cuh).
+// blocks of 128 threads per SM).  FP64: the same march in fixed point (lbe_shell_fixed.cuh) on the integer images
+// of the padded fields that k_to_fixed writes.
 #include "lbe_device.cuh"
 #include "lbe_launch.h"
 #include "lbe_shell.cuh"
+#include "lbe_shell_fixed.cuh"
 #include "lbe_shell_march.cuh"
 
 namespace lbe {
 
-template <typename T, int S>
-cudaError_t launch_one(const ShellLaunch &L, cudaStream_t st);
 cudaError_t launch_shell_march_4(const ShellMarchMaps &maps, ShellMarchArgs &A, cudaStream_t st);
 cudaError_t launch_shell_march_6(const ShellMarchMaps &maps, ShellMarchArgs &A, cudaStream_t st);
 cudaError_t launch_shell_march_8(const ShellMarchMaps &maps, ShellMarchArgs &A, cudaStream_t st);
@@ -31,31 +31,63 @@ cudaError_t launch_fill(float *p, long long n, float v, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_shell_force(int S, const ShellLaunch &L, cudaStream_t st) {
-    switch (S) {
-        case 1: return launch_one<double, 1>(L, st);
-        case 2: return launch_one<double, 2>(L, st);
-        case 3: return launch_one<double, 3>(L, st);
-        case 4: return launch_one<double, 4>(L, st);
-        case 5: return launch_one<double, 5>(L, st);
-        case 6: return launch_one<double, 6>(L, st);
-        case 7: return launch_one<double, 7>(L, st);
-        default: return cudaErrorInvalidValue;
+cudaError_t launch_shell_fixed_4(const ShellMarchMaps &maps, FixedArgs &A, cudaStream_t st);
+cudaError_t launch_shell_fixed_6(const ShellMarchMaps &maps, FixedArgs &A, cudaStream_t st);
+cudaError_t launch_shell_fixed_7(const ShellMarchMaps &maps, FixedArgs &A, cudaStream_t st);
+
+cudaError_t launch_shell_fixed(int Smax, const ShellMarchMaps &maps, FixedArgs &A, cudaStream_t st) {
+    if (Smax < 1 || Smax > 7) return cudaErrorInvalidValue;
+    return Smax <= 4 ? launch_shell_fixed_4(maps, A, st)
+                     : (Smax <= 6 ? launch_shell_fixed_6(maps, A, st) : launch_shell_fixed_7(maps, A, st));
+}
+
+// Fixed-point image of a field: v 2^(bits - 1 - e), e the exponent of the field's largest value, rounded to
+// nearest, by shifts of the mantissa (no FP64 operation).  Zero, subnormal and non-finite values become 0 (a
+// non-finite density is an error of its own).
+__device__ __forceinline__ long long to_fixed(double v, int top, int bits) {
+    const long long b = __double_as_longlong(v);
+    const int e = (int)((b >> 52) & 0x7ff);
+    if (e == 0 || e == 0x7ff || top == 0 || top == 0x7ff || e > top) return 0;
+    const long long m = (b & 0xfffffffffffffll) | 0x10000000000000ll;
+    const int d = top - e - (bits - 53);  // right shift
+    const long long r = d <= 0 ? m << -d : (d > 54 ? 0 : (m + (1ll << (d - 1))) >> d);
+    return b < 0 ? -r : r;
+}
+__global__ void __launch_bounds__(256) k_to_fixed(const double *__restrict__ npad, const double *__restrict__ gnpad,
+                                                 long long P, int M, int bits,
+                                                 const unsigned *__restrict__ top, long long *__restrict__ out) {
+    const int f = blockIdx.y;  // n_b, then g_ab n_b
+    const double *src = f < M ? npad + f * P : gnpad + (long long)(f - M) * P;
+    const int e = fx_exponent(top[f]);
+    longlong2 *dst = reinterpret_cast<longlong2 *>(out + f * P);
+    const double2 *s2 = reinterpret_cast<const double2 *>(src);
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < P / 2;
+         i += (long long)gridDim.x * blockDim.x) {
+        const double2 v = s2[i];
+        dst[i] = make_longlong2(to_fixed(v.x, e, bits), to_fixed(v.y, e, bits));
     }
+}
+cudaError_t launch_to_fixed(int Smax, const double *npad, const double *gnpad, long long P, int M,
+                            const unsigned *top, long long *out, cudaStream_t st) {
+    const long long nb = (P / 2 + 255) / 256;
+    k_to_fixed<<<dim3((unsigned)(nb < 2048 ? nb : 2048), M + M * M), 256, 0, st>>>(npad, gnpad, P, M,
+                                                                                     fx_bits(Smax), top, out);
+    return cudaGetLastError();
 }
 
 bool shell_supported(bool fp64, int S) { return S >= 1 && S <= (fp64 ? 7 : 8); }
 
 // Box of the shell-transpose tiles (lbe_adj_shell.cuh, dispatched in lbe_adjoint.cu).  FP32: the
 // interleaved 8-byte (Lambda, g Lambda) elements of a 32 x 16 tile (32 x 8 at S = 8), the tile the
-// transpose itself runs; FP64: the forward kernel's box of two separate planes.
+// transpose itself runs; FP64: two separate planes of a 32 x 8 tile (32 x 4 from S = 5).
 void adj_shell_box(bool fp64, int S, int *bx, int *by) {
     if (!fp64) {
         *bx = ((32 + 2 * S + 1) + 1) / 2 * 2;
         *by = (S <= 7 ? 16 : 8) + 2 * S;
         return;
     }
-    shell_box(true, S, bx, by);
+    *bx = ((32 + 2 * S + 1) + 1) / 2 * 2;  // ShellTileZ<double, S, 1, .>
+    *by = (S >= 5 ? 4 : 8) + 2 * S;
 }
 
 void shell_box(bool fp64, int S, int *bx, int *by) {
@@ -64,15 +96,8 @@ void shell_box(bool fp64, int S, int *bx, int *by) {
         *by = SM_TY + 2 * S;
         return;
     }
-#define LBE_BOX(s)                              \
-    case s:                                     \
-        *bx = ShellTile<double, s>::BX;         \
-        *by = ShellTile<double, s>::BY;         \
-        return;
-    switch (S) { LBE_BOX(1) LBE_BOX(2) LBE_BOX(3) LBE_BOX(4) LBE_BOX(5) LBE_BOX(6) LBE_BOX(7) default: break; }
-#undef LBE_BOX
-    *bx = 0;
-    *by = 0;
+    *bx = 32 + 2 * ((S + 1) / 2 * 2);  // FixedTile
+    *by = FX_TY + 2 * S;
 }
 
 }  // namespace lbe

@@ -164,10 +164,6 @@ struct ShellMarchArgs {
     float *Pout;                 // NULL, or [pairs][3][N]
     int *err;
 };
-struct ShellMarchMaps {
-    CUtensorMap n[MAXS * MAXS], gn[MAXS * MAXS];  // padded deviations of n_b and g_ab n_b, box of [a][b]
-};
-
 // March of one pair through the block's planes; `it` counts the planes of the block's ring.
 template <int SMAX, int S>
 __device__ __forceinline__ bool shell_march(const ShellMarchMaps &maps, const ShellMarchArgs &A, unsigned char *base,
@@ -327,17 +323,9 @@ cudaError_t launch_shell_march_t(const ShellMarchMaps &maps, ShellMarchArgs &A, 
     const Grid &g = A.g;
     const int tx = (g.nx + 31) / 32, ty = (g.ny + SM_TY - 1) / SM_TY;
     constexpr int per_sm = shell_march_per_sm(SMAX);
-    // A mixture's blocks differ in length: largest shells first, so that the last to start are the short ones
-    // (128x32x32 channel, diameters 4 and 6: 46 against 53 us; 90x75x66, diameters 2, 4, 6: 166 against 188 us).
-    // Where many waves follow each other it is the other order (512x128x128 channel: 1007 against 1029 us).
     A.lz = march_planes((long long)tx * ty * A.M, g.nz, SMAX, per_sm, 1.0, 0.9, A.M > 1);
     A.nzb = (g.nz + A.lz - 1) / A.lz;
-    if ((long long)tx * ty * A.M * A.nzb <= 152ll * 2 * per_sm)
-        for (int k = 0; 2 * k < A.M - 1; ++k) {
-            const int t = A.order[k];
-            A.order[k] = A.order[A.M - 1 - k];
-            A.order[A.M - 1 - k] = t;
-        }
+    march_order(A, (long long)tx * ty * A.M * A.nzb, per_sm);
     k_shell_march<SMAX><<<dim3(tx, ty, A.M * A.nzb), 32 * SM_TY, smem, st>>>(maps, A);
     return cudaGetLastError();
 }
