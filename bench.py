@@ -201,11 +201,12 @@ KERNEL_SOURCES = {
     "collide": ["paper_1202_3842_gb300/csrc/lbe_collide_pair.cu", "paper_1202_3842_gb300/csrc/lbe_device.cuh",
                 "paper_1202_3842_gb300/csrc/lbe_node.cuh"],
     "shell": ["paper_1202_3842_gb300/csrc/lbe_shell.cu", "paper_1202_3842_gb300/csrc/lbe_shell.cuh",
-              "paper_1202_3842_gb300/csrc/lbe_shell_kernels.cuh", "paper_1202_3842_gb300/csrc/lbe_device.cuh"],
+              "paper_1202_3842_gb300/csrc/lbe_march.cuh", "paper_1202_3842_gb300/csrc/lbe_shell_march.cuh",
+              "paper_1202_3842_gb300/csrc/lbe_shell_fixed.cuh", "paper_1202_3842_gb300/csrc/lbe_device.cuh"],
     "density": ["paper_1202_3842_gb300/csrc/lbe_kernels.cu", "paper_1202_3842_gb300/csrc/lbe_collide_pair.cu",
                 "paper_1202_3842_gb300/csrc/lbe_device.cuh", "paper_1202_3842_gb300/csrc/lbe_node.cuh"],
     "contact": ["paper_1202_3842_gb300/csrc/lbe_contact.cu", "paper_1202_3842_gb300/csrc/lbe_contact.cuh",
-                "paper_1202_3842_gb300/csrc/lbe_device.cuh"],
+                "paper_1202_3842_gb300/csrc/lbe_march.cuh", "paper_1202_3842_gb300/csrc/lbe_device.cuh"],
     "flux": ["paper_1202_3842_gb300/csrc/lbe_kernels.cu"],
     "shell_spectral": ["paper_1202_3842_gb300/csrc/lbe_spectral.cu"],
     "contact_spectral": ["paper_1202_3842_gb300/csrc/lbe_spectral.cu"],
@@ -423,8 +424,8 @@ def kernel_rooflines(stages, w, prec, N, M, sb, hbm, roof, sms, clk, shell_metho
     K4: reads and writes f~ and g~ (76 populations) per node and species; HBM bound with 32- and 16-bit
     storage; with FP64 storage it is bound by GB300's FP64 rate, so it also carries the FP64-rate roofline
     of K4_FLOPS_PER_NODE_SPECIES flops per node and species against the nominal FP64 rate.
-    K2, stencil form: sum_b |B_b| shared-memory loads of the padded densities per node, against the
-    shared-memory load bandwidth (32 banks x 4 B per clock per SM); in spectral form its fields through
+    K2, stencil form: the sum_b |B_b| ball points per node as shared-memory loads of the padded densities (the
+    kernel shares sums between heights and reads fewer), against the shared-memory load bandwidth (32 banks x 4 B per clock per SM); in spectral form its fields through
     HBM.  K3: the shell stage's roofline in the form in use (stencil: algorithmic flops against the FP32
     FMA peak; spectral: its fields through HBM, or FP64 transform flops)."""
     rb = 8 if prec == "fp64" else 4
@@ -466,7 +467,7 @@ def kernel_rooflines(stages, w, prec, N, M, sb, hbm, roof, sms, clk, shell_metho
             out["contact"] = {"bound": "smem", "algorithmic_smem_bytes_per_launch": b, "avg_launch_ms": t * 1e3,
                               "achieved_gbs": b / t / 1e9, "peak_gbs": peak, "frac": b / t / 1e9 / peak,
                               "peak_source": "shared-memory loads: %d SMs x 128 B/clock x %.0f MHz" % (sms, clk),
-                              "note": "ball sums from a TMA-staged ring: %d shared loads per node" % loads,
+                              "note": "%d points per node by the definition; the kernel reads a plane's discs" % loads,
                               "traffic": traffic_for("contact", name, prec)}
         else:
             # spectral contact stage: M densities embedded and transformed forward, ball spectra applied,
@@ -581,11 +582,14 @@ def shell_roofline(w, prec, N, M, stage, peaks, peaks_kind, sms, wname, shell_me
     else:
         S_list = [int(round(0.5 * (w["sigma"][a] + w["sigma"][b]))) for a in range(M) for b in range(M)]
         flops = sum(shell_flops_per_node(S) for S in S_list) * N
-        per_launch_flops = flops / len(S_list)
+        per_launch_flops = flops / len(S_list)  # the stage counts pairs; one launch takes them all
         achieved = per_launch_flops / (per_launch_ms * 1e-3) / 1e12
         clk = float(peaks.get("sm_max_mhz", 2070.0))
         peak = sms * FP32_LANES_PER_SM * 2 * clk * 1e6 / 1e12 if prec != "fp64" else None
-        roof = {"kernel": "k_shell_force (K3 mean-field shell force)", "bound": "alu", "achieved": achieved,
+        # flops by the definition's half shell; the kernel shares work between outputs and executes fewer
+        name = "k_shell_fixed (K3 mean-field shell force, fixed point)" if prec == "fp64" else \
+            "k_shell_march (K3 mean-field shell force)"
+        roof = {"kernel": name, "bound": "alu", "achieved": achieved,
                 "peak": peak, "unit": "TFLOP/s", "frac": (achieved / peak) if peak else None,
                 "traffic": traffic_for("shell", wname, prec), "algorithmic_flops_per_launch": per_launch_flops,
                 "launches": dom_n, "avg_launch_ms": per_launch_ms,

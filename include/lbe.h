@@ -303,7 +303,7 @@ lbe_status lbe_set_stage_timing(lbe_ctx *ctx, int on);
 #define LBE_NUM_STAGES 5
 enum { LBE_STAGE_DENSITY = 0,  /* K1: pulled zeroth moment into the padded field */
        LBE_STAGE_CONTACT = 1,  /* K2: ball averages and contact values         */
-       LBE_STAGE_SHELL = 2,    /* K3: mean-field shell force, one launch per pair */
+       LBE_STAGE_SHELL = 2,    /* K3: mean-field shell force, counted per pair   */
        LBE_STAGE_COLLIDE = 3,  /* K4: moments + DD-TR collision + streaming     */
        LBE_STAGE_FLUX = 4 };   /* K5: plane flux reduction                      */
 

@@ -814,7 +814,7 @@ lbe_status force_stage_core(lbe_ctx *c, const void *pop, void *Pbase, void *xiba
         LAUNCH(launch_contact_tma(f64, L, c->stream), "contact kernel");
     }
     std::vector<int> first(c->M, 1);
-    StageTimer t(c, LBE_STAGE_SHELL, f64 ? 2 : 1);
+    StageTimer t(c, LBE_STAGE_SHELL, (int)c->pairs.size());  // counted per pair; one launch takes them all
     int Smax = 0, shells[MAXS] = {0};
     auto fill = [&](auto &A, auto zero) {  // the launch's arguments, in the precision of `zero`
         using T = decltype(zero);
