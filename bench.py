@@ -198,7 +198,8 @@ def source_hash(files):
 
 
 KERNEL_SOURCES = {
-    "collide": ["paper_1202_3842_gb300/csrc/lbe_collide_pair.cu", "paper_1202_3842_gb300/csrc/lbe_device.cuh",
+    "collide": ["paper_1202_3842_gb300/csrc/lbe_collide_pair.cu", "paper_1202_3842_gb300/csrc/lbe_collide.cuh",
+                "paper_1202_3842_gb300/csrc/lbe_device.cuh",
                 "paper_1202_3842_gb300/csrc/lbe_node.cuh"],
     "shell": ["paper_1202_3842_gb300/csrc/lbe_shell.cu", "paper_1202_3842_gb300/csrc/lbe_shell.cuh",
               "paper_1202_3842_gb300/csrc/lbe_march.cuh", "paper_1202_3842_gb300/csrc/lbe_shell_march.cuh",
@@ -536,7 +537,7 @@ def collide_roofline(N, M, sb, stage, peaks, peaks_kind, wname, prec):
     alg = N * M * 4 * QPOP * sb
     achieved = alg / (per_launch_ms * 1e-3) / 1e9
     peak = float(peaks["hbm_gbs"])
-    kname = "k_collide_pair" if M <= 2 else "k_collide"
+    kname = "k_collide_pair"
     return {"kernel": kname + " (K4 fused moments + DD-TR collision + streaming)", "bound": "hbm",
             "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
             "traffic": traffic_for("collide", wname, prec), "algorithmic_bytes_per_launch": alg,

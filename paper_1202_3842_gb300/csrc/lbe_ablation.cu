@@ -2,8 +2,8 @@
 //   SD-TR  one distribution f; trapezoidal update; J = J~ + (h/2)(C + nF) with J~ = sum c f~;
 //   SD-EU  one distribution; Euler update f* = f + (1/tau)(f_eq - f) + h S_f; J = sum c f;
 //   DD-EU  two distributions; Euler update of f and g; J = sum c g, Pi = sum g.
-// (DD-TR, the method itself, runs in k_collide.)  Both updates have the form
-//   f* = f + omega_eff (f_eq - f) + inv S,   omega_eff = 1/tau,
+// (DD-TR, the method itself, runs in k_collide_pair.)  Both updates have the form
+//   f* = f + omega_eff (f_eq - f) + inv S,   omega_eff = 1/tau   (lbe_collide.cuh),
 // with inv = 1/(1 + omega h/2) for TR and inv = h for EU (set on the host).  f_eq, g_eq, S_f and
 // S_g are those of the DD-TR kernel; in the SD schemes S_f carries the whole force C + nF and g is
 // not evolved: it is written as a copy of f.  FP64 and FP32 storage, one or two species; every
@@ -11,6 +11,7 @@
 #include <utility>
 
 #include "../../include/lbe.h"
+#include "lbe_collide.cuh"
 #include "lbe_device.cuh"
 #include "lbe_launch.h"
 #include "lbe_node.cuh"
@@ -40,7 +41,7 @@ __global__ void __launch_bounds__(NTA)
     const bool sd = sp.scheme == LBE_SD_TR || sp.scheme == LBE_SD_EU;
     const bool eu = sp.scheme == LBE_SD_EU || sp.scheme == LBE_DD_EU;
     const NbrOff o = nbr_offsets(g, x, y, z);
-    T fv[M][Q], gv[M][Q];
+    T fv[M][Q], gv[M][Q] = {};
     T n[M], Pi[M], J[M][3], Cv[M][3], nF[M][3], ua[M][3];
     T ntot = 0, Jtot[3] = {0, 0, 0};
 #pragma unroll
@@ -52,15 +53,16 @@ __global__ void __launch_bounds__(NTA)
             ((fv[a][P] = pull<S, T, P, SOLID>(fb, g.N, i, o, m, n0)), ...);
             if (!sd) ((gv[a][P] = pull<S, T, P, SOLID>(gb, g.N, i, o, m, n0)), ...);
         }(std::make_integer_sequence<int, Q>{});
-        const T *mom = sd ? fv[a] : gv[a];
-        T na = 0, Pit = 0, Jt[3] = {0, 0, 0};
-        [&]<int... P>(std::integer_sequence<int, P...>) {
-            ((na += fv[a][P]), ...);
-            ((Pit += mom[P]), ...);
-            ((Jt[0] += (T)cx(P) * mom[P]), ...);
-            ((Jt[1] += (T)cy(P) * mom[P]), ...);
-            ((Jt[2] += (T)cz(P) * mom[P]), ...);
-        }(std::make_integer_sequence<int, Q>{});
+        const T na = zeroth_moment<false>(fv[a]);
+        T Pit, Jt[3];
+        if constexpr (sizeof(T) == 4) {
+            Pit = zeroth_moment<false>(sd ? fv[a] : gv[a]);
+            ordered_momentum(sd ? fv[a] : gv[a], Jt);
+        } else if (sd) {
+            pair_moments<false>(fv[a], Pit, Jt);
+        } else {
+            pair_moments<false>(gv[a], Pit, Jt);
+        }
         const T inv_n = na > (T)0 ? (T)1 / na : (T)0;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -83,48 +85,38 @@ __global__ void __launch_bounds__(NTA)
         for (int a = 0; a < M; ++a)
             flux_buf[(long long)a * psize + plane_index(g, sp.flux_axis, x, y, z)] = (double)J[a][sp.flux_axis];
     }
-    const T uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
 #pragma unroll
     for (int a = 0; a < M; ++a) {
-        const T na = n[a];
-        const T uau = ua[a][0] * u[0] + ua[a][1] * u[1] + ua[a][2] * u[2];
-        const T iso = (T)1.5 * na * ((T)2 * uau - uu);
-        const T A = na - iso, B = Pi[a] - iso;
-        T X[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) X[c] = Cv[a][c] + nF[a][c];
-        const T sf0 = (T)-3 * (X[0] * ua[a][0] + X[1] * ua[a][1] + X[2] * ua[a][2]);
-        const T om = (T)sp.sp[a].omega_eff, inv = (T)sp.sp[a].inv;
         const T n0a = (T)sp.sp[a].n0;
-        const T in0 = sp.sp[a].n0 > 0.0 ? (T)(1.0 / sp.sp[a].n0) : (T)0;
+        const T in0 = sp.sp[a].n0 > 0.0 ? (T)sp.sp[a].in0 : (T)0;
         S *fo = dst + pop_off(a, 0, 0, g.N) + i;
         S *go = dst + pop_off(a, 1, 0, g.N) + i;
-        [&]<int... P>(std::integer_sequence<int, P...>) {
+        auto put = [&](auto Pc) {
+            constexpr int P = decltype(Pc)::value;
+            constexpr T w = (T)wq(P), iw = (T)(1.0 / wq(P));
+            Store<S, T>::store(fo + (long long)P * g.N, fv[a][P], w * n0a, iw * in0);
+            Store<S, T>::store(go + (long long)P * g.N, sd ? fv[a][P] : gv[a][P], w * n0a, iw * in0);
+        };
+        if constexpr (sizeof(T) == 4) {  // FP32 on f itself: as it has always rounded (see k_collide_pair)
+            collide_whole(n[a], Pi[a], ua[a], u, Cv[a], nF[a], (T)sp.sp[a].omega_eff, (T)sp.sp[a].inv, fv[a], gv[a]);
+            [&]<int... P>(std::integer_sequence<int, P...>) { (put(std::integral_constant<int, P>{}), ...); }
+            (std::make_integer_sequence<int, Q>{});
+            continue;
+        }
+        Collision<T> col;
+        col.set(n[a], n[a], Pi[a], ua[a], u, Cv[a], nF[a], (T)sp.sp[a].omega_eff, (T)sp.sp[a].inv, (T)0);
+        col.rest(fv[a][0], gv[a][0]);
+        put(std::integral_constant<int, 0>{});
+        [&]<int... K>(std::integer_sequence<int, K...>) {
             (
                 [&] {
-                    constexpr T w = (T)wq(P);
-                    const T cua = cdot<T, P>(ua[a]);
-                    const T cu = cdot<T, P>(u);
-                    const T cX = cdot<T, P>(X);
-                    const T t1 = (T)3 * na * cua + (T)4.5 * na * ((T)2 * cua * cu - cu * cu);
-                    const T feq = w * (A + t1);
-                    const T Sf = w * (sf0 + (T)3 * cX + (T)9 * cX * cua);
-                    const T fs = fv[a][P] + om * (feq - fv[a][P]) + inv * Sf;
-                    constexpr T iw = (T)(1.0 / wq(P));
-                    Store<S, T>::store(fo + (long long)P * g.N, fs, w * n0a, iw * in0);
-                    if (sd) {
-                        Store<S, T>::store(go + (long long)P * g.N, fs, w * n0a, iw * in0);
-                    } else {
-                        const T cY = cdot<T, P>(nF[a]);
-                        const T cC = cdot<T, P>(Cv[a]);
-                        const T geq = w * (B + t1);
-                        const T Sg = w * (sf0 + (T)3 * cY + (T)18 * cC * cua + (T)9 * cY * cua);
-                        const T gs = gv[a][P] + om * (geq - gv[a][P]) + inv * Sg;
-                        Store<S, T>::store(go + (long long)P * g.N, gs, w * n0a, iw * in0);
-                    }
+                    constexpr int P = 2 * K + 1;
+                    col.template pair<P>(fv[a][P], fv[a][P + 1], gv[a][P], gv[a][P + 1]);
+                    put(std::integral_constant<int, P>{});
+                    put(std::integral_constant<int, P + 1>{});
                 }(),
                 ...);
-        }(std::make_integer_sequence<int, Q>{});
+        }(std::make_integer_sequence<int, 9>{});
     }
 }
 

@@ -51,6 +51,7 @@ enum : int {
 //   store(p, f, wn0, iwn0)       <- f
 //   load_dev(p, wn0)             -> d = f - w_p n0
 //   store_dev(p, d, wn0, iwn0)   <- d
+//   load_unit(p), store_unit(p, v)  the stored number itself (FP64 f, FP32 d, 16-bit s)
 // with wn0 = w_p n0 and iwn0 = 1/(w_p n0).  The fused collision works on the
 // deviations throughout, so its rounding is relative to them as well.
 // ---------------------------------------------------------------------------
@@ -59,6 +60,8 @@ struct Store;
 
 template <>
 struct Store<double, double> {
+    static __device__ __forceinline__ double load_unit(const double *p) { return __ldg(p); }
+    static __device__ __forceinline__ void store_unit(double *p, double v) { *p = v; }
     static __device__ __forceinline__ double load(const double *p, double) { return __ldg(p); }
     static __device__ __forceinline__ void store(double *p, double v, double, double) { *p = v; }
     static __device__ __forceinline__ double load_dev(const double *p, double wn0) { return __ldg(p) - wn0; }
@@ -67,6 +70,8 @@ struct Store<double, double> {
 };
 template <>
 struct Store<float, float> {
+    static __device__ __forceinline__ float load_unit(const float *p) { return __ldg(p); }
+    static __device__ __forceinline__ void store_unit(float *p, float v) { *p = v; }
     static __device__ __forceinline__ float load(const float *p, float wn0) { return __ldg(p) + wn0; }
     static __device__ __forceinline__ void store(float *p, float v, float wn0, float) { *p = v - wn0; }
     static __device__ __forceinline__ float load_dev(const float *p, float) { return __ldg(p); }
@@ -75,6 +80,8 @@ struct Store<float, float> {
 };
 template <>
 struct Store<__nv_bfloat16, float> {
+    static __device__ __forceinline__ float load_unit(const __nv_bfloat16 *p) { return __bfloat162float(__ldg(p)); }
+    static __device__ __forceinline__ void store_unit(__nv_bfloat16 *p, float v) { *p = __float2bfloat16_rn(v); }
     static __device__ __forceinline__ float load(const __nv_bfloat16 *p, float wn0) {
         return fmaf(wn0, __bfloat162float(__ldg(p)), wn0);
     }
@@ -91,6 +98,8 @@ struct Store<__nv_bfloat16, float> {
 };
 template <>
 struct Store<__half, float> {
+    static __device__ __forceinline__ float load_unit(const __half *p) { return __half2float(__ldg(p)); }
+    static __device__ __forceinline__ void store_unit(__half *p, float v) { *p = __float2half_rn(v); }
     static __device__ __forceinline__ float load(const __half *p, float wn0) {
         return fmaf(wn0, __half2float(__ldg(p)), wn0);
     }
@@ -137,9 +146,14 @@ __device__ __forceinline__ bool wrap(int &v, int n, int periodic) {
 template <typename T>
 __device__ __forceinline__ void write_padded(const Grid &g, T *f, int x, int y, int z, T v) {
     int kx0 = 0, kx1 = 0, ky0 = 0, ky1 = 0, kz0 = 0, kz1 = 0;
-    if (g.per[0]) { kx0 = -((x + g.H) / g.nx); kx1 = (g.nx + g.H - 1 - x) / g.nx; }
-    if (g.per[1]) { ky0 = -((y + g.H) / g.ny); ky1 = (g.ny + g.H - 1 - y) / g.ny; }
-    if (g.per[2]) { kz0 = -((z + g.H) / g.nz); kz1 = (g.nz + g.H - 1 - z) / g.nz; }
+    // only nodes within H of a side have images: the others skip the divisions
+    if (g.per[0] && (x < g.H || x >= g.nx - g.H)) { kx0 = -((x + g.H) / g.nx); kx1 = (g.nx + g.H - 1 - x) / g.nx; }
+    if (g.per[1] && (y < g.H || y >= g.ny - g.H)) { ky0 = -((y + g.H) / g.ny); ky1 = (g.ny + g.H - 1 - y) / g.ny; }
+    if (g.per[2] && (z < g.H || z >= g.nz - g.H)) { kz0 = -((z + g.H) / g.nz); kz1 = (g.nz + g.H - 1 - z) / g.nz; }
+    if ((kx0 | kx1 | ky0 | ky1 | kz0 | kz1) == 0) {
+        f[pidx(g, x, y, z)] = v;
+        return;
+    }
     for (int kz = kz0; kz <= kz1; ++kz)
         for (int ky = ky0; ky <= ky1; ++ky)
             for (int kx = kx0; kx <= kx1; ++kx)

@@ -1,7 +1,6 @@
 // D3Q19 Lattice Boltzmann-Enskog kernels (sm_103a): geometry, force field,
-// population set/get, K1 density, K2 contact values, K4 fused DD-TR
-// collide-stream, moments and FP64 reductions.  The shell force (K3) is in
-// lbe_shell.cu.
+// population set/get, K1 density, moments and FP64 reductions.  The contact values (K2) are in lbe_contact.cuh,
+// the shell force (K3) in lbe_shell_march.cuh and lbe_shell_fixed.cuh, the collision (K4) in lbe_collide_pair.cu.
 //
 // Population storage: [M][2 (f, g)][19][N] of the storage type S, holding the
 // post-collision populations f~*(r, t-1); the streamed populations of step t
@@ -12,6 +11,7 @@
 
 #include <utility>
 
+#include "lbe_collide.cuh"
 #include "lbe_device.cuh"
 #include "lbe_launch.h"
 #include "lbe_node.cuh"
@@ -229,14 +229,13 @@ cudaError_t launch_stream_out(Prec p, const Grid &g, const uint32_t *mask, const
 // ---------------------------------------------------------------------------
 template <typename S, typename T, bool SOLID, int MC>
 __global__ void __launch_bounds__(NT) k_density(Grid g, const S *__restrict__ pop, const uint32_t *__restrict__ mask,
-                                                int M, N0Vec n0v, N0VecF n0f, T *__restrict__ npad,
-                                                int *err) {
+                                                N0Vec n0v, N0VecF n0f, T *__restrict__ npad, int *err) {
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const bool valid = i < g.N;
     const uint32_t m = valid ? (SOLID ? mask[i] : 0u) : 1u;
-    // two species: a warp none of whose nodes has a blocked link pulls without the bounce-back selects
+    // a warp none of whose nodes has a blocked link pulls without the bounce-back selects
     // (0.257 -> 0.227 ms on the 512x128x128 channel)
-    const bool plain = MC == 2 && (!SOLID || __all_sync(0xffffffffu, (m >> 1) == 0u));
+    const bool plain = (!SOLID || __all_sync(0xffffffffu, (m >> 1) == 0u));
     if (!valid) return;
     int x, y, z;
     node_xyz(g, i, x, y, z);
@@ -247,65 +246,42 @@ __global__ void __launch_bounds__(NT) k_density(Grid g, const S *__restrict__ po
         else
             return (T)n0v.v[a];
     };
-    // one species' pulled populations (shifted storage: their deviations from w_p n0)
-    auto pull_all = [&](int a, T *v) {
-        const S *fb = pop + pop_off(a, 0, 0, g.N);
-        const T n0 = n0_of(a);
-        if (plain) {
-            [&]<int... P>(std::integer_sequence<int, P...>) {
-                if constexpr (Store<S, T>::shifted)
-                    ((v[P] = pull_dev<S, T, P, false>(fb, g.N, i, o, m, n0)), ...);
-                else
-                    ((v[P] = pull<S, T, P, false>(fb, g.N, i, o, m, n0)), ...);
-            }(std::make_integer_sequence<int, Q>{});
-        } else {
-            [&]<int... P>(std::integer_sequence<int, P...>) {
-                if constexpr (Store<S, T>::shifted)
-                    ((v[P] = pull_dev<S, T, P, SOLID>(fb, g.N, i, o, m, n0)), ...);
-                else
-                    ((v[P] = pull<S, T, P, SOLID>(fb, g.N, i, o, m, n0)), ...);
-            }(std::make_integer_sequence<int, Q>{});
-        }
+    auto pull_species = [&](int a, T(&v)[Q]) {
+        pull_all<S, T, SOLID>(pop + pop_off(a, 0, 0, g.N), g.N, i, o, m, plain, v);
     };
-    // n = n0 + the sum of the deviations (shifted storage), the sum itself otherwise
     auto finish = [&](int a, const T *v) -> T {
-        T n = (T)0;
-#pragma unroll
-        for (int p = 0; p < Q; ++p) n += v[p];
-        if constexpr (Store<S, T>::shifted) n = n0_of(a) + n;
+        const T n = density_of<S, T>(v, n0_of(a));
         if (!(n >= (T)0) || !isfinite(n)) atomicOr(err, ERR_DENSITY);
         return n;
     };
-    if constexpr (MC == 2) {
-        // two species: all 38 loads issue before either sum
-        T n[2] = {(T)0, (T)0};
-        if (!(m & 1u)) {
+    T n[MC];
+#pragma unroll
+    for (int a = 0; a < MC; ++a) n[a] = (T)0;
+    if (!(m & 1u)) {
+        if constexpr (MC == 2) {  // all 38 loads issue before either sum
             T v0[Q], v1[Q];
-            pull_all(0, v0);
-            pull_all(1, v1);
+            pull_species(0, v0);
+            pull_species(1, v1);
             n[0] = finish(0, v0);
             n[1] = finish(1, v1);
-        }
-        write_padded<T>(g, npad, x, y, z, n[0]);
-        write_padded<T>(g, npad + g.P, x, y, z, n[1]);
-    } else {
-        for (int a = 0; a < M; ++a) {
-            T n = (T)0;
-            if (!(m & 1u)) {
+        } else {
+#pragma unroll
+            for (int a = 0; a < MC; ++a) {
                 T v[Q];
-                pull_all(a, v);
-                n = finish(a, v);
+                pull_species(a, v);
+                n[a] = finish(a, v);
             }
-            write_padded<T>(g, npad + (long long)a * g.P, x, y, z, n);
         }
     }
+#pragma unroll
+    for (int a = 0; a < MC; ++a) write_padded<T>(g, npad + (long long)a * g.P, x, y, z, n[a]);
 }
 
 cudaError_t launch_density(Prec p, const Grid &g, const void *pop, const uint32_t *mask, bool solid, int M,
                            const double *n0, void *npad, int *err, cudaStream_t st) {
     // one species: one thread per node at 32-42 registers (lbe_collide_pair.cu); measured faster than this
     // kernel for one species (256^3 well 0.42 -> 0.31 ms) and slower for two (0.29 -> 0.31 ms)
-    if (M == 1) return launch_density_pair(p, g, pop, mask, solid, M, n0, npad, err, st);
+    if (M == 1) return launch_density_pair(p, g, pop, mask, solid, n0[0], npad, err, st);
     unsigned nb = (unsigned)((g.N + NT - 1) / NT);
     N0Vec n0v;
     N0VecF n0f;
@@ -314,211 +290,31 @@ cudaError_t launch_density(Prec p, const Grid &g, const void *pop, const uint32_
         n0f.v[a] = (float)n0v.v[a];
     }
 #define LBE_K1(SOL, MC) \
-    LBE_DISPATCH_PREC(p, (k_density<S, T, SOL, MC><<<nb, NT, 0, st>>>(g, (const S *)pop, mask, M, n0v, n0f, (T *)npad, err)))
-    if (M == 2) {
-        if (solid) {
-            LBE_K1(true, 2);
-        } else {
-            LBE_K1(false, 2);
-        }
-    } else if (solid) {
-        LBE_K1(true, 0);
-    } else {
-        LBE_K1(false, 0);
+    LBE_DISPATCH_PREC(p, (k_density<S, T, SOL, MC><<<nb, NT, 0, st>>>(g, (const S *)pop, mask, n0v, n0f, (T *)npad, err)))
+#define LBE_K1_M(MC)       \
+    if (solid) {           \
+        LBE_K1(true, MC);  \
+    } else {               \
+        LBE_K1(false, MC); \
     }
+    switch (M) {
+        case 2: LBE_K1_M(2) break;
+        case 3: LBE_K1_M(3) break;
+        case 4: LBE_K1_M(4) break;
+        default: return cudaErrorInvalidValue;
+    }
+#undef LBE_K1_M
 #undef LBE_K1
     return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
-// K4: fused moments + DD-TR collision + streaming (Sec. "Hard sphere fluid
-// mixture in a potential well"):
+// Moments of the current state (the collision itself: lbe_collide_pair.cu):
 //   n = sum f~, Pi~ = sum g~, J~ = sum c g~;
-//   printed recovery:    J = J~ + (C + nF)/2,  Pi = Pi~ - C.u^a/2;
-//   consistent recovery: J = J~ + nF/2,        Pi = Pi~ + beta C.u^a/2;
-//   u^a = J/n, u = sum J / sum n;
-//   f_eq = w [n + n u^a.H1 + n (2 u^a u - u u):H2],  g_eq = same with Pi first;
-//   S_f = w (C + nF).[H1 + 2 H2.u^a];
-//   S_g = w { C.[u^a/v_T^2 + 4 H2.u^a] + nF.[H1 + 2 H2.u^a] };
-//   f~* = f~ + [omega (f_eq - f~) + S_f] / (1 + omega/2)   (same for g~).
-// With v_T^2 = 1/3 the Hermite contractions expand to the scalar forms below
-// (A, B isotropic parts; sf0 = -3 (C + nF).u^a is shared by S_f and S_g).
+//   printed recovery:    J = J~ + (C + nF)/2;
+//   consistent recovery: J = J~ + nF/2.
 // ---------------------------------------------------------------------------
-// Per-node moments of every species.  With KEEP the pulled populations stay
-// in registers for the collision (one species); otherwise they are pulled
-// again species by species in the collision pass (the second pull hits L2).
-template <typename S, typename T, int M, bool KEEP>
-struct NodeState {
-    T f[KEEP ? M : 1][Q], g[KEEP ? M : 1][Q];
-    T n[M], Pi[M], J[M][3], C[M][3], nF[M][3], ua[M][3];
-    T u[3];
-};
-
-template <typename S, typename T, bool SOLID>
-__device__ __forceinline__ void pull_species(const Grid &g, const S *__restrict__ src, int a, T n0, long long i,
-                                             const NbrOff &o, uint32_t m, T *f, T *gq) {
-    const S *fb = src + pop_off(a, 0, 0, g.N);
-    const S *gb = src + pop_off(a, 1, 0, g.N);
-    [&]<int... P>(std::integer_sequence<int, P...>) {
-        ((f[P] = pull<S, T, P, SOLID>(fb, g.N, i, o, m, n0)), ...);
-        ((gq[P] = pull<S, T, P, SOLID>(gb, g.N, i, o, m, n0)), ...);
-    }(std::make_integer_sequence<int, Q>{});
-}
-
-template <typename S, typename T, int M, bool SOLID, bool KEEP>
-__device__ __forceinline__ void load_moments(const Grid &g, const S *__restrict__ src, const T *__restrict__ C,
-                                             const T *__restrict__ F, const StepParams &sp, long long i,
-                                             const NbrOff &o, uint32_t m, NodeState<S, T, M, KEEP> &st) {
-    T ntot = 0, Jtot[3] = {0, 0, 0};
-#pragma unroll
-    for (int a = 0; a < M; ++a) {
-        const T n0 = sc_n0<S, T>(sp.sp[a]);
-        T fl[Q], gl[Q];
-        T *f = KEEP ? st.f[KEEP ? a : 0] : fl;
-        T *gq = KEEP ? st.g[KEEP ? a : 0] : gl;
-        pull_species<S, T, SOLID>(g, src, a, n0, i, o, m, f, gq);
-        T n = 0, Pit = 0, Jt[3] = {0, 0, 0};
-        [&]<int... P>(std::integer_sequence<int, P...>) {
-            ((n += f[P]), ...);
-            ((Pit += gq[P]), ...);
-            ((Jt[0] += (T)cx(P) * gq[P]), ...);
-            ((Jt[1] += (T)cy(P) * gq[P]), ...);
-            ((Jt[2] += (T)cz(P) * gq[P]), ...);
-        }(std::make_integer_sequence<int, Q>{});
-        const T *Ca = C + (long long)a * 3 * g.N + i;
-        const T *Fa = F + (long long)a * 3 * g.N + i;
-        T Cu = 0;
-        const T inv_n = n > (T)0 ? (T)1 / n : (T)0;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            st.C[a][c] = Ca[(long long)c * g.N];
-            st.nF[a][c] = n * Fa[(long long)c * g.N];
-            st.J[a][c] = sp.consistent ? Jt[c] + (T)0.5 * st.nF[a][c]
-                                       : Jt[c] + (T)0.5 * (st.C[a][c] + st.nF[a][c]);
-            st.ua[a][c] = st.J[a][c] * inv_n;
-            Cu += st.C[a][c] * st.ua[a][c];
-            Jtot[c] += st.J[a][c];
-        }
-        st.n[a] = n;
-        st.Pi[a] = sp.consistent ? Pit + (T)1.5 * Cu : Pit - (T)0.5 * Cu;
-        ntot += n;
-    }
-    const T inv_tot = ntot > (T)0 ? (T)1 / ntot : (T)0;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) st.u[c] = Jtot[c] * inv_tot;
-}
-
-template <typename S, typename T, int M, bool SOLID>
-__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? (M == 1 ? 3 : 2) : 1)
-    k_collide(Grid g, const S *__restrict__ src, S *__restrict__ dst,
-                                                const uint32_t *__restrict__ mask, const T *__restrict__ C,
-                                                const T *__restrict__ F, StepParams sp,
-                                                double *__restrict__ flux_buf) {
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= g.N) return;
-    int x, y, z;
-    node_xyz(g, i, x, y, z);
-    const uint32_t m = SOLID ? mask[i] : 0u;
-    const int coord = sp.flux_axis == 0 ? x : (sp.flux_axis == 1 ? y : z);
-    const bool on_plane = sp.flux_axis >= 0 && coord == sp.flux_plane;
-    const int psize = sp.flux_axis == 0 ? g.ny * g.nz : (sp.flux_axis == 1 ? g.nx * g.nz : g.nx * g.ny);
-    if (m & 1u) {  // solid node: no fluid
-        if (on_plane)
-            for (int a = 0; a < M; ++a) flux_buf[(long long)a * psize + plane_index(g, sp.flux_axis, x, y, z)] = 0.0;
-        return;
-    }
-    const NbrOff o = nbr_offsets(g, x, y, z);
-    constexpr bool KEEP = (M == 1);
-    NodeState<S, T, M, KEEP> st;
-    load_moments<S, T, M, SOLID, KEEP>(g, src, C, F, sp, i, o, m, st);
-    if (on_plane) {
-#pragma unroll
-        for (int a = 0; a < M; ++a)
-            flux_buf[(long long)a * psize + plane_index(g, sp.flux_axis, x, y, z)] = (double)st.J[a][sp.flux_axis];
-    }
-#pragma unroll
-    for (int a = 0; a < M; ++a) {
-        const T n = st.n[a];
-        const T *ua = st.ua[a];
-        const T uau = ua[0] * st.u[0] + ua[1] * st.u[1] + ua[2] * st.u[2];
-        const T uu = st.u[0] * st.u[0] + st.u[1] * st.u[1] + st.u[2] * st.u[2];
-        const T iso = (T)1.5 * n * ((T)2 * uau - uu);
-        const T A = n - iso;
-        const T B = st.Pi[a] - iso;
-        T X[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) X[c] = st.C[a][c] + st.nF[a][c];
-        const T sf0 = (T)-3 * (X[0] * ua[0] + X[1] * ua[1] + X[2] * ua[2]);
-        const T om = sc_omega<S, T>(sp.sp[a]);
-        const T inv = sc_inv<S, T>(sp.sp[a]);
-        const T in0 = sc_in0<S, T>(sp.sp[a]);
-        T fl[Q], gl[Q];
-        const T *fa = st.f[0];
-        const T *ga = st.g[0];
-        if constexpr (KEEP) {
-            fa = st.f[KEEP ? a : 0];
-            ga = st.g[KEEP ? a : 0];
-        } else {
-            pull_species<S, T, SOLID>(g, src, a, sc_n0<S, T>(sp.sp[a]), i, o, m, fl, gl);
-            fa = fl;
-            ga = gl;
-        }
-        S *fo = dst + pop_off(a, 0, 0, g.N) + i;
-        S *go = dst + pop_off(a, 1, 0, g.N) + i;
-        [&]<int... P>(std::integer_sequence<int, P...>) {
-            (
-                [&] {
-                    constexpr T w = (T)wq(P);
-                    const T cua = cdot<T, P>(ua);
-                    const T cu = cdot<T, P>(st.u);
-                    const T cX = cdot<T, P>(X);
-                    const T cY = cdot<T, P>(st.nF[a]);
-                    const T cC = cdot<T, P>(st.C[a]);
-                    const T t1 = (T)3 * n * cua + (T)4.5 * n * ((T)2 * cua * cu - cu * cu);
-                    const T feq = w * (A + t1);
-                    const T geq = w * (B + t1);
-                    const T Sf = w * (sf0 + (T)3 * cX + (T)9 * cX * cua);
-                    const T Sg = w * (sf0 + (T)3 * cY + (T)18 * cC * cua + (T)9 * cY * cua);
-                    const T fs = fa[P] + om * (feq - fa[P]) + inv * Sf;
-                    const T gs = ga[P] + om * (geq - ga[P]) + inv * Sg;
-                    constexpr T iw = (T)(1.0 / wq(P));
-                    Store<S, T>::store(fo + (long long)P * g.N, fs, w * sc_n0<S, T>(sp.sp[a]), iw * in0);
-                    Store<S, T>::store(go + (long long)P * g.N, gs, w * sc_n0<S, T>(sp.sp[a]), iw * in0);
-                }(),
-                ...);
-        }(std::make_integer_sequence<int, Q>{});
-    }
-}
-
-template <typename S, typename T, bool SOLID>
-static cudaError_t collide_m(int M, const Grid &g, const void *src, void *dst, const uint32_t *mask, const void *C,
-                             const void *F, const StepParams &sp, double *flux_buf, cudaStream_t st) {
-    unsigned nb = (unsigned)((g.N + NT - 1) / NT);
-#define LBE_COLLIDE(MM)                                                                                   \
-    k_collide<S, T, MM, SOLID><<<nb, NT, 0, st>>>(g, (const S *)src, (S *)dst, mask, (const T *)C, (const T *)F, \
-                                                  sp, flux_buf)
-    switch (M) {  // one or two species: k_collide_pair (lbe_collide_pair.cu)
-        case 3: LBE_COLLIDE(3); break;
-        case 4: LBE_COLLIDE(4); break;
-        default: return cudaErrorInvalidValue;
-    }
-#undef LBE_COLLIDE
-    return cudaGetLastError();
-}
-
-cudaError_t launch_collide(Prec p, const Grid &g, const void *src, void *dst, const uint32_t *mask, bool solid,
-                           const void *C, const void *F, const StepParams &sp, double *flux_buf, cudaStream_t st) {
-    if (sp.M <= 2) return launch_collide_pair(p, g, src, dst, mask, solid, C, F, sp, flux_buf, st);
-    cudaError_t e = cudaSuccess;
-    if (solid) {
-        LBE_DISPATCH_PREC(p, (e = collide_m<S, T, true>(sp.M, g, src, dst, mask, C, F, sp, flux_buf, st)));
-    } else {
-        LBE_DISPATCH_PREC(p, (e = collide_m<S, T, false>(sp.M, g, src, dst, mask, C, F, sp, flux_buf, st)));
-    }
-    return e;
-}
-
-// Moments of the current state for the getters: n [M][N], J [M][3][N] (FP64).
+// For the getters: n [M][N], J [M][3][N] (FP64).
 template <typename S, typename T, int M>
 __global__ void __launch_bounds__(NT) k_moments(Grid g, const S *__restrict__ src, const uint32_t *__restrict__ mask,
                                                 const T *__restrict__ C, const T *__restrict__ F, StepParams sp,
@@ -528,19 +324,36 @@ __global__ void __launch_bounds__(NT) k_moments(Grid g, const S *__restrict__ sr
     int x, y, z;
     node_xyz(g, i, x, y, z);
     const uint32_t m = mask[i];
-    if (m & 1u) {
-        for (int a = 0; a < M; ++a) {
-            nout[(long long)a * g.N + i] = 0.0;
-            for (int c = 0; c < 3; ++c) Jout[((long long)a * 3 + c) * g.N + i] = 0.0;
-        }
-        return;
-    }
-    const NbrOff o = nbr_offsets(g, x, y, z);
-    NodeState<S, T, M, false> st;
-    load_moments<S, T, M, true, false>(g, src, C, F, sp, i, o, m, st);
+    const bool solid = m & 1u;
+    NbrOff o{};
+    if (!solid) o = nbr_offsets(g, x, y, z);
+#pragma unroll
     for (int a = 0; a < M; ++a) {
-        nout[(long long)a * g.N + i] = (double)st.n[a];
-        for (int c = 0; c < 3; ++c) Jout[((long long)a * 3 + c) * g.N + i] = (double)st.J[a][c];
+        T n = 0, J[3] = {0, 0, 0};
+        if (!solid) {
+            const T n0 = sc_n0<S, T>(sp.sp[a]);
+            const S *fb = src + pop_off(a, 0, 0, g.N);
+            const S *gb = src + pop_off(a, 1, 0, g.N);
+            T f[Q], gq[Q], Pi;
+            [&]<int... P>(std::integer_sequence<int, P...>) {
+                ((f[P] = pull<S, T, P, true>(fb, g.N, i, o, m, n0)), ...);
+                ((gq[P] = pull<S, T, P, true>(gb, g.N, i, o, m, n0)), ...);
+            }(std::make_integer_sequence<int, Q>{});
+            n = zeroth_moment<false>(f);
+            if constexpr (sizeof(T) == 4)  // rounds as the getters always have
+                ordered_momentum(gq, J);
+            else
+                pair_moments<false>(gq, Pi, J);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const T Cc = C[((long long)a * 3 + c) * g.N + i];
+                const T nF = n * F[((long long)a * 3 + c) * g.N + i];
+                J[c] += (T)0.5 * (sp.consistent ? nF : Cc + nF);
+            }
+        }
+        nout[(long long)a * g.N + i] = (double)n;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) Jout[((long long)a * 3 + c) * g.N + i] = (double)J[c];
     }
 }
 

@@ -63,7 +63,7 @@ __host__ __device__ __forceinline__ T sc_in0(const SpeciesConst &s) {
 
 struct StepParams {
     int M;
-    int scheme;          // lbe_scheme: DD_TR (k_collide) or an ablation (k_collide_ablation)
+    int scheme;          // lbe_scheme: DD_TR (k_collide_pair) or an ablation (k_collide_ablation)
     int consistent;      // moment recovery: 0 printed, 1 map-consistent
     int flux_axis;       // -1: no flux plane
     int flux_plane;
@@ -159,13 +159,9 @@ cudaError_t launch_collide_ablation(Prec p, const Grid &g, const void *src, void
                                     double *flux_buf, cudaStream_t st);
 cudaError_t launch_moments_ablation(Prec p, const Grid &g, const void *pop, const uint32_t *mask, const void *C,
                                     const void *F, const StepParams &sp, double *n, double *J, cudaStream_t st);
-// K1 for one or two species, species-parallel lanes (lbe_collide_pair.cu).
-cudaError_t launch_density_pair(Prec p, const Grid &g, const void *pop, const uint32_t *mask, bool solid, int M,
-                                const double *n0, void *npad, int *err, cudaStream_t st);
-// K4 for one or two species, species-parallel lanes (lbe_collide_pair.cu).
-cudaError_t launch_collide_pair(Prec p, const Grid &g, const void *src, void *dst, const uint32_t *mask, bool solid,
-                                const void *C, const void *F, const StepParams &sp, double *flux_buf,
-                                cudaStream_t st);
+// K1 for one species (lbe_collide_pair.cu).
+cudaError_t launch_density_pair(Prec p, const Grid &g, const void *pop, const uint32_t *mask, bool solid,
+                                double n0, void *npad, int *err, cudaStream_t st);
 // Moments of the current state (FP64 out): n [M][N], J [M][3][N].
 cudaError_t launch_moments(Prec p, const Grid &g, const void *pop, const uint32_t *mask, const void *C,
                            const void *F, const StepParams &sp, double *n, double *J, cudaStream_t st);

@@ -80,6 +80,33 @@ __device__ __forceinline__ T pull_dev(const S *__restrict__ fg_base, long long N
     }
 }
 
+// The pulls of the step's kernels (K1, K4), in the units the storage form computes in:
+//   FP64: f itself;  FP32: the deviation d = f - w_p n0 as stored;  16 bits: s = d / (w_p n0) as stored.
+template <typename S, typename T, int P, bool SOLID>
+__device__ __forceinline__ T pull_unit(const S *__restrict__ fg_base, long long N, long long i, const NbrOff &o,
+                                       uint32_t m) {
+    if constexpr (SOLID) {
+        const long long off = (m & (1u << P)) ? (long long)opp(P) * N + i : (long long)P * N + i + src_off<P>(o);
+        return Store<S, T>::load_unit(fg_base + off);
+    } else {
+        return Store<S, T>::load_unit(fg_base + (long long)P * N + i + src_off<P>(o));
+    }
+}
+// All 19 of one distribution; a warp without blocked links (plain) pulls without the bounce-back selects.
+template <typename S, typename T, bool SOLID>
+__device__ __forceinline__ void pull_all(const S *__restrict__ fg_base, long long N, long long i, const NbrOff &o,
+                                         uint32_t m, bool plain, T (&v)[Q]) {
+    if (plain) {
+        [&]<int... P>(std::integer_sequence<int, P...>) {
+            ((v[P] = pull_unit<S, T, P, false>(fg_base, N, i, o, m)), ...);
+        }(std::make_integer_sequence<int, Q>{});
+    } else {
+        [&]<int... P>(std::integer_sequence<int, P...>) {
+            ((v[P] = pull_unit<S, T, P, SOLID>(fg_base, N, i, o, m)), ...);
+        }(std::make_integer_sequence<int, Q>{});
+    }
+}
+
 template <typename T, int P>
 __device__ __forceinline__ T cdot(const T *v) {
     T r = (T)0;
