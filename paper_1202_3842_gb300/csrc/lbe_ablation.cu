@@ -25,6 +25,7 @@ __global__ void __launch_bounds__(NTA)
     k_collide_ablation(Grid g, const S *__restrict__ src, S *__restrict__ dst, const uint32_t *__restrict__ mask,
                        const T *__restrict__ C, const T *__restrict__ F, StepParams sp,
                        double *__restrict__ flux_buf) {
+    pdl_wait();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= g.N) return;
     int x, y, z;
@@ -176,9 +177,10 @@ cudaError_t launch_collide_ablation(Prec p, const Grid &g, const void *src, void
                                     bool solid, const void *C, const void *F, const StepParams &sp,
                                     double *flux_buf, cudaStream_t st) {
     const unsigned nb = (unsigned)((g.N + NTA - 1) / NTA);
+    cudaError_t e = cudaSuccess;
 #define LBE_ABL(MM, SOL)                                                                                    \
-    k_collide_ablation<S, T, MM, SOL><<<nb, NTA, 0, st>>>(g, (const S *)src, (S *)dst, mask, (const T *)C, \
-                                                          (const T *)F, sp, flux_buf)
+    e = launch_pdl(k_collide_ablation<S, T, MM, SOL>, nb, NTA, 0, st, g, (const S *)src, (S *)dst, mask,   \
+                   (const T *)C, (const T *)F, sp, flux_buf)
     LBE_ABL_DISPATCH(p, {
         if (sp.M == 1) {
             if (solid) LBE_ABL(1, true); else LBE_ABL(1, false);
@@ -189,7 +191,7 @@ cudaError_t launch_collide_ablation(Prec p, const Grid &g, const void *src, void
         }
     });
 #undef LBE_ABL
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_moments_ablation(Prec p, const Grid &g, const void *pop, const uint32_t *mask, const void *C,

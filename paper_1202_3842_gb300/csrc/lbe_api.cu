@@ -531,7 +531,7 @@ lbe_status spectral_force(lbe_ctx *c, void *Pbase, void *xibase) {
     return LBE_OK;
 }
 
-// Shell tables of the viscous force (the pairs' shells, offsets and unit vectors in FP64) and its
+// Shell tables of the viscous force (the pairs' shells: offsets, and unit vectors in the arithmetic's type) and its
 // fields: the tilde velocities and the effective force F + C^visc / n.
 lbe_status visc_setup(lbe_ctx *c) {
     const size_t rb = real_bytes(c);
@@ -560,13 +560,15 @@ lbe_status visc_setup(lbe_ctx *c) {
     }
     c->vp = vp;
     TRY(dev_alloc(c, c->veoff, sizeof(int) * std::max<size_t>(eo.size(), 3)));
-    TRY(dev_alloc(c, c->vehat, sizeof(double) * std::max<size_t>(eh.size(), 3)));
+    const std::vector<float> ef(eh.begin(), eh.end());
+    const void *const eh_data = rb == 8 ? (const void *)eh.data() : (const void *)ef.data();
+    TRY(dev_alloc(c, c->vehat, rb * std::max<size_t>(eh.size(), 3)));
     TRY(dev_alloc(c, c->vut, rb * 3 * (size_t)c->M * N));
     TRY(dev_alloc(c, c->Feff, rb * 3 * (size_t)c->M * N));
     if (!eo.empty()) {
         CK(cudaMemcpyAsync(c->veoff.p, eo.data(), sizeof(int) * eo.size(), cudaMemcpyHostToDevice, c->stream),
            "copy viscous shell offsets");
-        CK(cudaMemcpyAsync(c->vehat.p, eh.data(), sizeof(double) * eh.size(), cudaMemcpyHostToDevice, c->stream),
+        CK(cudaMemcpyAsync(c->vehat.p, eh_data, rb * eh.size(), cudaMemcpyHostToDevice, c->stream),
            "copy viscous shell vectors");
         CK(cudaStreamSynchronize(c->stream), "stream sync");  // the host tables die here
     }
@@ -781,7 +783,7 @@ lbe_status update_refs(lbe_ctx *c) {
 // npad, gab, gnpad, C.  With Pbase, the shell kernels also store P of every
 // pair into Pbase [npairs][3][N], and with xibase the contact kernel stores
 // xi2, xi3 into xibase [2][N] (both for the adjoint).
-lbe_status force_stage_core(lbe_ctx *c, const void *pop, void *Pbase, void *xibase) {
+lbe_status force_stage_core(lbe_ctx *c, const void *pop, void *Pbase, void *xibase, bool shell = true) {
     const bool f64 = prec_fp64(c->prec);
     const size_t rb = real_bytes(c);
     if (!pop) pop = c->pop[c->cur].p;
@@ -813,6 +815,7 @@ lbe_status force_stage_core(lbe_ctx *c, const void *pop, void *Pbase, void *xiba
         L.err = (int *)c->err.p;
         LAUNCH(launch_contact_tma(f64, L, c->stream), "contact kernel");
     }
+    if (!shell) return LBE_OK;
     std::vector<int> first(c->M, 1);
     StageTimer t(c, LBE_STAGE_SHELL, (int)c->pairs.size());  // counted per pair; one launch takes them all
     int Smax = 0, shells[MAXS] = {0};
@@ -866,7 +869,7 @@ lbe_status force_stage(lbe_ctx *c, const void *pop = nullptr, void *Pbase = null
     if (c->cfg.enable_visc && !c->pairs.empty()) {
         StageTimer t(c, LBE_STAGE_SHELL);
         LAUNCH(launch_visc(c->prec, c->g, pop, (const uint32_t *)c->mask.p, c->npad.p, c->gab.p, c->F.p,
-                           step_params(c), c->vp, (const int *)c->veoff.p, (const double *)c->vehat.p, c->vut.p,
+                           step_params(c), c->vp, (const int *)c->veoff.p, c->vehat.p, c->vut.p,
                            c->Feff.p, c->stream),
                "viscous force");
         c->launches += 1;  // two kernels
@@ -1273,9 +1276,15 @@ lbe_status lbe_step(lbe_ctx *c, int nsteps) {
 lbe_status lbe_get_density(lbe_ctx *c, int s, double *out) {
     TRY(ready(c));
     if (s < 0 || s >= c->M || !out) return fail(c, LBE_ERR_INVALID_ARG, "bad species index or null output");
-    double *n, *J;
-    TRY(state_moments(c, &n, &J));
-    CK(cudaMemcpyAsync(out, n + (long long)s * c->g.N, 8 * c->g.N, cudaMemcpyDeviceToHost, c->stream), "copy density");
+    // K1 holds the density; K2 follows for its check of the packing (the spectral form runs its force stage)
+    const long long N = c->g.N;
+    TRY(prepare(c));
+    TRY(force_stage_core(c, nullptr, nullptr, nullptr, false));
+    TRY(dev_alloc(c, c->scratch64, sizeof(double) * N));
+    LAUNCH(launch_unpad(prec_fp64(c->prec), c->g, (const char *)c->npad.p + real_bytes(c) * s * c->g.P,
+                        (double *)c->scratch64.p, c->stream),
+           "density of the interior");
+    CK(cudaMemcpyAsync(out, c->scratch64.p, 8 * N, cudaMemcpyDeviceToHost, c->stream), "copy density");
     return check_error_word(c);
 }
 

@@ -40,6 +40,7 @@ template <typename S, typename T, int M, bool SOLID>
 __global__ void __launch_bounds__(collide_threads(M), collide_ctas(M, sizeof(T) == 4))
     k_collide_pair(Grid g, const S *__restrict__ src, S *__restrict__ dst, const uint32_t *__restrict__ mask,
                    const T *__restrict__ C, const T *__restrict__ F, StepParams sp, double *__restrict__ flux_buf) {
+    pdl_wait();
     const int a = M >= 2 ? (int)(threadIdx.x >> 7) : 0;         // species of this thread
     const int loc = M >= 2 ? (int)(threadIdx.x & 127) : 0;      // node within the CTA's 128
     const long long i = M >= 2 ? (long long)blockIdx.x * NPC + loc : (long long)blockIdx.x * NTP + threadIdx.x;
@@ -214,6 +215,7 @@ template <typename S, typename T, bool SOLID>
 __global__ void __launch_bounds__(NTP)
     k_density_pair(Grid g, const S *__restrict__ pop, const uint32_t *__restrict__ mask, double n00,
                    T *__restrict__ npad, int *err) {
+    pdl_wait();
     const long long i = (long long)blockIdx.x * NTP + threadIdx.x;
     const bool valid = i < g.N;
     const uint32_t m = valid ? (SOLID ? mask[i] : 0u) : 1u;
@@ -245,9 +247,10 @@ cudaError_t launch_collide(Prec p, const Grid &g, const void *src, void *dst, co
                            const void *C, const void *F, const StepParams &sp, double *flux_buf, cudaStream_t st) {
     const int per_cta = sp.M >= 2 ? NPC : NTP;
     const unsigned nb = (unsigned)((g.N + per_cta - 1) / per_cta);
-#define LBE_PAIR(MM, SOL)                                                                                       \
-    k_collide_pair<S, T, MM, SOL><<<nb, collide_threads(MM), 0, st>>>(g, (const S *)src, (S *)dst, mask,       \
-                                                                      (const T *)C, (const T *)F, sp, flux_buf)
+    cudaError_t e = cudaSuccess;
+#define LBE_PAIR(MM, SOL)                                                                                     \
+    e = launch_pdl(k_collide_pair<S, T, MM, SOL>, nb, collide_threads(MM), 0, st, g, (const S *)src, (S *)dst, \
+                   mask, (const T *)C, (const T *)F, sp, flux_buf)
 #define LBE_PAIR_M(MM)                          \
     if (solid) {                                \
         LBE_PAIR_DISPATCH(p, LBE_PAIR(MM, true)); \
@@ -263,20 +266,22 @@ cudaError_t launch_collide(Prec p, const Grid &g, const void *src, void *dst, co
     }
 #undef LBE_PAIR_M
 #undef LBE_PAIR
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_density_pair(Prec p, const Grid &g, const void *pop, const uint32_t *mask, bool solid,
                                 double n0, void *npad, int *err, cudaStream_t st) {
     const unsigned nb = (unsigned)((g.N + NTP - 1) / NTP);
-#define LBE_DPAIR(SOL) k_density_pair<S, T, SOL><<<nb, NTP, 0, st>>>(g, (const S *)pop, mask, n0, (T *)npad, err)
+    cudaError_t e = cudaSuccess;
+#define LBE_DPAIR(SOL) \
+    e = launch_pdl(k_density_pair<S, T, SOL>, nb, NTP, 0, st, g, (const S *)pop, mask, n0, (T *)npad, err)
     if (solid) {
         LBE_PAIR_DISPATCH(p, LBE_DPAIR(true));
     } else {
         LBE_PAIR_DISPATCH(p, LBE_DPAIR(false));
     }
 #undef LBE_DPAIR
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace lbe

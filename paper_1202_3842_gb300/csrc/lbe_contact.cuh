@@ -210,6 +210,7 @@ __global__ void __launch_bounds__(CT_THREADS)
         fence_mbar_init();
     }
     __syncthreads();
+    pdl_wait();
     auto issue = [&](int j) {
         const int slot = j % Tl::R;
         unsigned char *dst = base + slot * Tl::SLOT_BYTES;
@@ -469,10 +470,8 @@ cudaError_t launch_ct(const ContactLaunch &L, cudaStream_t st) {
     const int nbx = (g.nx + Tl::TX - 1) / Tl::TX, nby = (g.ny + Tl::TY - 1) / Tl::TY;
     cs.lz = march_planes((long long)nbx * nby, g.nz, RB, per_sm, 0.35, 2.4);
     dim3 grid(nbx, nby, (g.nz + cs.lz - 1) / cs.lz);
-    k_contact_tma<T, M, RB, MODE><<<grid, CT_THREADS, Tl::SMEM, st>>>(maps, g, cs, (T *)L.gab,
-                                                                 (T *)L.npad2, (T *)L.gnpad, (T *)L.xi, L.mask,
-                                                                 (T *)L.ln, L.top, L.err);
-    return cudaGetLastError();
+    return launch_pdl(k_contact_tma<T, M, RB, MODE>, grid, CT_THREADS, Tl::SMEM, st, maps, g, cs, (T *)L.gab,
+                      (T *)L.npad2, (T *)L.gnpad, (T *)L.xi, L.mask, (T *)L.ln, L.top, L.err);
 }
 
 template <typename T, int M, int MODE>

@@ -251,6 +251,11 @@ __device__ __forceinline__ void mbar_inval(uint64_t *bar) {
     asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
+// Programmatic dependent launch: a kernel of the step may be launched once the blocks of the one before it have
+// exited, before that one's completion is processed.  Each of these kernels calls pdl_wait before its first access
+// to global memory (it returns when the grids before it have completed and their writes are visible).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // 3-D tiled TMA load of one box into shared memory; completion is signalled on bar.
 __device__ __forceinline__ void tma_load_3d(void *smem_dst, const CUtensorMap *map, int x, int y, int z,
                                             uint64_t *bar) {

@@ -11,6 +11,24 @@
 
 namespace lbe {
 
+// Launch of a kernel of the step that begins with pdl_wait: its blocks may be placed before the kernel ahead of it on
+// the stream has finished, which hides the launch latency and the index arithmetic of the first blocks (a step of
+// a 24^3 lattice is five kernels of a few microseconds).
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Storage of the populations: [M][2 (f, g)][19][N] elements of the storage type.
 enum class Prec : int { F64 = 0, F32 = 1, BF16 = 2, F16 = 3 };
 
@@ -251,7 +269,7 @@ struct ViscPairs {
 // u~ [M][3][N] scratch; Feff [M][3][N] = F + C^visc / n
 cudaError_t launch_visc(Prec p, const Grid &g, const void *pop, const uint32_t *mask, const void *npad,
                         const void *gab, const void *F, const StepParams &sp, const ViscPairs &vp, const int *eoff,
-                        const double *ehat, void *ut, void *Feff, cudaStream_t st);
+                        const void *ehat /* FP64 or FP32 */, void *ut, void *Feff, cudaStream_t st);
 
 // K3 by fast Fourier transforms (lbe_spectral.cu).
 struct SpecPairs {

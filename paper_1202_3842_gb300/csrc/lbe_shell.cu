@@ -56,6 +56,7 @@ __device__ __forceinline__ long long to_fixed(double v, int top, int bits) {
 __global__ void __launch_bounds__(256) k_to_fixed(const double *__restrict__ npad, const double *__restrict__ gnpad,
                                                  long long P, int M, int bits,
                                                  const unsigned *__restrict__ top, long long *__restrict__ out) {
+    pdl_wait();
     const int f = blockIdx.y;  // n_b, then g_ab n_b
     const double *src = f < M ? npad + f * P : gnpad + (long long)(f - M) * P;
     const int e = fx_exponent(top[f]);
@@ -70,9 +71,8 @@ __global__ void __launch_bounds__(256) k_to_fixed(const double *__restrict__ npa
 cudaError_t launch_to_fixed(int Smax, const double *npad, const double *gnpad, long long P, int M,
                             const unsigned *top, long long *out, cudaStream_t st) {
     const long long nb = (P / 2 + 255) / 256;
-    k_to_fixed<<<dim3((unsigned)(nb < 2048 ? nb : 2048), M + M * M), 256, 0, st>>>(npad, gnpad, P, M,
-                                                                                     fx_bits(Smax), top, out);
-    return cudaGetLastError();
+    return launch_pdl(k_to_fixed, dim3((unsigned)(nb < 2048 ? nb : 2048), M + M * M), 256, 0, st, npad, gnpad, P, M,
+                      fx_bits(Smax), top, out);
 }
 
 bool shell_supported(bool fp64, int S) { return S >= 1 && S <= (fp64 ? 7 : 8); }

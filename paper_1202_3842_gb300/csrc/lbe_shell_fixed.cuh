@@ -357,6 +357,7 @@ __global__ void __launch_bounds__(64 * FX_TY, fixed_per_sm(SMAX))
         fence_mbar_init();
     }
     __syncthreads();
+    pdl_wait();
     if (nout <= 0) return;
     int it = 0;
     bool accumulate = false;
@@ -392,8 +393,7 @@ cudaError_t launch_shell_fixed_t(const ShellMarchMaps &maps, FixedArgs &A, cudaS
     A.lz = march_planes((long long)tx * ty * A.M, g.nz, SMAX, fixed_per_sm(SMAX), 1.0, 0.9, A.M > 1);
     A.nzb = (g.nz + A.lz - 1) / A.lz;
     march_order(A, (long long)tx * ty * A.M * A.nzb, fixed_per_sm(SMAX));
-    k_shell_fixed<SMAX><<<dim3(tx, ty, A.M * A.nzb), 64 * FX_TY, smem, st>>>(maps, A);
-    return cudaGetLastError();
+    return launch_pdl(k_shell_fixed<SMAX>, dim3(tx, ty, A.M * A.nzb), 64 * FX_TY, smem, st, maps, A);
 }
 
 }  // namespace lbe

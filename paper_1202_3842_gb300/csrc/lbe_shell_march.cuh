@@ -290,6 +290,7 @@ __global__ void __launch_bounds__(32 * SM_TY, shell_march_per_sm(SMAX))
         fence_mbar_init();
     }
     __syncthreads();
+    pdl_wait();
     if (nout <= 0) return;
     int it = 0;
     bool accumulate = false;
@@ -326,8 +327,7 @@ cudaError_t launch_shell_march_t(const ShellMarchMaps &maps, ShellMarchArgs &A, 
     A.lz = march_planes((long long)tx * ty * A.M, g.nz, SMAX, per_sm, 1.0, 0.9, A.M > 1);
     A.nzb = (g.nz + A.lz - 1) / A.lz;
     march_order(A, (long long)tx * ty * A.M * A.nzb, per_sm);
-    k_shell_march<SMAX><<<dim3(tx, ty, A.M * A.nzb), 32 * SM_TY, smem, st>>>(maps, A);
-    return cudaGetLastError();
+    return launch_pdl(k_shell_march<SMAX>, dim3(tx, ty, A.M * A.nzb), 32 * SM_TY, smem, st, maps, A);
 }
 
 }  // namespace lbe

@@ -12,9 +12,9 @@
 // which the collide and the moment getters take in place of F.
 //
 // k_tilde_velocity pulls the g populations of every species; k_visc_force
-// gathers the shell of every ordered pair from global memory (one thread per
-// node; neighbours wrapped on periodic axes, skipped beyond closed axes and on
-// solid nodes, where n_b = 0).  This is a plain gather, not a tiled stencil:
+// gathers the shell of every ordered pair from global memory (neighbours
+// wrapped on periodic axes, skipped beyond closed axes and on solid nodes,
+// where n_b = 0).  This is a plain gather, not a tiled stencil:
 // the term is an option, about four times the mean-field stencil's work.
 #include <utility>
 
@@ -60,17 +60,25 @@ __global__ void __launch_bounds__(VNT) k_tilde_velocity(Grid g, const S *__restr
     }
 }
 
+// A block takes 32 consecutive nodes; each of its eight warps gathers every eighth point of the shells for all of
+// them (a warp's loads stay runs of neighbouring nodes), and the warps' sums meet in shared memory.  One thread per
+// node walked up to 762 points alone, on 54 blocks for a 24^3 lattice, and converted three unit-vector components
+// per point from double on GB300's slow FP64 pipe; the table now has the arithmetic's type.
+constexpr int VW = VNT / 32;
+
 template <typename T>
 __global__ void __launch_bounds__(VNT) k_visc_force(Grid g, const uint32_t *__restrict__ mask,
                                                    const T *__restrict__ npad, const T *__restrict__ gab,
                                                    const T *__restrict__ ut, const T *__restrict__ F, ViscPairs vp,
-                                                   const int *__restrict__ eoff, const double *__restrict__ ehat,
+                                                   const int *__restrict__ eoff, const T *__restrict__ ehat,
                                                    T *__restrict__ Feff) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= g.N) return;
-    int x, y, z;
-    node_xyz(g, i, x, y, z);
-    const bool fluid = !(mask[i] & 1u);
+    __shared__ T part[VW][3][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long i = (long long)blockIdx.x * 32 + lane;
+    const bool valid = i < g.N;
+    int x = 0, y = 0, z = 0;
+    if (valid) node_xyz(g, i, x, y, z);
+    const bool fluid = valid && !(mask[i] & 1u);
     for (int a = 0; a < vp.M; ++a) {
         T V[3] = {0, 0, 0};
         const T na = fluid ? npad[(long long)a * g.P + pidx(g, x, y, z)] : (T)0;
@@ -80,17 +88,18 @@ __global__ void __launch_bounds__(VNT) k_visc_force(Grid g, const uint32_t *__re
                 const int b = vp.b[q];
                 const T *gq = gab + (long long)(a * vp.M + b) * g.N;
                 const T *ub = ut + (long long)b * 3 * g.N;
+                const T *nb = npad + (long long)b * g.P;
                 const T gr = gq[i];
                 const T u0[3] = {ub[i], ub[g.N + i], ub[2 * (long long)g.N + i]};
                 T sum[3] = {0, 0, 0};
-                for (int k = vp.first[q]; k < vp.first[q] + vp.count[q]; ++k) {
+                for (int k = vp.first[q] + warp; k < vp.first[q] + vp.count[q]; k += VW) {
                     int X = x + eoff[3 * k], Y = y + eoff[3 * k + 1], Z = z + eoff[3 * k + 2];
                     if (!wrap(X, g.nx, g.per[0]) || !wrap(Y, g.ny, g.per[1]) || !wrap(Z, g.nz, g.per[2])) continue;
                     const long long s = (long long)X + (long long)g.nx * ((long long)Y + (long long)g.ny * Z);
                     if (mask[s] & 1u) continue;
-                    const T e0 = (T)ehat[3 * k], e1 = (T)ehat[3 * k + 1], e2 = (T)ehat[3 * k + 2];
+                    const T e0 = ehat[3 * k], e1 = ehat[3 * k + 1], e2 = ehat[3 * k + 2];
                     const T edu = e0 * (ub[s] - u0[0]) + e1 * (ub[g.N + s] - u0[1]) + e2 * (ub[2 * (long long)g.N + s] - u0[2]);
-                    const T w = (T)0.5 * (gr + gq[s]) * npad[(long long)b * g.P + pidx(g, X, Y, Z)] * edu;
+                    const T w = (T)0.5 * (gr + gq[s]) * nb[pidx(g, X, Y, Z)] * edu;
                     sum[0] += e0 * w;
                     sum[1] += e1 * w;
                     sum[2] += e2 * w;
@@ -99,10 +108,17 @@ __global__ void __launch_bounds__(VNT) k_visc_force(Grid g, const uint32_t *__re
                 for (int c = 0; c < 3; ++c) V[c] += pre * sum[c];
             }
         }
-        for (int c = 0; c < 3; ++c) {
-            const long long k = ((long long)a * 3 + c) * g.N + i;
-            Feff[k] = na > (T)0 ? F[k] + V[c] : F[k];  // V holds C^visc / n_a
+#pragma unroll
+        for (int c = 0; c < 3; ++c) part[warp][c][lane] = V[c];
+        __syncthreads();
+        if (warp < 3 && valid) {  // warp c finishes component c
+            T v = part[0][warp][lane];
+#pragma unroll
+            for (int w = 1; w < VW; ++w) v += part[w][warp][lane];
+            const long long k = ((long long)a * 3 + warp) * g.N + i;
+            Feff[k] = na > (T)0 ? F[k] + v : F[k];  // v holds C^visc / n_a
         }
+        __syncthreads();
     }
 }
 
@@ -122,7 +138,7 @@ static cudaError_t tilde_m(const Grid &g, const void *pop, const uint32_t *mask,
 
 cudaError_t launch_visc(Prec p, const Grid &g, const void *pop, const uint32_t *mask, const void *npad,
                         const void *gab, const void *F, const StepParams &sp, const ViscPairs &vp, const int *eoff,
-                        const double *ehat, void *ut, void *Feff, cudaStream_t st) {
+                        const void *ehat, void *ut, void *Feff, cudaStream_t st) {
     cudaError_t e = cudaSuccess;
     switch (p) {
         case Prec::F64: e = tilde_m<double, double>(g, pop, mask, npad, sp, ut, st); break;
@@ -131,14 +147,14 @@ cudaError_t launch_visc(Prec p, const Grid &g, const void *pop, const uint32_t *
         case Prec::F16: e = tilde_m<__half, float>(g, pop, mask, npad, sp, ut, st); break;
     }
     if (e != cudaSuccess) return e;
-    const unsigned nb = (unsigned)((g.N + VNT - 1) / VNT);
+    const unsigned nb = (unsigned)((g.N + 31) / 32);
     if (p == Prec::F64)
         k_visc_force<double><<<nb, VNT, 0, st>>>(g, mask, (const double *)npad, (const double *)gab,
-                                                 (const double *)ut, (const double *)F, vp, eoff, ehat,
+                                                 (const double *)ut, (const double *)F, vp, eoff, (const double *)ehat,
                                                  (double *)Feff);
     else
         k_visc_force<float><<<nb, VNT, 0, st>>>(g, mask, (const float *)npad, (const float *)gab, (const float *)ut,
-                                                (const float *)F, vp, eoff, ehat, (float *)Feff);
+                                                (const float *)F, vp, eoff, (const float *)ehat, (float *)Feff);
     return cudaGetLastError();
 }
 
