@@ -1,20 +1,25 @@
-// K4 transposed for one or two species with species-parallel lanes (the
-// arithmetic is that of k_adj_collide + k_adj_write in lbe_adjoint.cu).
+// K4 transposed for one or two species (the arithmetic of k_adj_collide + k_adj_write in lbe_adjoint.cu, opposite
+// populations together).
 //
-// Two species: lanes 0-15 of a warp take species 0 and lanes 16-31 species 1
-// of the same 16 consecutive nodes (one species: one thread per node).  Each
-// thread
-//   pass A  pulls its own species' populations and forms its moments; n and J
-//           of the partner species (lane ^ 16) give the barycentric u;
-//   pass B  push-gathers the adjoint of its post-collision populations (kept in
-//           registers) and transposes the collision; the adjoint of u is the
-//           sum over both species, again by one exchange with the partner;
-//   pass C  transposes the moment recovery, adds lambda_F, writes lambda_C and
-//           the adjoint of its pre-collision populations.
-// Cross-species sums are formed in species order (0 then 1), as in the
-// one-thread-per-node kernel.
+// Two species: the layout of the forward collision (lbe_collide_pair.cu), warps 0 - 3 of a 256-thread CTA with species
+// 0 and warps 4 - 7 with species 1 of the same 128 nodes (one species: one thread per node).  Each thread
+//   pass A  pulls its own species' populations and forms its moments; n and J of the partner species, through
+//           shared memory, give the barycentric u;
+//   pass B  push-gathers the adjoint of its post-collision populations (kept in registers) and transposes the
+//           collision; the adjoint of u is the sum over both species, again by one exchange with the partner;
+//   pass C  transposes the moment recovery, adds lambda_F, writes lambda_C and the adjoint of its pre-collision
+//           populations.
+// Cross-species sums are formed in species order (0 then 1), as in the one-thread-per-node kernel.
+// A warp none of whose nodes has a blocked link pulls and gathers without the bounce-back selects, as the forward
+// kernels do.  In pass B the two populations of an opposite pair share their dot products and enter as the sum E and
+// the difference D of their adjoints.
+// Bounds: latency of the pulls and gathers (38 loads each pass); three CTAs per SM in FP32 hide more of it than two
+// (gradient of 20 steps of the 256x64x64 channel, FP32: 30.7 ms with a second pull of the populations instead of
+// registers, 30.5 with registers and two CTAs, 29.0 with three).
+#include <type_traits>
 #include <utility>
 
+#include "lbe_collide.cuh"
 #include "lbe_device.cuh"
 #include "lbe_launch.h"
 #include "lbe_node.cuh"
@@ -24,22 +29,34 @@ namespace lbe {
 constexpr int ACP = 256;  // threads per CTA: 128 nodes (two species) or 256 (one)
 
 // adjoint of the post-collision population p (streaming transposed), density adjoint added for f
-template <typename T, int P>
+template <typename T, int P, bool SEL>
 __device__ __forceinline__ T gather_post_pair(const T *__restrict__ lY, const T *__restrict__ ln, long long N,
                                               long long i, const NbrOff &o, uint32_t m) {
-    if (m & (1u << opp(P))) {
-        const T v = lY[(long long)opp(P) * N + i];
-        return ln ? v + ln[i] : v;
+    if constexpr (SEL) {
+        if (m & (1u << opp(P))) {
+            const T v = lY[(long long)opp(P) * N + i];
+            return ln ? v + ln[i] : v;
+        }
     }
     const long long j = i + src_off<opp(P)>(o);  // r + c_P
     const T v = lY[(long long)P * N + j];
     return ln ? v + ln[j] : v;
 }
 
-template <typename T, int M>
-__device__ __forceinline__ T partner(T v) {
-    if constexpr (M == 2) return __shfl_xor_sync(0xffffffffu, v, 16);
-    return (T)0;
+// Values of the partner species at the same node, through shared memory; the two warps over the same 32 nodes wait
+// for each other at named barrier 1 + w.  Every thread takes part.
+template <typename T, int M, int K>
+__device__ __forceinline__ void partners(T (*xch)[K][128], int a, int loc, const T (&v)[K], T (&p)[K]) {
+    if constexpr (M == 2) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) xch[a][k][loc] = v[k];
+        asm volatile("bar.sync %0, 64;" ::"r"(1 + (loc >> 5)) : "memory");
+#pragma unroll
+        for (int k = 0; k < K; ++k) p[k] = xch[1 - a][k][loc];
+    } else {
+#pragma unroll
+        for (int k = 0; k < K; ++k) p[k] = (T)0;
+    }
 }
 
 template <typename S, typename T, int M>
@@ -49,15 +66,16 @@ __global__ void __launch_bounds__(ACP, sizeof(T) == 4 ? 3 : 1)
                        const T *__restrict__ lYg_in, const T *__restrict__ lnd_in, T *__restrict__ lYf_out,
                        T *__restrict__ lYg_out, T *__restrict__ lC, T *__restrict__ lF) {
     static_assert(M == 1 || M == 2, "one or two species");
-    const int lane = threadIdx.x & 31;
-    const int a = M == 2 ? lane >> 4 : 0;
-    const long long i = M == 2 ? (long long)blockIdx.x * (ACP / 2) + (threadIdx.x >> 5) * 16 + (lane & 15)
-                               : (long long)blockIdx.x * ACP + threadIdx.x;
+    __shared__ T xa[M][4][128], xb[M][3][128];
+    const int a = M == 2 ? (int)(threadIdx.x >> 7) : 0;
+    const int loc = M == 2 ? (int)(threadIdx.x & 127) : 0;
+    const long long i = M == 2 ? (long long)blockIdx.x * (ACP / 2) + loc : (long long)blockIdx.x * ACP + threadIdx.x;
     const bool valid = i < g.N;
     int x = 0, y = 0, z = 0;
     if (valid) node_xyz(g, i, x, y, z);
     const uint32_t m = valid ? mask[i] : 1u;
     const bool fluid = !(m & 1u);
+    const bool plain = __all_sync(0xffffffffu, (m >> 1) == 0u);
     const double n0d = a == 0 ? ap.sp[0].n0 : ap.sp[1].n0;
     const T om = (T)(a == 0 ? ap.sp[0].omega_eff : ap.sp[1].omega_eff);
     const T inv = (T)(a == 0 ? ap.sp[0].inv : ap.sp[1].inv);
@@ -67,107 +85,112 @@ __global__ void __launch_bounds__(ACP, sizeof(T) == 4 ? 3 : 1)
     // ---- pass A: forward moments of this species
     T n = 0, inv_n = 0, J[3] = {0, 0, 0}, ua[3] = {0, 0, 0}, Cv[3] = {0, 0, 0}, Fv[3] = {0, 0, 0};
     T nF[3] = {0, 0, 0};
+    T lf[Q], lg[Q];
     if (fluid) {
         const T n0 = (T)n0d;
         const S *fb = post + pop_off(a, 0, 0, g.N);
         const S *gb = post + pop_off(a, 1, 0, g.N);
-        T Jt[3] = {0, 0, 0};
-        [&]<int... P>(std::integer_sequence<int, P...>) {
-            (
-                [&] {
-                    const T fv = pull<S, T, P, true>(fb, g.N, i, o, m, n0);
-                    const T gv = pull<S, T, P, true>(gb, g.N, i, o, m, n0);
-                    n += fv;
-                    Jt[0] += (T)cx(P) * gv;
-                    Jt[1] += (T)cy(P) * gv;
-                    Jt[2] += (T)cz(P) * gv;
-                }(),
-                ...);
-        }(std::make_integer_sequence<int, Q>{});
-        inv_n = n > (T)0 ? (T)1 / n : (T)0;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             Cv[c] = C[((long long)a * 3 + c) * g.N + i];
             Fv[c] = F[((long long)a * 3 + c) * g.N + i];
+        }
+        T Jt[3] = {0, 0, 0};
+        auto moments = [&](auto Sel) {
+            constexpr bool SEL = decltype(Sel)::value;
+            T f[Q], gq[Q];
+            [&]<int... P>(std::integer_sequence<int, P...>) {
+                ((f[P] = pull<S, T, P, SEL>(fb, g.N, i, o, m, n0)), ...);
+                ((gq[P] = pull<S, T, P, SEL>(gb, g.N, i, o, m, n0)), ...);
+            }(std::make_integer_sequence<int, Q>{});
+            n = zeroth_moment<false>(f);
+            ordered_momentum(gq, Jt);
+        };
+        if (plain)
+            moments(std::false_type{});
+        else
+            moments(std::true_type{});
+        inv_n = n > (T)0 ? (T)1 / n : (T)0;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
             nF[c] = n * Fv[c];
             J[c] = ap.consistent ? Jt[c] + (T)0.5 * nF[c] : Jt[c] + (T)0.5 * (Cv[c] + nF[c]);
             ua[c] = J[c] * inv_n;
         }
+        // the gather's loads are issued before the exchange
+        const T *lYf = lYf_in + (long long)a * Q * g.N;
+        const T *lYg = lYg_in + (long long)a * Q * g.N;
+        const T *lnd = lnd_in + (long long)a * g.N;
+        auto gather = [&](auto Sel) {
+            constexpr bool SEL = decltype(Sel)::value;
+            [&]<int... P>(std::integer_sequence<int, P...>) {
+                ((lf[P] = gather_post_pair<T, P, SEL>(lYf, lnd, g.N, i, o, m)), ...);
+                ((lg[P] = gather_post_pair<T, P, SEL>(lYg, nullptr, g.N, i, o, m)), ...);
+            }(std::make_integer_sequence<int, Q>{});
+        };
+        if (plain)
+            gather(std::false_type{});
+        else
+            gather(std::true_type{});
     }
-    const T np = partner<T, M>(n);
-    T Jp[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) Jp[c] = partner<T, M>(J[c]);
-    const T ntot = a == 0 ? n + np : np + n;
+    const T va[4] = {n, J[0], J[1], J[2]};
+    T pa[4];
+    partners<T, M, 4>(xa, a, loc, va, pa);
+    const T ntot = a == 0 ? n + pa[0] : pa[0] + n;
     const T inv_tot = ntot > (T)0 ? (T)1 / ntot : (T)0;
     T u[3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) u[c] = (a == 0 ? J[c] + Jp[c] : Jp[c] + J[c]) * inv_tot;
+    for (int c = 0; c < 3; ++c) u[c] = (a == 0 ? J[c] + pa[c + 1] : pa[c + 1] + J[c]) * inv_tot;
     const T uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
 
     // ---- pass B: collision transposed
-    // FP32: the gathered adjoint populations wait for the last pass in shared memory (39 KB per CTA),
-    // which leaves the registers for three CTAs per SM; FP64 keeps them in registers
-    constexpr bool SMEM = sizeof(T) == 4;
-    __shared__ T sl[SMEM ? 2 : 1][SMEM ? Q : 1][SMEM ? ACP : 1];
-    T lfk[SMEM ? 1 : Q], lgk[SMEM ? 1 : Q];
-    const int tid = threadIdx.x;
     T lu[3] = {0, 0, 0}, lua[3] = {0, 0, 0}, lCs[3] = {0, 0, 0}, lnFs[3] = {0, 0, 0}, lns = 0, lPis = 0;
     if (fluid) {
         const T uau = ua[0] * u[0] + ua[1] * u[1] + ua[2] * u[2];
         T X[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) X[c] = Cv[c] + nF[c];
-        T lA = 0, lB = 0, lsf0 = 0, lnv = 0;
+        constexpr T w0 = (T)wq(0);
+        T lA = w0 * om * lf[0], lB = w0 * om * lg[0], lsf0 = w0 * inv * (lf[0] + lg[0]), lnv = 0;
         T lX[3] = {0, 0, 0}, lnFv[3] = {0, 0, 0}, lCv[3] = {0, 0, 0}, luav[3] = {0, 0, 0}, lua_u[3] = {0, 0, 0};
-        const T *lYf = lYf_in + (long long)a * Q * g.N;
-        const T *lYg = lYg_in + (long long)a * Q * g.N;
-        const T *lnd = lnd_in + (long long)a * g.N;
-        [&]<int... P>(std::integer_sequence<int, P...>) {
+        [&]<int... KP>(std::integer_sequence<int, KP...>) {
             (
                 [&] {
+                    constexpr int P = 2 * KP + 1;  // and its opposite, P + 1
                     constexpr T w = (T)wq(P);
-                    const T lfs = gather_post_pair<T, P>(lYf, lnd, g.N, i, o, m);
-                    const T lgs = gather_post_pair<T, P>(lYg, nullptr, g.N, i, o, m);
-                    if constexpr (SMEM) {
-                        sl[0][P][tid] = lfs;
-                        sl[1][P][tid] = lgs;
-                    } else {
-                        lfk[P] = lfs;
-                        lgk[P] = lgs;
-                    }
-                    const T cua = cdot<T, P>(ua);
-                    const T cu = cdot<T, P>(u);
-                    const T cX = cdot<T, P>(X);
-                    const T cY = cdot<T, P>(nF);
-                    const T cC = cdot<T, P>(Cv);
-                    const T lSf = inv * lfs, lSg = inv * lgs;
-                    const T lt1 = w * om * (lfs + lgs);
-                    lA += w * om * lfs;
-                    lB += w * om * lgs;
-                    lsf0 += w * (lSf + lSg);
-                    const T lcX = w * lSf * ((T)3 + (T)9 * cua);
-                    const T lcY = w * lSg * ((T)3 + (T)9 * cua);
-                    const T lcC = (T)18 * w * lSg * cua;
-                    const T lcua = (T)9 * w * lSf * cX + w * lSg * ((T)18 * cC + (T)9 * cY) +
-                                   lt1 * ((T)3 * n + (T)9 * n * cu);
-                    const T lcu = (T)9 * n * (cua - cu) * lt1;
-                    lnv += lt1 * ((T)3 * cua + (T)4.5 * ((T)2 * cua * cu - cu * cu));
-                    if constexpr (cx(P) != 0) {
-                        luav[0] += (T)cx(P) * lcua; lua_u[0] += (T)cx(P) * lcu; lX[0] += (T)cx(P) * lcX;
-                        lnFv[0] += (T)cx(P) * lcY; lCv[0] += (T)cx(P) * lcC;
-                    }
-                    if constexpr (cy(P) != 0) {
-                        luav[1] += (T)cy(P) * lcua; lua_u[1] += (T)cy(P) * lcu; lX[1] += (T)cy(P) * lcX;
-                        lnFv[1] += (T)cy(P) * lcY; lCv[1] += (T)cy(P) * lcC;
-                    }
-                    if constexpr (cz(P) != 0) {
-                        luav[2] += (T)cz(P) * lcua; lua_u[2] += (T)cz(P) * lcu; lX[2] += (T)cz(P) * lcX;
-                        lnFv[2] += (T)cz(P) * lcY; lCv[2] += (T)cz(P) * lcC;
-                    }
+                    const T wom = w * om, winv = w * inv;
+                    const T Ef = lf[P] + lf[P + 1], Df = lf[P] - lf[P + 1];
+                    const T Eg = lg[P] + lg[P + 1], Dg = lg[P] - lg[P + 1];
+                    const T H = wom * (Ef + Eg), K = wom * (Df + Dg);
+                    const T s = link_dot<T, P>(ua), t = link_dot<T, P>(u);
+                    const T cX = link_dot<T, P>(X), cY = link_dot<T, P>(nF), cC = link_dot<T, P>(Cv);
+                    lA += wom * Ef;
+                    lB += wom * Eg;
+                    lsf0 += winv * (Ef + Eg);
+                    const T lcX = winv * ((T)3 * Df + (T)9 * s * Ef);
+                    const T lcY = winv * ((T)3 * Dg + (T)9 * s * Eg);
+                    const T lcC = (T)18 * winv * s * Eg;
+                    const T lcua = winv * ((T)9 * cX * Ef + ((T)18 * cC + (T)9 * cY) * Eg) +
+                                   n * ((T)3 * K + (T)9 * t * H);
+                    const T lcu = (T)9 * n * (s - t) * H;
+                    lnv += (T)3 * s * K + (T)4.5 * ((T)2 * s - t) * t * H;
+                    auto add = [&](auto Cc) {
+                        constexpr int c = decltype(Cc)::value;
+                        constexpr int cc = c == 0 ? cx(P) : (c == 1 ? cy(P) : cz(P));
+                        if constexpr (cc != 0) {
+                            luav[c] += (T)cc * lcua;
+                            lua_u[c] += (T)cc * lcu;
+                            lX[c] += (T)cc * lcX;
+                            lnFv[c] += (T)cc * lcY;
+                            lCv[c] += (T)cc * lcC;
+                        }
+                    };
+                    add(std::integral_constant<int, 0>{});
+                    add(std::integral_constant<int, 1>{});
+                    add(std::integral_constant<int, 2>{});
                 }(),
                 ...);
-        }(std::make_integer_sequence<int, Q>{});
+        }(std::make_integer_sequence<int, 9>{});
         // sf0 = -3 X.u^a ; X = C + nF ; A = n - iso ; B = Pi - iso ; iso = 1.5 n (2 u^a.u - u.u)
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -192,10 +215,11 @@ __global__ void __launch_bounds__(ACP, sizeof(T) == 4 ? 3 : 1)
         lPis = lB;
     }
     // ---- u = sum J / sum n: the adjoint of u summed over both species (species order)
-    T lJtot[3] = {0, 0, 0}, lntot = 0;
+    T lJtot[3] = {0, 0, 0}, lntot = 0, pb[3];
+    partners<T, M, 3>(xb, a, loc, lu, pb);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const T lp = partner<T, M>(lu[c]);
+        const T lp = pb[c];
         const T lut = a == 0 ? lu[c] + lp : lp + lu[c];
         if (ntot > (T)0) {
             lJtot[c] = lut * inv_tot;
@@ -245,10 +269,11 @@ __global__ void __launch_bounds__(ACP, sizeof(T) == 4 ? 3 : 1)
     [&]<int... P>(std::integer_sequence<int, P...>) {
         (
             [&] {
-                const T lfs = SMEM ? sl[0][P][tid] : lfk[SMEM ? 0 : P];
-                const T lgs = SMEM ? sl[1][P][tid] : lgk[SMEM ? 0 : P];
-                of[(long long)P * g.N] = om1 * lfs + ln;
-                og[(long long)P * g.N] = om1 * lgs + lPit + cdot<T, P>(lJ);
+                of[(long long)P * g.N] = om1 * lf[P] + ln;
+                if constexpr (P == 0)
+                    og[0] = om1 * lg[0] + lPit;
+                else
+                    og[(long long)P * g.N] = om1 * lg[P] + lPit + link_dot<T, P>(lJ);
             }(),
             ...);
     }(std::make_integer_sequence<int, Q>{});
