@@ -20,7 +20,8 @@ namespace lbe {
 
 constexpr int NTA = 128;
 
-template <typename S, typename T, int M, bool SOLID>
+// SD: one distribution, g is a copy of f and nothing of g is pulled or computed (48^3, FP64: 71 -> 53 us).
+template <typename S, typename T, int M, bool SOLID, bool SD>
 __global__ void __launch_bounds__(NTA)
     k_collide_ablation(Grid g, const S *__restrict__ src, S *__restrict__ dst, const uint32_t *__restrict__ mask,
                        const T *__restrict__ C, const T *__restrict__ F, StepParams sp,
@@ -39,7 +40,6 @@ __global__ void __launch_bounds__(NTA)
             for (int a = 0; a < M; ++a) flux_buf[(long long)a * psize + plane_index(g, sp.flux_axis, x, y, z)] = 0.0;
         return;
     }
-    const bool sd = sp.scheme == LBE_SD_TR || sp.scheme == LBE_SD_EU;
     const bool eu = sp.scheme == LBE_SD_EU || sp.scheme == LBE_DD_EU;
     const NbrOff o = nbr_offsets(g, x, y, z);
     T fv[M][Q], gv[M][Q] = {};
@@ -52,17 +52,16 @@ __global__ void __launch_bounds__(NTA)
         const S *gb = src + pop_off(a, 1, 0, g.N);
         [&]<int... P>(std::integer_sequence<int, P...>) {
             ((fv[a][P] = pull<S, T, P, SOLID>(fb, g.N, i, o, m, n0)), ...);
-            if (!sd) ((gv[a][P] = pull<S, T, P, SOLID>(gb, g.N, i, o, m, n0)), ...);
+            if constexpr (!SD) ((gv[a][P] = pull<S, T, P, SOLID>(gb, g.N, i, o, m, n0)), ...);
         }(std::make_integer_sequence<int, Q>{});
         const T na = zeroth_moment<false>(fv[a]);
         T Pit, Jt[3];
+        const T *mom = SD ? fv[a] : gv[a];
         if constexpr (sizeof(T) == 4) {
-            Pit = zeroth_moment<false>(sd ? fv[a] : gv[a]);
-            ordered_momentum(sd ? fv[a] : gv[a], Jt);
-        } else if (sd) {
-            pair_moments<false>(fv[a], Pit, Jt);
+            Pit = zeroth_moment<false>(mom);
+            ordered_momentum(mom, Jt);
         } else {
-            pair_moments<false>(gv[a], Pit, Jt);
+            pair_moments<false>(mom, Pit, Jt);
         }
         const T inv_n = na > (T)0 ? (T)1 / na : (T)0;
 #pragma unroll
@@ -74,7 +73,7 @@ __global__ void __launch_bounds__(NTA)
             Jtot[c] += J[a][c];
         }
         n[a] = na;
-        Pi[a] = sd ? na : Pit;
+        Pi[a] = SD ? na : Pit;
         ntot += na;
     }
     const T inv_tot = ntot > (T)0 ? (T)1 / ntot : (T)0;
@@ -96,7 +95,7 @@ __global__ void __launch_bounds__(NTA)
             constexpr int P = decltype(Pc)::value;
             constexpr T w = (T)wq(P), iw = (T)(1.0 / wq(P));
             Store<S, T>::store(fo + (long long)P * g.N, fv[a][P], w * n0a, iw * in0);
-            Store<S, T>::store(go + (long long)P * g.N, sd ? fv[a][P] : gv[a][P], w * n0a, iw * in0);
+            Store<S, T>::store(go + (long long)P * g.N, SD ? fv[a][P] : gv[a][P], w * n0a, iw * in0);
         };
         if constexpr (sizeof(T) == 4) {  // FP32 on f itself: as it has always rounded (see k_collide_pair)
             collide_whole(n[a], Pi[a], ua[a], u, Cv[a], nF[a], (T)sp.sp[a].omega_eff, (T)sp.sp[a].inv, fv[a], gv[a]);
@@ -106,13 +105,13 @@ __global__ void __launch_bounds__(NTA)
         }
         Collision<T> col;
         col.set(n[a], n[a], Pi[a], ua[a], u, Cv[a], nF[a], (T)sp.sp[a].omega_eff, (T)sp.sp[a].inv, (T)0);
-        col.rest(fv[a][0], gv[a][0]);
+        col.template rest<!SD>(fv[a][0], gv[a][0]);
         put(std::integral_constant<int, 0>{});
         [&]<int... K>(std::integer_sequence<int, K...>) {
             (
                 [&] {
                     constexpr int P = 2 * K + 1;
-                    col.template pair<P>(fv[a][P], fv[a][P + 1], gv[a][P], gv[a][P + 1]);
+                    col.template pair<P, !SD>(fv[a][P], fv[a][P + 1], gv[a][P], gv[a][P + 1]);
                     put(std::integral_constant<int, P>{});
                     put(std::integral_constant<int, P + 1>{});
                 }(),
@@ -176,20 +175,29 @@ bool ablation_supported(Prec p, int M) { return (p == Prec::F64 || p == Prec::F3
 cudaError_t launch_collide_ablation(Prec p, const Grid &g, const void *src, void *dst, const uint32_t *mask,
                                     bool solid, const void *C, const void *F, const StepParams &sp,
                                     double *flux_buf, cudaStream_t st) {
-    const unsigned nb = (unsigned)((g.N + NTA - 1) / NTA);
+    const int threads = node_threads(g.N, NTA);
+    const unsigned nb = (unsigned)((g.N + threads - 1) / threads);
+    const bool sd = sp.scheme == LBE_SD_TR || sp.scheme == LBE_SD_EU;
     cudaError_t e = cudaSuccess;
-#define LBE_ABL(MM, SOL)                                                                                    \
-    e = launch_pdl(k_collide_ablation<S, T, MM, SOL>, nb, NTA, 0, st, g, (const S *)src, (S *)dst, mask,   \
-                   (const T *)C, (const T *)F, sp, flux_buf)
+#define LBE_ABL(MM, SOL, SD)                                                                                 \
+    e = launch_pdl(k_collide_ablation<S, T, MM, SOL, SD>, nb, threads, 0, st, g, (const S *)src, (S *)dst,   \
+                   mask, (const T *)C, (const T *)F, sp, flux_buf)
+#define LBE_ABL_M(MM)                                                      \
+    if (sd) {                                                              \
+        if (solid) LBE_ABL(MM, true, true); else LBE_ABL(MM, false, true);   \
+    } else {                                                               \
+        if (solid) LBE_ABL(MM, true, false); else LBE_ABL(MM, false, false); \
+    }
     LBE_ABL_DISPATCH(p, {
         if (sp.M == 1) {
-            if (solid) LBE_ABL(1, true); else LBE_ABL(1, false);
+            LBE_ABL_M(1)
         } else if (sp.M == 2) {
-            if (solid) LBE_ABL(2, true); else LBE_ABL(2, false);
+            LBE_ABL_M(2)
         } else {
             return cudaErrorInvalidValue;
         }
     });
+#undef LBE_ABL_M
 #undef LBE_ABL
     return e;
 }

@@ -9,8 +9,8 @@
 // odd in c:
 //   even_f = kf + k2 (2s - t) t + (c.X9) s,  even_g = kg + k2 (2s - t) t + (c.G9) s,  s = c.u^a, t = c.u,
 //   odd_f  = c.Of,  odd_g = c.Og,
-// so a pair shares its dot products, and the constants carry om, inv and the edge links' weight 1/36 (or 1/n0, below).  That is 9 to
-// 10 operations per population where each population's own f_eq, S_f and update took 36.
+// so a pair shares its dot products, and the constants carry om, inv and the edge links' weight 1/36 (or 1/n0,
+// below).  That is 14 flops per population where each population's own f_eq, S_f and update took 36.
 #pragma once
 #include <utility>
 
@@ -115,29 +115,26 @@ struct Collision {
         omc = (T)1 - om;
     }
 
-    // the rest populations
+    // the rest populations (G false: f only)
+    template <bool G = true>
     __device__ __forceinline__ void rest(T &f, T &g) const {
         f = UNIT ? omc * f + kf : omc * f + (T)12 * kf;
-        g = UNIT ? omc * g + kg : omc * g + (T)12 * kg;
+        if constexpr (G) g = UNIT ? omc * g + kg : omc * g + (T)12 * kg;
     }
     // the populations of the pair P, P + 1 = opposite of P
-    template <int P>
+    template <int P, bool G = true>
     __device__ __forceinline__ void pair(T &fp, T &fm, T &gp, T &gm) const {
         static_assert(P % 2 == 1 && P < Q, "first population of a pair");
         const T s = link_dot<T, P>(ua), t = link_dot<T, P>(u);
         const T h = ((T)2 * s - t) * t;
         const T ef = link_dot<T, P>(X9) * s + (k2 * h + kf), of = link_dot<T, P>(Of);
-        const T eg = link_dot<T, P>(G9) * s + (k2 * h + kg), og = link_dot<T, P>(Og);
-        if constexpr (!UNIT && P < 7) {  // axis links: weight 1/18
-            fp = omc * fp + (T)2 * (ef + of);
-            fm = omc * fm + (T)2 * (ef - of);
-            gp = omc * gp + (T)2 * (eg + og);
-            gm = omc * gm + (T)2 * (eg - og);
-        } else {
-            fp = omc * fp + (ef + of);
-            fm = omc * fm + (ef - of);
-            gp = omc * gp + (eg + og);
-            gm = omc * gm + (eg - og);
+        constexpr T wp = (T)(!UNIT && P < 7 ? 2 : 1);  // axis links: weight 1/18
+        fp = omc * fp + wp * (ef + of);
+        fm = omc * fm + wp * (ef - of);
+        if constexpr (G) {
+            const T eg = link_dot<T, P>(G9) * s + (k2 * h + kg), og = link_dot<T, P>(Og);
+            gp = omc * gp + wp * (eg + og);
+            gm = omc * gm + wp * (eg - og);
         }
     }
 };

@@ -1,9 +1,9 @@
 // K4: fused moments + DD-TR collision + pull streaming (Sec. "Hard sphere fluid mixture in a potential well"; the
 // collision itself is in lbe_collide.cuh), and K1 for one species.
 //
-// Two species or more: a CTA takes 128 consecutive nodes, warps 4a .. 4a + 3 species a of the same nodes, 32
-// consecutive nodes per warp.  Each thread pulls only its own species' 38 populations and keeps them in registers,
-// computes that species' moments, and gets the other species' n and J through shared memory to form the
+// Two species or more: a CTA takes 128 consecutive nodes (fewer on small lattices), warps 4a .. 4a + 3 species a of
+// the same nodes, 32 consecutive nodes per warp.  Each thread pulls only its own species' 38 populations, keeps them
+// in registers, computes that species' moments, and gets the other species' n and J through shared memory to form the
 // barycentric velocity u = sum J / sum n.  A warp's load of one population is one 128-byte run of one species'
 // array (FP32), as in the one-species kernel.  Compared with one thread per node holding every species, the live
 // state per thread shrinks to one species', so more warps share an SM, and nothing is pulled twice.
@@ -39,11 +39,12 @@ __host__ __device__ constexpr int collide_ctas(int M, bool f32) {
 template <typename S, typename T, int M, bool SOLID>
 __global__ void __launch_bounds__(collide_threads(M), collide_ctas(M, sizeof(T) == 4))
     k_collide_pair(Grid g, const S *__restrict__ src, S *__restrict__ dst, const uint32_t *__restrict__ mask,
-                   const T *__restrict__ C, const T *__restrict__ F, StepParams sp, double *__restrict__ flux_buf) {
+                   const T *__restrict__ C, const T *__restrict__ F, StepParams sp, double *__restrict__ flux_buf,
+                   int lg) {
     pdl_wait();
-    const int a = M >= 2 ? (int)(threadIdx.x >> 7) : 0;         // species of this thread
-    const int loc = M >= 2 ? (int)(threadIdx.x & 127) : 0;      // node within the CTA's 128
-    const long long i = M >= 2 ? (long long)blockIdx.x * NPC + loc : (long long)blockIdx.x * NTP + threadIdx.x;
+    const int a = M >= 2 ? (int)(threadIdx.x >> lg) : 0;           // species of this thread
+    const int loc = M >= 2 ? (int)(threadIdx.x & ((1 << lg) - 1)) : 0;  // node within the CTA's 2^lg (128 at most)
+    const long long i = M >= 2 ? ((long long)blockIdx.x << lg) + loc : (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const bool valid = i < g.N;
     int x = 0, y = 0, z = 0;
     if (valid) node_xyz(g, i, x, y, z);
@@ -216,7 +217,7 @@ __global__ void __launch_bounds__(NTP)
     k_density_pair(Grid g, const S *__restrict__ pop, const uint32_t *__restrict__ mask, double n00,
                    T *__restrict__ npad, int *err) {
     pdl_wait();
-    const long long i = (long long)blockIdx.x * NTP + threadIdx.x;
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const bool valid = i < g.N;
     const uint32_t m = valid ? (SOLID ? mask[i] : 0u) : 1u;
     // a warp none of whose nodes has a blocked link pulls without the bounce-back selects
@@ -245,12 +246,16 @@ __global__ void __launch_bounds__(NTP)
 
 cudaError_t launch_collide(Prec p, const Grid &g, const void *src, void *dst, const uint32_t *mask, bool solid,
                            const void *C, const void *F, const StepParams &sp, double *flux_buf, cudaStream_t st) {
-    const int per_cta = sp.M >= 2 ? NPC : NTP;
+    // nodes per CTA: 256 (one species) or 128, fewer on small lattices (24^3, FP64: 30.4 -> 18.3 us)
+    int lg = 7;
+    while (sp.M >= 2 && lg > 5 && ((g.N + (1 << lg) - 1) >> lg) < 2 * 152) --lg;
+    const int per_cta = sp.M >= 2 ? 1 << lg : node_threads(g.N, NTP);
+    const int threads = sp.M >= 2 ? sp.M << lg : per_cta;
     const unsigned nb = (unsigned)((g.N + per_cta - 1) / per_cta);
     cudaError_t e = cudaSuccess;
-#define LBE_PAIR(MM, SOL)                                                                                     \
-    e = launch_pdl(k_collide_pair<S, T, MM, SOL>, nb, collide_threads(MM), 0, st, g, (const S *)src, (S *)dst, \
-                   mask, (const T *)C, (const T *)F, sp, flux_buf)
+#define LBE_PAIR(MM, SOL)                                                                                       \
+    e = launch_pdl(k_collide_pair<S, T, MM, SOL>, nb, threads, 0, st, g, (const S *)src, (S *)dst, mask,        \
+                   (const T *)C, (const T *)F, sp, flux_buf, lg)
 #define LBE_PAIR_M(MM)                          \
     if (solid) {                                \
         LBE_PAIR_DISPATCH(p, LBE_PAIR(MM, true)); \
@@ -271,10 +276,11 @@ cudaError_t launch_collide(Prec p, const Grid &g, const void *src, void *dst, co
 
 cudaError_t launch_density_pair(Prec p, const Grid &g, const void *pop, const uint32_t *mask, bool solid,
                                 double n0, void *npad, int *err, cudaStream_t st) {
-    const unsigned nb = (unsigned)((g.N + NTP - 1) / NTP);
+    const int threads = node_threads(g.N, NTP);
+    const unsigned nb = (unsigned)((g.N + threads - 1) / threads);
     cudaError_t e = cudaSuccess;
 #define LBE_DPAIR(SOL) \
-    e = launch_pdl(k_density_pair<S, T, SOL>, nb, NTP, 0, st, g, (const S *)pop, mask, n0, (T *)npad, err)
+    e = launch_pdl(k_density_pair<S, T, SOL>, nb, threads, 0, st, g, (const S *)pop, mask, n0, (T *)npad, err)
     if (solid) {
         LBE_PAIR_DISPATCH(p, LBE_DPAIR(true));
     } else {

@@ -283,7 +283,8 @@ cudaError_t launch_density(Prec p, const Grid &g, const void *pop, const uint32_
     // one species: one thread per node at 32-42 registers (lbe_collide_pair.cu); measured faster than this
     // kernel for one species (256^3 well 0.42 -> 0.31 ms) and slower for two (0.29 -> 0.31 ms)
     if (M == 1) return launch_density_pair(p, g, pop, mask, solid, n0[0], npad, err, st);
-    unsigned nb = (unsigned)((g.N + NT - 1) / NT);
+    const int threads = node_threads(g.N, NT);
+    const unsigned nb = (unsigned)((g.N + threads - 1) / threads);
     N0Vec n0v;
     N0VecF n0f;
     for (int a = 0; a < MAXS; ++a) {
@@ -292,7 +293,7 @@ cudaError_t launch_density(Prec p, const Grid &g, const void *pop, const uint32_
     }
     cudaError_t e = cudaSuccess;
 #define LBE_K1(SOL, MC) \
-    LBE_DISPATCH_PREC(p, (e = launch_pdl(k_density<S, T, SOL, MC>, nb, NT, 0, st, g, (const S *)pop, mask, n0v, n0f, (T *)npad, err)))
+    LBE_DISPATCH_PREC(p, (e = launch_pdl(k_density<S, T, SOL, MC>, nb, threads, 0, st, g, (const S *)pop, mask, n0v, n0f, (T *)npad, err)))
 #define LBE_K1_M(MC)       \
     if (solid) {           \
         LBE_K1(true, MC);  \
@@ -362,12 +363,13 @@ __global__ void __launch_bounds__(NT) k_moments(Grid g, const S *__restrict__ sr
 template <typename S, typename T>
 static cudaError_t moments_m(int M, const Grid &g, const void *pop, const uint32_t *mask, const void *C, const void *F,
                              const StepParams &sp, double *n, double *J, cudaStream_t st) {
-    unsigned nb = (unsigned)((g.N + NT - 1) / NT);
+    const int nt = node_threads(g.N, NT);
+    const unsigned nb = (unsigned)((g.N + nt - 1) / nt);
     switch (M) {
-        case 1: k_moments<S, T, 1><<<nb, NT, 0, st>>>(g, (const S *)pop, mask, (const T *)C, (const T *)F, sp, n, J); break;
-        case 2: k_moments<S, T, 2><<<nb, NT, 0, st>>>(g, (const S *)pop, mask, (const T *)C, (const T *)F, sp, n, J); break;
-        case 3: k_moments<S, T, 3><<<nb, NT, 0, st>>>(g, (const S *)pop, mask, (const T *)C, (const T *)F, sp, n, J); break;
-        case 4: k_moments<S, T, 4><<<nb, NT, 0, st>>>(g, (const S *)pop, mask, (const T *)C, (const T *)F, sp, n, J); break;
+        case 1: k_moments<S, T, 1><<<nb, nt, 0, st>>>(g, (const S *)pop, mask, (const T *)C, (const T *)F, sp, n, J); break;
+        case 2: k_moments<S, T, 2><<<nb, nt, 0, st>>>(g, (const S *)pop, mask, (const T *)C, (const T *)F, sp, n, J); break;
+        case 3: k_moments<S, T, 3><<<nb, nt, 0, st>>>(g, (const S *)pop, mask, (const T *)C, (const T *)F, sp, n, J); break;
+        case 4: k_moments<S, T, 4><<<nb, nt, 0, st>>>(g, (const S *)pop, mask, (const T *)C, (const T *)F, sp, n, J); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

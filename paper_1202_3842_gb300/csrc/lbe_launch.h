@@ -29,6 +29,15 @@ inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
+// Threads per block of a kernel with one thread per node (or one group per node): `most` on large lattices, halved down
+// to 64 while the blocks are too few to reach every multiprocessor twice (a 24^3 lattice is 54 blocks of 256 for
+// 152 multiprocessors).
+inline int node_threads(long long nodes, int most) {
+    int t = most;
+    while (t > 64 && (nodes + t - 1) / t < 2 * 152) t /= 2;
+    return t;
+}
+
 // Storage of the populations: [M][2 (f, g)][19][N] elements of the storage type.
 enum class Prec : int { F64 = 0, F32 = 1, BF16 = 2, F16 = 3 };
 
