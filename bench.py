@@ -44,11 +44,11 @@ SMS_NOMINAL = 152          # GB300; the run uses the device's own multiprocessor
 FP32_LANES_PER_SM = 128
 SMEM_BYTES_PER_CLK_PER_SM = 128  # 32 banks x 4 bytes
 QPOP = 19
-# Algorithmic flops of the fused collide (K4) per node and species, counted from its source
-# (csrc/lbe_collide_pair.cu): moments 63 (n, Pi~: 18 adds each; J~: 9 adds per component), recovery,
-# velocities and the isotropic terms 57, and per population 36 (t1 7, f_eq and g_eq 4, S_f 6, S_g 9,
-# the two TR updates 10) plus one add per dot product c_p . v on the 12 edge links (5 dot products).
-K4_FLOPS_PER_NODE_SPECIES = 63 + 57 + 19 * 36 + 12 * 5
+# Flops of the fused collide (K4) per node and species, counted from its source (csrc/lbe_collide_pair.cu,
+# lbe_collide.cuh; a multiply-add is two): moments 57 (n, Pi~: 18 adds each; J~: 9 differences and 12 adds), recovery
+# and velocities 31, the constants of the collision 64, the rest populations 6, and per opposite pair of f and g 27
+# on the 3 axes and 29 on the 6 edges (each population by itself took 36 and more: 864 in all).
+K4_FLOPS_PER_NODE_SPECIES = 57 + 31 + 64 + 6 + 3 * 27 + 6 * 29
 STAGE_STEPS = 20  # steps of the instrumented pass that gives the per-stage times
 
 WORKLOAD_TEXT = {
