@@ -12,8 +12,10 @@
 // so a pair shares its dot products, and the constants carry om, inv and the edge links' weight 1/36 (or 1/n0,
 // below).  That is 14 flops per population where each population's own f_eq, S_f and update took 36.
 #pragma once
+#include <type_traits>
 #include <utility>
 
+#include "lbe_block_sum.cuh"
 #include "lbe_device.cuh"
 
 namespace lbe {
@@ -45,6 +47,8 @@ __device__ __forceinline__ T zeroth_moment(const T *f) {
 #pragma unroll
         for (int p = 8; p < Q; ++p) e += f[p];
         return (T)12 * f[0] + ((T)2 * a + e);
+    } else if constexpr (std::is_same_v<T, double>) {
+        return block_sum(f);
     } else {
         T n = f[0];
 #pragma unroll
@@ -55,6 +59,10 @@ __device__ __forceinline__ T zeroth_moment(const T *f) {
 // Sum and first moment (UNIT: of 36 w_p s_p) from the sums and differences of opposite pairs.
 template <bool UNIT, typename T>
 __device__ __forceinline__ void pair_moments(const T *g, T &Pi, T J[3]) {
+    if constexpr (std::is_same_v<T, double>) {
+        block_moments(g, Pi, J);
+        return;
+    }
     // pairs: x, y, z; (1,1,0), (1,-1,0), (1,0,1), (1,0,-1), (0,1,1), (0,1,-1)
     T d[9], s = UNIT ? g[1] + g[2] : g[0];
 #pragma unroll

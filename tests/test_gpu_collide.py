@@ -71,3 +71,26 @@ def test_auto_takes_the_stencil_on_large_lattices(prec):
     auto, spectral = setup_gpu(w, arr, prec), setup_gpu(w, arr, prec, shell="spectral")
     assert auto.shell_method() == "direct" and spectral.shell_method() == "spectral"
     assert rel_err(auto.force(0), spectral.force(0)) <= (1e-12 if prec == "fp64" else 1e-5)
+
+
+@pytest.mark.parametrize("scale", [1e-312, 1e-290, 1e-20, 1.0, 1e200])
+def test_fp64_moments_of_any_magnitude(scale):
+    """Density and momentum of FP64 populations over 30 decades at one node, at both ends of the exponent range, and
+    with zeros: a sum of 19 terms is within 18 round-offs of the terms' magnitudes (a subnormal term's last bit)."""
+    shape, N = (9, 4, 3), 108
+    rng = np.random.default_rng(11)
+    arr = dict(solid=np.zeros(N, np.uint8), V=np.zeros((1, N)), phi=np.zeros(N), amp=np.zeros(N), n=np.ones((1, N)))
+    w = dict(shape=shape, periodic=(1, 1, 1), sigma=[0.0], tau=[1.0], body=[(0.0, 0.0, 0.0)])
+    g = setup_gpu(w, arr, "fp64")
+    f = scale * rng.random((19, N)) * 10.0 ** rng.uniform(-20, 3, (19, N)) * (rng.random((19, N)) < 0.8)
+    gq = scale * rng.standard_normal((19, N)) * 10.0 ** rng.uniform(-20, 3, (19, N))
+    g.set_populations(0, f, gq)
+    ulp = 18 * 2.0 ** -53
+    assert (np.abs(g.density(0) - f.sum(0)) <= 2 * ulp * f.sum(0) + 19 * 5e-324).all()
+    pairs = [(1, 0, 0), (0, 1, 0), (0, 0, 1), (1, 1, 0), (1, -1, 0), (1, 0, 1), (1, 0, -1), (0, 1, 1), (0, 1, -1)]
+    J = np.asarray(g.momentum(0)).reshape(3, N)
+    for c in range(3):
+        ref = sum(p[c] * (gq[1 + 2 * k] - gq[2 + 2 * k]) for k, p in enumerate(pairs))
+        assert (np.abs(J[c] - ref) <= 2 * ulp * np.abs(gq).sum(0) + 19 * 5e-324).all()
+    back_f, back_g = g.populations(0)
+    assert np.array_equal(back_f, f) and np.array_equal(back_g, gq)
