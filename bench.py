@@ -44,11 +44,11 @@ SMS_NOMINAL = 152          # GB300; the run uses the device's own multiprocessor
 FP32_LANES_PER_SM = 128
 SMEM_BYTES_PER_CLK_PER_SM = 128  # 32 banks x 4 bytes
 QPOP = 19
-# Flops of the fused collide (K4) per node and species, counted from its source (csrc/lbe_collide_pair.cu,
-# lbe_collide.cuh; a multiply-add is two): moments 57 (n, Pi~: 18 adds each; J~: 9 differences and 12 adds), recovery
-# and velocities 31, the constants of the collision 64, the rest populations 6, and per opposite pair of f and g 27
-# on the 3 axes and 29 on the 6 edges (each population by itself took 36 and more: 864 in all).
-K4_FLOPS_PER_NODE_SPECIES = 57 + 31 + 64 + 6 + 3 * 27 + 6 * 29
+# FP64 flops of the fused collide (K4) per node and species, counted from its source (csrc/lbe_collide_pair.cu,
+# Collision64 in lbe_collide.cuh; a multiply-add is two): recovery and velocities 31, the constants of f 81, their
+# change to g's 18, and of f and g together the rest populations 6, the axis pairs 42 and the edge pairs 108.  The
+# 57 additions of the moments run on the integer pipe (lbe_block_sum.cuh).  (Each population by itself took 864.)
+K4_FLOPS_PER_NODE_SPECIES = 31 + 81 + 18 + 6 + 42 + 108
 STAGE_STEPS = 20  # steps of the instrumented pass that gives the per-stage times
 
 WORKLOAD_TEXT = {

@@ -20,7 +20,8 @@ namespace lbe {
 
 constexpr int NTA = 128;
 
-// SD: one distribution, g is a copy of f and nothing of g is pulled or computed (48^3, FP64: 71 -> 53 us).
+// SD: one distribution, g is a copy of f and nothing of g is pulled or computed (48^3, FP64: 71 -> 53 us, 38 with the FP64
+// forms of lbe_block_sum.cuh and Collision64).
 template <typename S, typename T, int M, bool SOLID, bool SD>
 __global__ void __launch_bounds__(NTA)
     k_collide_ablation(Grid g, const S *__restrict__ src, S *__restrict__ dst, const uint32_t *__restrict__ mask,
@@ -99,24 +100,17 @@ __global__ void __launch_bounds__(NTA)
         };
         if constexpr (sizeof(T) == 4) {  // FP32 on f itself: as it has always rounded (see k_collide_pair)
             collide_whole(n[a], Pi[a], ua[a], u, Cv[a], nF[a], (T)sp.sp[a].omega_eff, (T)sp.sp[a].inv, fv[a], gv[a]);
-            [&]<int... P>(std::integer_sequence<int, P...>) { (put(std::integral_constant<int, P>{}), ...); }
-            (std::make_integer_sequence<int, Q>{});
-            continue;
+        } else {
+            Collision64 col;
+            col.set(n[a], Pi[a], ua[a], u, Cv[a], nF[a], sp.sp[a].omega_eff, sp.sp[a].inv);
+            col.all(fv[a]);
+            if constexpr (!SD) {
+                col.next();
+                col.all(gv[a]);
+            }
         }
-        Collision<T> col;
-        col.set(n[a], n[a], Pi[a], ua[a], u, Cv[a], nF[a], (T)sp.sp[a].omega_eff, (T)sp.sp[a].inv, (T)0);
-        col.template rest<!SD>(fv[a][0], gv[a][0]);
-        put(std::integral_constant<int, 0>{});
-        [&]<int... K>(std::integer_sequence<int, K...>) {
-            (
-                [&] {
-                    constexpr int P = 2 * K + 1;
-                    col.template pair<P, !SD>(fv[a][P], fv[a][P + 1], gv[a][P], gv[a][P + 1]);
-                    put(std::integral_constant<int, P>{});
-                    put(std::integral_constant<int, P + 1>{});
-                }(),
-                ...);
-        }(std::make_integer_sequence<int, 9>{});
+        [&]<int... P>(std::integer_sequence<int, P...>) { (put(std::integral_constant<int, P>{}), ...); }
+        (std::make_integer_sequence<int, Q>{});
     }
 }
 

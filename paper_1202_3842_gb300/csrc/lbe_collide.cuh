@@ -123,27 +123,106 @@ struct Collision {
         omc = (T)1 - om;
     }
 
-    // the rest populations (G false: f only)
-    template <bool G = true>
+    // the rest populations
     __device__ __forceinline__ void rest(T &f, T &g) const {
         f = UNIT ? omc * f + kf : omc * f + (T)12 * kf;
-        if constexpr (G) g = UNIT ? omc * g + kg : omc * g + (T)12 * kg;
+        g = UNIT ? omc * g + kg : omc * g + (T)12 * kg;
     }
     // the populations of the pair P, P + 1 = opposite of P
-    template <int P, bool G = true>
+    template <int P>
     __device__ __forceinline__ void pair(T &fp, T &fm, T &gp, T &gm) const {
         static_assert(P % 2 == 1 && P < Q, "first population of a pair");
         const T s = link_dot<T, P>(ua), t = link_dot<T, P>(u);
         const T h = ((T)2 * s - t) * t;
         const T ef = link_dot<T, P>(X9) * s + (k2 * h + kf), of = link_dot<T, P>(Of);
+        const T eg = link_dot<T, P>(G9) * s + (k2 * h + kg), og = link_dot<T, P>(Og);
         constexpr T wp = (T)(!UNIT && P < 7 ? 2 : 1);  // axis links: weight 1/18
         fp = omc * fp + wp * (ef + of);
         fm = omc * fm + wp * (ef - of);
-        if constexpr (G) {
-            const T eg = link_dot<T, P>(G9) * s + (k2 * h + kg), og = link_dot<T, P>(Og);
-            gp = omc * gp + wp * (eg + og);
-            gm = omc * gm + wp * (eg - og);
+        gp = omc * gp + wp * (eg + og);
+        gm = omc * gm + wp * (eg - og);
+    }
+};
+
+// The same for FP64 populations, where every operation counts (GB300 has two FP64 lanes per SM): the even part of a pair is a
+// quadratic form in c,
+//   k + c.Q.c,  Q_ij = k2 (2u^a - u)_i u_j + X9_i u^a_j  (symmetric part),
+// so an axis takes k + Q_ii, an edge k + Q_ii + Q_jj +- 2 Q_ij, and with iso and s0 the constants are
+//   kf = w om n - tr(Q) / 3,  kg = w om Pi - tr(Q) / 3.
+// One distribution at a time, g's form from f's (G9 - X9 = 3 b C): about 200 FP64 instructions per node and species
+// besides the moments instead of 243.  K4 of the 256x64x64 channel 989 -> 811 us, of the 48^3 well with SD-TR 47 -> 38.
+struct Collision64 {
+    double k, omc, q[3], r[3], o[3];  // r: 2 Q_xy, 2 Q_xz, 2 Q_yz; o: odd part
+    double kg, og[3], d[3], ua[3];    // what next() needs
+
+    __device__ __forceinline__ void set(double n, double Pi, const double *ua_, const double *u, const double *C,
+                                        const double *nF, double om, double inv) {
+        const double wom = 1.0 / 36.0 * om, a = 3.0 * wom * n, b = 3.0 / 36.0 * inv, k2 = 4.5 * wom * n;
+        double v[3], X9[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const double m = a * ua_[c], bX = b * (C[c] + nF[c]);
+            ua[c] = ua_[c];
+            v[c] = k2 * (2.0 * ua[c] - u[c]);
+            X9[c] = 3.0 * bX;
+            d[c] = 3.0 * b * C[c];
+            o[c] = m + bX;
+            og[c] = m + b * nF[c];
+            q[c] = v[c] * u[c] + X9[c] * ua[c];
         }
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+            const int i = e == 2 ? 1 : 0, j = e == 0 ? 1 : 2;
+            r[e] = v[i] * u[j] + v[j] * u[i] + X9[i] * ua[j] + X9[j] * ua[i];
+        }
+        const double tr = q[0] + q[1] + q[2];
+        k = wom * n - 1.0 / 3.0 * tr;
+        kg = wom * Pi - 1.0 / 3.0 * tr;
+        omc = 1.0 - om;
+    }
+    // from f to g
+    __device__ __forceinline__ void next() {
+        k = kg;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            o[c] = og[c];
+            q[c] += d[c] * ua[c];
+        }
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+            const int i = e == 2 ? 1 : 0, j = e == 0 ? 1 : 2;
+            r[e] += d[i] * ua[j] + d[j] * ua[i];
+        }
+    }
+    // 2 v by its exponent (zero, subnormal and non-finite values as they are)
+    static __device__ __forceinline__ double twice(double v) {
+        const int h = __double2hiint(v);
+        const unsigned e = (unsigned)h >> 20 & 0x7ffu;
+        return __hiloint2double(e - 1u < 0x7fdu ? h + 0x100000 : h, __double2loint(v));
+    }
+    __device__ __forceinline__ void rest(double &f) const { f = omc * f + 12.0 * k; }
+    template <int P>
+    __device__ __forceinline__ void pair(double &fp, double &fm) const {
+        if constexpr (P < 7) {  // axis links: weight 1/18
+            constexpr int i = (P - 1) / 2;
+            const double e = k + q[i];
+            fp = omc * fp + twice(e + o[i]);
+            fm = omc * fm + twice(e - o[i]);
+        } else {
+            constexpr int i = cx(P) ? 0 : 1, j = cz(P) ? 2 : 1;
+            constexpr bool same = (i == 0 ? cx(P) : cy(P)) * (j == 1 ? cy(P) : cz(P)) > 0;
+            static_assert((i == 0 ? cx(P) : cy(P)) == 1, "first population of a pair");
+            const double t = (k + q[i]) + q[j], e = same ? t + r[i + j - 1] : t - r[i + j - 1];
+            const double h = same ? o[i] + o[j] : o[i] - o[j];
+            fp = omc * fp + (e + h);
+            fm = omc * fm + (e - h);
+        }
+    }
+    __device__ __forceinline__ void all(double *v) const {
+        rest(v[0]);
+        [&]<int... K>(std::integer_sequence<int, K...>) {
+            (pair<2 * K + 1>(v[2 * K + 1], v[2 * K + 2]), ...);
+        }(std::make_integer_sequence<int, 9>{});
     }
 };
 

@@ -10,8 +10,8 @@
 // One species: one thread per node, 32 consecutive nodes per warp, u = J/n.
 //
 // Bounds: HBM with FP32 storage (783 us for the 512x128x128 channel's 5.1 GB, 96% of the measured copy bandwidth; 886
-// before the collision's pairs shared their parts); the FP64 pipe in FP64 (256x64x64 channel 2.55 -> 1.20 ms; 330
-// operations per node and species, 79% of that pipe's cycles before the second CTA); issue with 16-bit storage
+// before the collision's pairs shared their parts); the FP64 pipe in FP64 (256x64x64 channel 2.55 -> 0.81 ms: 1.20
+// with shared pairs and two CTAs, 0.99 with the moments on the integer pipe, the rest by Collision64); issue with 16-bit storage
 // (channel 887 -> 701 us, half of them integer instructions for addresses and conversions).  Three species: the
 // kernel with one thread per node for all of them pulled every population twice (90x75x66 166 -> 86 us).
 #include <math.h>
@@ -191,6 +191,28 @@ __global__ void __launch_bounds__(collide_threads(M), collide_ctas(M, sizeof(T) 
         [&]<int... P>(std::integer_sequence<int, P...>) {
             (put(std::integral_constant<int, P>{}, f[P] - (T)wq(P) * n0s, gq[P] - (T)wq(P) * n0s), ...);
         }(std::make_integer_sequence<int, Q>{});
+        return;
+    }
+    if constexpr (sizeof(T) == 8) {
+        Collision64 col;
+        col.set(n, Pi, ua, u, Cv, nF, sc.omega_eff, sc.inv);
+        auto half = [&](S *out, T(&v)[Q]) {
+            col.rest(v[0]);
+            Store<S, T>::store_unit(out, v[0]);
+            [&]<int... K>(std::integer_sequence<int, K...>) {
+                (
+                    [&] {
+                        constexpr int P = 2 * K + 1;
+                        col.template pair<P>(v[P], v[P + 1]);
+                        Store<S, T>::store_unit(out + (long long)P * g.N, v[P]);
+                        Store<S, T>::store_unit(out + (long long)(P + 1) * g.N, v[P + 1]);
+                    }(),
+                    ...);
+            }(std::make_integer_sequence<int, 9>{});
+        };
+        half(fo, f);
+        col.next();
+        half(go, gq);
         return;
     }
     Collision<T, UNIT> col;

@@ -63,7 +63,8 @@ __global__ void __launch_bounds__(VNT) k_tilde_velocity(Grid g, const S *__restr
 // A block takes 32 consecutive nodes; each of its eight warps gathers every eighth point of the shells for all of
 // them (a warp's loads stay runs of neighbouring nodes), and the warps' sums meet in shared memory.  One thread per
 // node walked up to 762 points alone, on 54 blocks for a 24^3 lattice, and converted three unit-vector components
-// per point from double on GB300's slow FP64 pipe; the table now has the arithmetic's type.
+// per point from double on GB300's slow FP64 pipe; the table now has the arithmetic's type
+// (a step of the 24^3 well with this term, FP32: 104 -> 34 us).
 constexpr int VW = VNT / 32;
 
 template <typename T>
