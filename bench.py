@@ -199,12 +199,13 @@ def source_hash(files):
 
 KERNEL_SOURCES = {
     "collide": ["paper_1202_3842_gb300/csrc/lbe_collide_pair.cu", "paper_1202_3842_gb300/csrc/lbe_collide.cuh",
-                "paper_1202_3842_gb300/csrc/lbe_device.cuh",
+                "paper_1202_3842_gb300/csrc/lbe_block_sum.cuh", "paper_1202_3842_gb300/csrc/lbe_device.cuh",
                 "paper_1202_3842_gb300/csrc/lbe_node.cuh"],
     "shell": ["paper_1202_3842_gb300/csrc/lbe_shell.cu", "paper_1202_3842_gb300/csrc/lbe_shell.cuh",
               "paper_1202_3842_gb300/csrc/lbe_march.cuh", "paper_1202_3842_gb300/csrc/lbe_shell_march.cuh",
               "paper_1202_3842_gb300/csrc/lbe_shell_fixed.cuh", "paper_1202_3842_gb300/csrc/lbe_device.cuh"],
     "density": ["paper_1202_3842_gb300/csrc/lbe_kernels.cu", "paper_1202_3842_gb300/csrc/lbe_collide_pair.cu",
+                "paper_1202_3842_gb300/csrc/lbe_collide.cuh", "paper_1202_3842_gb300/csrc/lbe_block_sum.cuh",
                 "paper_1202_3842_gb300/csrc/lbe_device.cuh", "paper_1202_3842_gb300/csrc/lbe_node.cuh"],
     "contact": ["paper_1202_3842_gb300/csrc/lbe_contact.cu", "paper_1202_3842_gb300/csrc/lbe_contact.cuh",
                 "paper_1202_3842_gb300/csrc/lbe_march.cuh", "paper_1202_3842_gb300/csrc/lbe_device.cuh"],
