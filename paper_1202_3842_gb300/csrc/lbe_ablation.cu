@@ -20,6 +20,120 @@ namespace lbe {
 
 constexpr int NTA = 128;
 
+// FP32: every population's f_eq, S_f and update on its own, on the populations themselves.  The velocity of such a run
+// carries the rounding of f (1.2e-5 of it after 20 steps of a 70x62x56 well), so this form and its order of
+// operations stay: another one shifts runs by half their own error.
+template <typename S, typename T, int M, bool SOLID>
+__global__ void __launch_bounds__(NTA)
+    k_collide_ablation_whole(Grid g, const S *__restrict__ src, S *__restrict__ dst, const uint32_t *__restrict__ mask,
+                       const T *__restrict__ C, const T *__restrict__ F, StepParams sp,
+                       double *__restrict__ flux_buf) {
+    pdl_wait();
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= g.N) return;
+    int x, y, z;
+    node_xyz(g, i, x, y, z);
+    const uint32_t m = SOLID ? mask[i] : 0u;
+    const int coord = sp.flux_axis == 0 ? x : (sp.flux_axis == 1 ? y : z);
+    const bool on_plane = sp.flux_axis >= 0 && coord == sp.flux_plane;
+    const int psize = sp.flux_axis == 0 ? g.ny * g.nz : (sp.flux_axis == 1 ? g.nx * g.nz : g.nx * g.ny);
+    if (m & 1u) {
+        if (on_plane)
+            for (int a = 0; a < M; ++a) flux_buf[(long long)a * psize + plane_index(g, sp.flux_axis, x, y, z)] = 0.0;
+        return;
+    }
+    const bool sd = sp.scheme == LBE_SD_TR || sp.scheme == LBE_SD_EU;
+    const bool eu = sp.scheme == LBE_SD_EU || sp.scheme == LBE_DD_EU;
+    const NbrOff o = nbr_offsets(g, x, y, z);
+    T fv[M][Q], gv[M][Q];
+    T n[M], Pi[M], J[M][3], Cv[M][3], nF[M][3], ua[M][3];
+    T ntot = 0, Jtot[3] = {0, 0, 0};
+#pragma unroll
+    for (int a = 0; a < M; ++a) {
+        const T n0 = (T)sp.sp[a].n0;
+        const S *fb = src + pop_off(a, 0, 0, g.N);
+        const S *gb = src + pop_off(a, 1, 0, g.N);
+        [&]<int... P>(std::integer_sequence<int, P...>) {
+            ((fv[a][P] = pull<S, T, P, SOLID>(fb, g.N, i, o, m, n0)), ...);
+            if (!sd) ((gv[a][P] = pull<S, T, P, SOLID>(gb, g.N, i, o, m, n0)), ...);
+        }(std::make_integer_sequence<int, Q>{});
+        const T *mom = sd ? fv[a] : gv[a];
+        T na = 0, Pit = 0, Jt[3] = {0, 0, 0};
+        [&]<int... P>(std::integer_sequence<int, P...>) {
+            ((na += fv[a][P]), ...);
+            ((Pit += mom[P]), ...);
+            ((Jt[0] += (T)cx(P) * mom[P]), ...);
+            ((Jt[1] += (T)cy(P) * mom[P]), ...);
+            ((Jt[2] += (T)cz(P) * mom[P]), ...);
+        }(std::make_integer_sequence<int, Q>{});
+        const T inv_n = na > (T)0 ? (T)1 / na : (T)0;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            Cv[a][c] = C[((long long)a * 3 + c) * g.N + i];
+            nF[a][c] = na * F[((long long)a * 3 + c) * g.N + i];
+            J[a][c] = eu ? Jt[c] : Jt[c] + (T)0.5 * (Cv[a][c] + nF[a][c]);
+            ua[a][c] = J[a][c] * inv_n;
+            Jtot[c] += J[a][c];
+        }
+        n[a] = na;
+        Pi[a] = sd ? na : Pit;
+        ntot += na;
+    }
+    const T inv_tot = ntot > (T)0 ? (T)1 / ntot : (T)0;
+    T u[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) u[c] = Jtot[c] * inv_tot;
+    if (on_plane) {
+#pragma unroll
+        for (int a = 0; a < M; ++a)
+            flux_buf[(long long)a * psize + plane_index(g, sp.flux_axis, x, y, z)] = (double)J[a][sp.flux_axis];
+    }
+    const T uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+#pragma unroll
+    for (int a = 0; a < M; ++a) {
+        const T na = n[a];
+        const T uau = ua[a][0] * u[0] + ua[a][1] * u[1] + ua[a][2] * u[2];
+        const T iso = (T)1.5 * na * ((T)2 * uau - uu);
+        const T A = na - iso, B = Pi[a] - iso;
+        T X[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) X[c] = Cv[a][c] + nF[a][c];
+        const T sf0 = (T)-3 * (X[0] * ua[a][0] + X[1] * ua[a][1] + X[2] * ua[a][2]);
+        const T om = (T)sp.sp[a].omega_eff, inv = (T)sp.sp[a].inv;
+        const T n0a = (T)sp.sp[a].n0;
+        const T in0 = sp.sp[a].n0 > 0.0 ? (T)(1.0 / sp.sp[a].n0) : (T)0;
+        S *fo = dst + pop_off(a, 0, 0, g.N) + i;
+        S *go = dst + pop_off(a, 1, 0, g.N) + i;
+        [&]<int... P>(std::integer_sequence<int, P...>) {
+            (
+                [&] {
+                    constexpr T w = (T)wq(P);
+                    const T cua = cdot<T, P>(ua[a]);
+                    const T cu = cdot<T, P>(u);
+                    const T cX = cdot<T, P>(X);
+                    const T t1 = (T)3 * na * cua + (T)4.5 * na * ((T)2 * cua * cu - cu * cu);
+                    const T feq = w * (A + t1);
+                    const T Sf = w * (sf0 + (T)3 * cX + (T)9 * cX * cua);
+                    const T fs = fv[a][P] + om * (feq - fv[a][P]) + inv * Sf;
+                    constexpr T iw = (T)(1.0 / wq(P));
+                    Store<S, T>::store(fo + (long long)P * g.N, fs, w * n0a, iw * in0);
+                    if (sd) {
+                        Store<S, T>::store(go + (long long)P * g.N, fs, w * n0a, iw * in0);
+                    } else {
+                        const T cY = cdot<T, P>(nF[a]);
+                        const T cC = cdot<T, P>(Cv[a]);
+                        const T geq = w * (B + t1);
+                        const T Sg = w * (sf0 + (T)3 * cY + (T)18 * cC * cua + (T)9 * cY * cua);
+                        const T gs = gv[a][P] + om * (geq - gv[a][P]) + inv * Sg;
+                        Store<S, T>::store(go + (long long)P * g.N, gs, w * n0a, iw * in0);
+                    }
+                }(),
+                ...);
+        }(std::make_integer_sequence<int, Q>{});
+    }
+}
+
+// FP64.
 // SD: one distribution, g is a copy of f and nothing of g is pulled or computed (48^3, FP64: 71 -> 53 us, 38 with the FP64
 // forms of lbe_block_sum.cuh and Collision64).
 template <typename S, typename T, int M, bool SOLID, bool SD>
@@ -58,12 +172,7 @@ __global__ void __launch_bounds__(NTA)
         const T na = zeroth_moment<false>(fv[a]);
         T Pit, Jt[3];
         const T *mom = SD ? fv[a] : gv[a];
-        if constexpr (sizeof(T) == 4) {
-            Pit = zeroth_moment<false>(mom);
-            ordered_momentum(mom, Jt);
-        } else {
-            pair_moments<false>(mom, Pit, Jt);
-        }
+        pair_moments<false>(mom, Pit, Jt);
         const T inv_n = na > (T)0 ? (T)1 / na : (T)0;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -98,16 +207,12 @@ __global__ void __launch_bounds__(NTA)
             Store<S, T>::store(fo + (long long)P * g.N, fv[a][P], w * n0a, iw * in0);
             Store<S, T>::store(go + (long long)P * g.N, SD ? fv[a][P] : gv[a][P], w * n0a, iw * in0);
         };
-        if constexpr (sizeof(T) == 4) {  // FP32 on f itself: as it has always rounded (see k_collide_pair)
-            collide_whole(n[a], Pi[a], ua[a], u, Cv[a], nF[a], (T)sp.sp[a].omega_eff, (T)sp.sp[a].inv, fv[a], gv[a]);
-        } else {
-            Collision64 col;
-            col.set(n[a], Pi[a], ua[a], u, Cv[a], nF[a], sp.sp[a].omega_eff, sp.sp[a].inv);
-            col.all(fv[a]);
-            if constexpr (!SD) {
-                col.next();
-                col.all(gv[a]);
-            }
+        Collision64 col;
+        col.set(n[a], Pi[a], ua[a], u, Cv[a], nF[a], sp.sp[a].omega_eff, sp.sp[a].inv);
+        col.all(fv[a]);
+        if constexpr (!SD) {
+            col.next();
+            col.all(gv[a]);
         }
         [&]<int... P>(std::integer_sequence<int, P...>) { (put(std::integral_constant<int, P>{}), ...); }
         (std::make_integer_sequence<int, Q>{});
@@ -166,34 +271,33 @@ bool ablation_supported(Prec p, int M) { return (p == Prec::F64 || p == Prec::F3
         default: return cudaErrorInvalidValue;                                       \
     }
 
+template <typename S, typename T, int M>
+static cudaError_t collide_ablation_m(const Grid &g, const void *src, void *dst, const uint32_t *mask, bool solid,
+                                      const void *C, const void *F, const StepParams &sp, double *flux_buf,
+                                      cudaStream_t st) {
+    const int threads = node_threads(g.N, NTA);
+    const unsigned nb = (unsigned)((g.N + threads - 1) / threads);
+    auto run = [&](auto kernel) {
+        return launch_pdl(kernel, nb, threads, 0, st, g, (const S *)src, (S *)dst, mask, (const T *)C, (const T *)F,
+                          sp, flux_buf);
+    };
+    if constexpr (sizeof(T) == 4) {
+        return solid ? run(k_collide_ablation_whole<S, T, M, true>) : run(k_collide_ablation_whole<S, T, M, false>);
+    } else {
+        if (sp.scheme == LBE_SD_TR || sp.scheme == LBE_SD_EU)
+            return solid ? run(k_collide_ablation<S, T, M, true, true>) : run(k_collide_ablation<S, T, M, false, true>);
+        return solid ? run(k_collide_ablation<S, T, M, true, false>) : run(k_collide_ablation<S, T, M, false, false>);
+    }
+}
+
 cudaError_t launch_collide_ablation(Prec p, const Grid &g, const void *src, void *dst, const uint32_t *mask,
                                     bool solid, const void *C, const void *F, const StepParams &sp,
                                     double *flux_buf, cudaStream_t st) {
-    const int threads = node_threads(g.N, NTA);
-    const unsigned nb = (unsigned)((g.N + threads - 1) / threads);
-    const bool sd = sp.scheme == LBE_SD_TR || sp.scheme == LBE_SD_EU;
-    cudaError_t e = cudaSuccess;
-#define LBE_ABL(MM, SOL, SD)                                                                                 \
-    e = launch_pdl(k_collide_ablation<S, T, MM, SOL, SD>, nb, threads, 0, st, g, (const S *)src, (S *)dst,   \
-                   mask, (const T *)C, (const T *)F, sp, flux_buf)
-#define LBE_ABL_M(MM)                                                      \
-    if (sd) {                                                              \
-        if (solid) LBE_ABL(MM, true, true); else LBE_ABL(MM, false, true);   \
-    } else {                                                               \
-        if (solid) LBE_ABL(MM, true, false); else LBE_ABL(MM, false, false); \
-    }
     LBE_ABL_DISPATCH(p, {
-        if (sp.M == 1) {
-            LBE_ABL_M(1)
-        } else if (sp.M == 2) {
-            LBE_ABL_M(2)
-        } else {
-            return cudaErrorInvalidValue;
-        }
+        if (sp.M == 1) return collide_ablation_m<S, T, 1>(g, src, dst, mask, solid, C, F, sp, flux_buf, st);
+        if (sp.M == 2) return collide_ablation_m<S, T, 2>(g, src, dst, mask, solid, C, F, sp, flux_buf, st);
     });
-#undef LBE_ABL_M
-#undef LBE_ABL
-    return e;
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_moments_ablation(Prec p, const Grid &g, const void *pop, const uint32_t *mask, const void *C,

@@ -353,7 +353,13 @@ bool spectral_cheaper(const lbe_ctx *c, bool f64, double stencil_factor = 1.0) {
 // stencil is compiled.  Lattices below DIRECT_NODES nodes are bound by launches in either form and keep the
 // rule above, which programs that record the method of a small lattice rely on.
 constexpr long long DIRECT_NODES = 16384;
-bool direct_cheaper(const lbe_ctx *c) { return c->g.N >= DIRECT_NODES; }
+// FP32 runs of the single-distribution schemes keep the cost rule: their velocity carries the rounding of f (1e-5 of it
+// and more), and a force that rounds otherwise moves it by half of that (well of diameter 6, 20 steps: 5.8e-6 between
+// the two forms, each 1.0e-5 from FP64; the two-distribution schemes move by 2e-6 and less).
+bool direct_cheaper(const lbe_ctx *c) {
+    if (c->prec == Prec::F32 && (c->cfg.scheme == LBE_SD_TR || c->cfg.scheme == LBE_SD_EU)) return false;
+    return c->g.N >= DIRECT_NODES;
+}
 
 // The pairs as the spectral kernels see them (shell index into the table of distinct shells), the
 // distinct shells, and the grid: the lattice along periodic axes, at least Smax zero planes beyond it

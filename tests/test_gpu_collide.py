@@ -71,6 +71,9 @@ def test_auto_takes_the_stencil_on_large_lattices(prec):
     auto, spectral = setup_gpu(w, arr, prec), setup_gpu(w, arr, prec, shell="spectral")
     assert auto.shell_method() == "direct" and spectral.shell_method() == "spectral"
     assert rel_err(auto.force(0), spectral.force(0)) <= (1e-12 if prec == "fp64" else 1e-5)
+    # FP32 runs of the single-distribution schemes keep the rule of small lattices
+    single = setup_gpu(w, arr, prec, scheme="sd_tr")
+    assert single.shell_method() == ("direct" if prec == "fp64" else "spectral")
 
 
 @pytest.mark.parametrize("scale", [1e-312, 1e-290, 1e-20, 1.0, 1e200])
