@@ -86,8 +86,9 @@ typedef enum { LBE_DD_TR = 0, LBE_SD_TR = 1, LBE_SD_EU = 2, LBE_DD_EU = 3 } lbe_
  *   LBE_SHELL_AUTO (default): spectral for diameters without a compiled
  *     stencil, direct for compiled diameters on lattices of 16384 nodes and
  *     more (measured on GB300); on smaller ones, and in FP32 runs of the
- *     single-distribution schemes, spectral where the mean shell of the pairs is above about 320 points (FP32) or 110 points (FP64),
- *     scaled by the padded grid over the lattice.
+ *     single-distribution schemes, spectral where the mean shell of the pairs
+ *     is above about 320 points (FP32) or 110 points (FP64), scaled by the
+ *     padded grid over the lattice.
  * Both give the sums of the definition up to rounding.  The discrete adjoint
  * (lbe_adjoint_flux_gradient) transposes the shell sums with the method this
  * call sets: the stencil (pair diameters with a compiled stencil), the
