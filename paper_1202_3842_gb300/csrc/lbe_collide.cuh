@@ -100,12 +100,17 @@ struct Collision {
     // (UNIT only)
     __device__ __forceinline__ void set(T n, T dn, T Pi, const T *ua_, const T *u_, const T *C, const T *nF, T om,
                                         T inv, T in0) {
-        const T w = UNIT ? in0 : (T)(1.0 / 36.0), wom = w * om, winv = w * inv;
+        constexpr T w36 = (T)(1.0 / 36.0), w36_lo = (T)(1.0 / 36.0 - (double)w36);
+        const T wom = in0 * om, winv = (UNIT ? in0 : w36) * inv;
+        // v om / 36 (UNIT: / n0).  Every step scales a node's density and momentum by this factor times 36, so what a
+        // rounded constant om / 36 is off (up to 5e-8) would add up from step to step; with 1/36 in two
+        // parts only v's own rounding is left (velocity of the 512x128x128 channel after 40 steps)
+        const auto share = [&](T v) { return UNIT ? wom * v : om * (w36 * v + w36_lo * v); };
         const T uau = ua_[0] * u_[0] + ua_[1] * u_[1] + ua_[2] * u_[2];
         const T uu = u_[0] * u_[0] + u_[1] * u_[1] + u_[2] * u_[2];
         const T iso = (T)1.5 * n * ((T)2 * uau - uu);
         T s0 = (T)0;
-        const T a = (T)3 * wom * n, b = (T)3 * winv;
+        const T a = (T)3 * share(n), b = (T)3 * winv;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const T X = C[c] + nF[c], m = a * ua_[c], bX = b * X, bY = b * nF[c];
@@ -117,9 +122,9 @@ struct Collision {
             Of[c] = m + bX;
             Og[c] = m + bY;
         }
-        kf = wom * (dn - iso) - s0;
-        kg = wom * (Pi - iso) - s0;
-        k2 = (T)4.5 * wom * n;
+        kf = share(dn - iso) - s0;
+        kg = share(Pi - iso) - s0;
+        k2 = (T)1.5 * a;
         omc = (T)1 - om;
     }
 
