@@ -27,6 +27,7 @@
 // and now: 512x128x128 channel of diameters 4 and 6 251 -> 91 us, 256^3 well of diameter 6 373 -> 127 us, 64^3
 // well 50 -> 14 us, 90x75x66 with diameters 2, 4 and 6 129 -> 34 us.
 #pragma once
+#include <algorithm>
 #include <utility>
 
 #include "lbe_device.cuh"
@@ -107,24 +108,38 @@ struct Lane<double> {
     };
 };
 
-// Largest a with 4 (a^2 + dy^2 + Z^2) <= SIG^2, or -1: half-width of row dy of the ball's section at height Z.
-__host__ __device__ constexpr int ball_row(int sig, int dy, int Z) {
+// Balls |d| <= sigma/2 by their largest |d|^2.  An integer sigma has floor(sigma^2 / 4); the diameters accepted may lie
+// a rounding below an even one (5.999999999999999 from a division), whose ball ends before the points at sigma/2:
+// 3, 8 and 14 for 4, 6 and 8 (and 0 for 2).
+constexpr int NBALLS = 12;
+__host__ __device__ constexpr int ball_d2(int k) {
+    constexpr int d2[NBALLS] = {0, 1, 2, 3, 4, 6, 8, 9, 12, 14, 16, 20};
+    return d2[k];
+}
+__host__ __device__ constexpr int ball_radius(int d2) {  // floor of the root
+    int r = 0;
+    while ((r + 1) * (r + 1) <= d2) ++r;
+    return r;
+}
+
+// Largest a with a^2 + dy^2 + Z^2 <= D2, or -1: half-width of row dy of the ball's section at height Z.
+__host__ __device__ constexpr int ball_row(int d2, int dy, int Z) {
     int a = -1;
-    while (4 * ((a + 1) * (a + 1) + dy * dy + Z * Z) <= sig * sig) ++a;
+    while ((a + 1) * (a + 1) + dy * dy + Z * Z <= d2) ++a;
     return a;
 }
 
-// Sums of the plane around c over the sections of the ball |d|^2 <= SIG^2/4: D[Z], Z = 0 .. SIG/2 <= RB.
-template <typename T, int BX, int SIG, int RB>
+// Sums of the plane around c over the sections of the ball |d|^2 <= D2: D[Z], Z = 0 .. its radius <= RB.
+template <typename T, int BX, int D2, int RB>
 __device__ __forceinline__ void ball_sections(const T *c, typename Lane<T>::V (&D)[RB + 1]) {
     using Ln = Lane<T>;
     using V = typename Ln::V;
-    constexpr int R = SIG / 2;
+    constexpr int R = ball_radius(D2);
     [&]<int... DY>(std::integer_sequence<int, DY...>) {
         (
             [&] {
                 constexpr int dy = DY;
-                constexpr int E = ball_row(SIG, dy, 0);
+                constexpr int E = ball_row(D2, dy, 0);
                 typename Ln::template Row<E> rp, rm;
                 rp.load(c + dy * BX);
                 if constexpr (dy > 0) rm.load(c - dy * BX);
@@ -142,7 +157,7 @@ __device__ __forceinline__ void ball_sections(const T *c, typename Lane<T>::V (&
                             [&]<int... Z>(std::integer_sequence<int, Z...>) {
                                 (
                                     [&] {
-                                        if constexpr (ball_row(SIG, dy, Z) == a) D[Z] = dy == 0 ? s : Ln::add(D[Z], s);
+                                        if constexpr (ball_row(D2, dy, Z) == a) D[Z] = dy == 0 ? s : Ln::add(D[Z], s);
                                     }(),
                                     ...);
                             }(std::make_integer_sequence<int, R + 1>{});
@@ -159,7 +174,7 @@ struct ContactMaps {
 };
 template <typename T>
 struct ContactConst {
-    int s[MAXS];         // integer diameters
+    int ball[MAXS];      // the species' balls (ball_d2)
     int lz;              // output planes per block
     T c2[MAXS], c3[MAXS];  // (pi/6) sigma^k over the points of the ball: the sums' weights in xi_k
     T s1[MAXS][MAXS], s2[MAXS][MAXS];  // 3 s_ab, 2 s_ab^2
@@ -261,16 +276,17 @@ __global__ void __launch_bounds__(CT_THREADS)
 #pragma unroll
             for (int Z = 0; Z <= RB; ++Z) D[Z] = Ln::zero();
             const T *c = sp + b * PL;
-            const int sig = cs.s[b];
-            [&]<int... SIG>(std::integer_sequence<int, SIG...>) {
+            const int ball = cs.ball[b];
+            [&]<int... K>(std::integer_sequence<int, K...>) {
                 (
                     [&] {
-                        // the widest ball of the launch first: the only one with one species
-                        constexpr int s = 2 * RB + 1 - SIG;
-                        if (sig == s) ball_sections<T, Tl::BX, s, RB>(c, D);
+                        constexpr int k = NBALLS - 1 - K, r = ball_radius(ball_d2(k));
+                        // one species: a ball of the launch's radius
+                        if constexpr (r == RB || (M > 1 && r < RB))
+                            if (ball == k) ball_sections<T, Tl::BX, ball_d2(k), RB>(c, D);
                     }(),
                     ...);
-            }(std::make_integer_sequence<int, 2 * RB + 2>{});
+            }(std::make_integer_sequence<int, NBALLS>{});
             // shift the running sums by one plane and add this plane's sections: output RB +- Z
 #pragma unroll
             for (int k = 0; k < 2 * RB; ++k) acc[b][k] = Ln::add(acc[b][k + 1], D[k < RB ? RB - k : k - RB]);
@@ -456,7 +472,14 @@ cudaError_t launch_ct(const ContactLaunch &L, cudaStream_t st) {
     for (int b = 0; b < M; ++b) maps.m[b] = L.maps[b];
     ContactConst<T> cs{};
     for (int b = 0; b < M; ++b) {
-        cs.s[b] = (int)(L.cp->sigma[b] + 0.5);
+        int d2 = 0;  // of the rows that also normalise the average
+        for (int dz = -4; dz <= 4; ++dz)
+            for (int k = L.br->first[b][dz + 4]; k < L.br->first[b][dz + 5]; ++k)
+                d2 = std::max(d2, dz * dz + L.br->dy[b][k] * L.br->dy[b][k] + L.br->a[b][k] * L.br->a[b][k]);
+        cs.ball[b] = -1;
+        for (int k = 0; k < NBALLS; ++k)
+            if (ball_d2(k) == d2) cs.ball[b] = k;
+        if (cs.ball[b] < 0) return cudaErrorInvalidValue;
         cs.c2[b] = (T)(L.cp->xi2c[b] / L.br->count[b]);
         cs.c3[b] = (T)(L.cp->xi3c[b] / L.br->count[b]);
         cs.refn[b] = (float)L.refn[b];

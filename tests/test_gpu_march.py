@@ -47,3 +47,27 @@ def test_march_edges(shape, periodic, sig, prec, tol):
             assert rel_err(g.force(a), obs["C"][a]) <= tol
         else:
             assert np.abs(g.force(a)).max() <= tol * n0
+
+
+@pytest.mark.parametrize("prec,tol", [("fp32", 1e-5), ("fp64", 1e-12)])
+@pytest.mark.parametrize("sig", [(2.0,), (4.0,), (6.0,), (7.0,), (8.0,), (2.0, 4.0, 6.0, 8.0), (6.0, 0.0)])
+def test_diameters_a_rounding_off_an_integer(sig, prec, tol):
+    """Diameters are integers to 1e-12.  Just below an even one the ball |d| <= sigma/2 ends before the points at sigma/2,
+    just above any it is the integer's."""
+    if prec == "fp64" and max(sig) > 7:
+        pytest.skip("no direct FP64 stencil of this diameter")
+    shape, N, M = (19, 10, 9), 1710, len(sig)
+    rng = np.random.default_rng(7)
+    n0 = 6.0 * 0.1 / (np.pi * sum(s ** 3 for s in sig))
+    for off in (-1e-13, 1e-13):
+        s = [v * (1.0 + off) for v in sig]
+        arr = dict(solid=np.zeros(N, np.uint8), V=np.zeros((M, N)), phi=np.zeros(N), amp=np.zeros(N),
+                   n=n0 * (1.0 + 0.3 * (rng.random((M, N)) - 0.5)))
+        w = dict(shape=shape, periodic=(1, 1, 1), sigma=s, tau=[1.0] * M, body=[(0.0, 0.0, 0.0)] * M)
+        g, o = setup_gpu(w, arr, prec, shell="direct"), setup_oracle(w, arr)
+        obs = o.observe()
+        for a in range(M):
+            for b in range(M):
+                if s[a] + s[b] > 0:
+                    assert rel_err(g.contact(a, b), obs["g"][a, b]) <= tol
+            assert rel_err(g.force(a), obs["C"][a]) <= tol
