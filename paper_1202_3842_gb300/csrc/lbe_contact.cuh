@@ -211,7 +211,8 @@ __global__ void __launch_bounds__(CT_THREADS)
 
     const int tid = threadIdx.x;
     const int tx = tid % (32 / NX) * NX, ty = tid / (32 / NX);
-    const int x0 = blockIdx.x * Tl::TX, y0 = blockIdx.y * Tl::TY, z0 = blockIdx.z * cs.lz;
+    const int nbx = (g.nx + Tl::TX - 1) / Tl::TX;  // tiles of a plane lie along the grid's x, which has room for all
+    const int x0 = blockIdx.x % nbx * Tl::TX, y0 = blockIdx.x / nbx * Tl::TY, z0 = blockIdx.z * cs.lz;
     const int nout = min(cs.lz, g.nz - z0);
     const int nplanes = nout + 2 * RB;
     const bool leader = tid == 0;
@@ -490,9 +491,9 @@ cudaError_t launch_ct(const ContactLaunch &L, cudaStream_t st) {
             cs.s2[a][b] = (T)(2.0 * s * s);
         }
     }
-    const int nbx = (g.nx + Tl::TX - 1) / Tl::TX, nby = (g.ny + Tl::TY - 1) / Tl::TY;
-    cs.lz = march_planes((long long)nbx * nby, g.nz, RB, per_sm, 0.35, 2.4);
-    dim3 grid(nbx, nby, (g.nz + cs.lz - 1) / cs.lz);
+    const int tiles = (g.nx + Tl::TX - 1) / Tl::TX * ((g.ny + Tl::TY - 1) / Tl::TY);
+    cs.lz = march_planes(tiles, g.nz, RB, per_sm, 0.35, 2.4, false, 65535);
+    dim3 grid(tiles, 1, (g.nz + cs.lz - 1) / cs.lz);
     return launch_pdl(k_contact_tma<T, M, RB, MODE>, grid, CT_THREADS, Tl::SMEM, st, maps, g, cs, (T *)L.gab,
                       (T *)L.npad2, (T *)L.gnpad, (T *)L.xi, L.mask, (T *)L.ln, L.top, L.err);
 }

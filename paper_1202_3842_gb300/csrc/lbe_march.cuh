@@ -86,22 +86,23 @@ __device__ __forceinline__ void store_pair(float *p, f2 v, bool vec, bool both) 
 // constants of both kernels are fits to sweeps of lz on GB300 (512x128x128, 256^3, 128x32x32 and 64^3; within
 // 10% of the measured times).
 // Where blocks differ in length (`mixed`), a round of resident blocks takes less than its longest.
-inline int march_planes(long long tiles, int nz, int r, int per_sm, double halo, double lat, bool mixed = false) {
-    int best = 1;
+// At most `most` parts (a grid has 65535 blocks along z).
+inline int march_planes(long long tiles, int nz, int r, int per_sm, double halo, double lat, bool mixed, int most) {
+    int best = 0;
     double cost = 0.0;
-    for (int parts = nz; parts >= 1; --parts) {
-        const int lz = (nz + parts - 1) / parts;
-        if ((nz + lz - 1) / lz != parts) continue;
+    for (int lz = (nz + most - 1) / most;;) {  // the shortest march of every number of parts
+        const int parts = (nz + lz - 1) / lz;
         const double b = (double)tiles * parts / 152.0;
         double n = b <= per_sm ? (double)(long long)(b + 0.999) : b + 0.4;
         if (mixed && n > 1.0 && b <= per_sm) n -= 0.4;
         const double t = (n + lat) * (lz + 2 * r * halo);
-        if (parts == nz || t <= cost) {
+        if (!best || t <= cost) {
             cost = t;
             best = lz;
         }
+        if (parts == 1) return best;
+        lz = (nz + parts - 2) / (parts - 1);
     }
-    return best;
 }
 
 // Tensor maps of the shell fields of every ordered pair [a][b]: n_b and g_ab n_b (FP32: their deviations), boxes

@@ -238,7 +238,8 @@ __device__ __forceinline__ bool fixed_march(const ShellMarchMaps &maps, const Fi
     const int fld = tid / (32 * FX_TY);  // 0: P (n_b), 1: Q (g_ab n_b)
     const int ot = tid - fld * (32 * FX_TY);
     const int row = ot >> 5, tx = ot & 31;
-    const int x0 = blockIdx.x * 32, y0 = blockIdx.y * FX_TY;
+    const int nbx = (g.nx + 31) / 32;  // tiles of a plane lie along the grid's x, which has room for all
+    const int x0 = blockIdx.x % nbx * 32, y0 = blockIdx.x / nbx * FX_TY;
     const int x = x0 + tx, y = y0 + row;
     const int pair = a * A.M + b;
     const int nplanes = nout + 2 * S;
@@ -389,11 +390,11 @@ cudaError_t launch_shell_fixed_t(const ShellMarchMaps &maps, FixedArgs &A, cudaS
         attr_set = true;
     }
     const Grid &g = A.g;
-    const int tx = (g.nx + 31) / 32, ty = (g.ny + FX_TY - 1) / FX_TY;
-    A.lz = march_planes((long long)tx * ty * A.M, g.nz, SMAX, fixed_per_sm(SMAX), 1.0, 0.9, A.M > 1);
+    const int tiles = (g.nx + 31) / 32 * ((g.ny + FX_TY - 1) / FX_TY);
+    A.lz = march_planes((long long)tiles * A.M, g.nz, SMAX, fixed_per_sm(SMAX), 1.0, 0.9, A.M > 1, 65535 / A.M);
     A.nzb = (g.nz + A.lz - 1) / A.lz;
-    march_order(A, (long long)tx * ty * A.M * A.nzb, fixed_per_sm(SMAX));
-    return launch_pdl(k_shell_fixed<SMAX>, dim3(tx, ty, A.M * A.nzb), 64 * FX_TY, smem, st, maps, A);
+    march_order(A, (long long)tiles * A.M * A.nzb, fixed_per_sm(SMAX));
+    return launch_pdl(k_shell_fixed<SMAX>, dim3(tiles, 1, A.M * A.nzb), 64 * FX_TY, smem, st, maps, A);
 }
 
 }  // namespace lbe

@@ -176,7 +176,8 @@ __device__ __forceinline__ bool shell_march(const ShellMarchMaps &maps, const Sh
     const int ot = tid - fld * (16 * SM_TY);
     const int row = 2 * (warp - fld * (SM_TY / 2)) + (lane >> 4);
     const int tx = 2 * (lane & 15);
-    const int x0 = blockIdx.x * 32, y0 = blockIdx.y * SM_TY;
+    const int nbx = (g.nx + 31) / 32;  // tiles of a plane lie along the grid's x, which has room for all
+    const int x0 = blockIdx.x % nbx * 32, y0 = blockIdx.x / nbx * SM_TY;
     const int x = x0 + tx, y = y0 + row;
     const int pair = a * A.M + b;
     const int nplanes = nout + 2 * S;
@@ -322,12 +323,12 @@ cudaError_t launch_shell_march_t(const ShellMarchMaps &maps, ShellMarchArgs &A, 
         attr_set = true;
     }
     const Grid &g = A.g;
-    const int tx = (g.nx + 31) / 32, ty = (g.ny + SM_TY - 1) / SM_TY;
+    const int tiles = (g.nx + 31) / 32 * ((g.ny + SM_TY - 1) / SM_TY);
     constexpr int per_sm = shell_march_per_sm(SMAX);
-    A.lz = march_planes((long long)tx * ty * A.M, g.nz, SMAX, per_sm, 1.0, 0.9, A.M > 1);
+    A.lz = march_planes((long long)tiles * A.M, g.nz, SMAX, per_sm, 1.0, 0.9, A.M > 1, 65535 / A.M);
     A.nzb = (g.nz + A.lz - 1) / A.lz;
-    march_order(A, (long long)tx * ty * A.M * A.nzb, per_sm);
-    return launch_pdl(k_shell_march<SMAX>, dim3(tx, ty, A.M * A.nzb), 32 * SM_TY, smem, st, maps, A);
+    march_order(A, (long long)tiles * A.M * A.nzb, per_sm);
+    return launch_pdl(k_shell_march<SMAX>, dim3(tiles, 1, A.M * A.nzb), 32 * SM_TY, smem, st, maps, A);
 }
 
 }  // namespace lbe

@@ -71,3 +71,33 @@ def test_diameters_a_rounding_off_an_integer(sig, prec, tol):
                 if s[a] + s[b] > 0:
                     assert rel_err(g.contact(a, b), obs["g"][a, b]) <= tol
             assert rel_err(g.force(a), obs["C"][a]) <= tol
+
+
+@pytest.mark.parametrize("prec,tol,shape,sig", [
+    ("fp64", 1e-12, (4, 131076, 2), 2.0),  # more rows than 65535 tiles of two hold
+    ("fp32", 1e-5, (2, 262148, 1), 3.0),   # of four
+    ("fp32", 1e-5, (4, 3, 65540), 1.0),    # more planes than a grid is long, where marches of one plane are cheapest
+    ("fp64", 1e-12, (4, 3, 65540), 1.0),
+])
+def test_long_axes(prec, tol, shape, sig):
+    """The same lattice with its long axis along x, where no limit lies, up to round-off."""
+    rng = np.random.default_rng(9)
+    nx, ny, nz = shape
+    n = 6.0 * 0.1 / (np.pi * sig ** 3) * (1.0 + 0.3 * (rng.random((nz, ny, nx)) - 0.5))
+
+    def run(n, shape):
+        N = n.size
+        arr = dict(solid=np.zeros(N, np.uint8), V=np.zeros((1, N)), phi=np.zeros(N), amp=np.zeros(N),
+                   n=np.ascontiguousarray(n).reshape(1, N))
+        w = dict(shape=shape, periodic=(1, 1, 1), sigma=[sig], tau=[1.0], body=[(0.0, 0.0, 0.0)])
+        g = setup_gpu(w, arr, prec, shell="direct")
+        c = g.force(0).reshape((3,) + n.shape)
+        g.step(2)
+        return g.density(0).reshape(n.shape), c
+
+    swap = 1 if ny > nz else 0  # the long axis of an array [z][y][x]
+    d, c = run(n, shape)
+    e, f = run(np.swapaxes(n, swap, 2), (ny, nx, nz) if swap else (nz, ny, nx))
+    order = [1, 0, 2] if swap else [2, 1, 0]
+    assert rel_err(d, np.swapaxes(e, swap, 2)) <= tol
+    assert rel_err(c, np.swapaxes(f, swap + 1, 3)[order]) <= tol
