@@ -344,13 +344,9 @@ __global__ void __launch_bounds__(32 * TYB, 1)
 template <int S, int TZ, int TYB, int CC>
 cudaError_t launch_adj_tile2_cc(const AdjShellTile &L, cudaStream_t st) {
     using Tl = ShellTileZ2<S, TZ, TYB>;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_adj_shell_tile2<S, TZ, TYB, CC>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, Tl::SMEM);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static PerDevice once;
+    const cudaError_t e = allow_smem(once, k_adj_shell_tile2<S, TZ, TYB, CC>, Tl::SMEM);
+    if (e != cudaSuccess) return e;
     const Grid &g = *L.grid;
     dim3 block(Tl::TX, Tl::TY, 1);
     dim3 grid((g.nx + Tl::TX - 1) / Tl::TX, (g.ny + Tl::TY - 1) / Tl::TY, (g.nz + Tl::LZ - 1) / Tl::LZ);
@@ -374,13 +370,9 @@ cudaError_t launch_adj_tile2(const AdjShellTile &L, cudaStream_t st) {
 template <typename T, int S, int TZ, int TYB, int CC>
 cudaError_t launch_adj_tile_cc(const AdjShellTile &L, cudaStream_t st) {
     using Tl = ShellTileZ<T, S, TZ, TYB>;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_adj_shell_tile<T, S, TZ, TYB, CC>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, Tl::SMEM);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static PerDevice once;
+    const cudaError_t e = allow_smem(once, k_adj_shell_tile<T, S, TZ, TYB, CC>, Tl::SMEM);
+    if (e != cudaSuccess) return e;
     const Grid &g = *L.grid;
     dim3 block(Tl::TX, Tl::TY, 1);
     dim3 grid((g.nx + Tl::TX - 1) / Tl::TX, (g.ny + Tl::TY - 1) / Tl::TY, (g.nz + Tl::LZ - 1) / Tl::LZ);

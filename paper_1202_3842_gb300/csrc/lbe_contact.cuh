@@ -28,6 +28,7 @@
 // well 50 -> 14 us, 90x75x66 with diameters 2, 4 and 6 129 -> 34 us.
 #pragma once
 #include <algorithm>
+#include <atomic>
 #include <utility>
 
 #include "lbe_device.cuh"
@@ -458,15 +459,16 @@ __global__ void __launch_bounds__(CT_THREADS)
 template <typename T, int M, int RB, int MODE>
 cudaError_t launch_ct(const ContactLaunch &L, cudaStream_t st) {
     using Tl = ContactTile<T, M, RB>;
-    static int per_sm = 0;
-    if (!per_sm) {
-        cudaError_t e = cudaFuncSetAttribute(k_contact_tma<T, M, RB, MODE>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, Tl::SMEM);
+    static PerDevice once;
+    cudaError_t e = allow_smem(once, k_contact_tma<T, M, RB, MODE>, Tl::SMEM);
+    if (e != cudaSuccess) return e;
+    static std::atomic<int> resident{0};  // blocks per SM, the same on every device this library runs on
+    int per_sm = resident.load(std::memory_order_relaxed);
+    if (per_sm == 0) {
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_contact_tma<T, M, RB, MODE>, CT_THREADS, Tl::SMEM);
         if (e != cudaSuccess) return e;
-        int n = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_contact_tma<T, M, RB, MODE>, CT_THREADS, Tl::SMEM);
-        if (e != cudaSuccess) return e;
-        per_sm = n > 0 ? n : 1;
+        per_sm = per_sm > 0 ? per_sm : 1;
+        resident.store(per_sm, std::memory_order_relaxed);
     }
     const Grid &g = *L.grid;
     ContactMaps maps;

@@ -8,6 +8,7 @@
 #include <string>
 
 #include "lbe_device.cuh"
+#include "lbe_once.h"
 
 namespace lbe {
 
@@ -27,6 +28,15 @@ inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+// Lets a kernel take `bytes` of dynamic shared memory on the current device (a context may live on any).
+template <typename K>
+inline cudaError_t allow_smem(PerDevice &once, K *kernel, int bytes) {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    return once(dev, [&] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); });
 }
 
 // Threads per block of a kernel with one thread per node (or one group per node): `most` on large lattices, halved down

@@ -381,14 +381,10 @@ __global__ void __launch_bounds__(64 * FX_TY, fixed_per_sm(SMAX))
 
 template <int SMAX>
 cudaError_t launch_shell_fixed_t(const ShellMarchMaps &maps, FixedArgs &A, cudaStream_t st) {
-    static bool attr_set = false;
     constexpr int smem = FixedSmem<SMAX>::BYTES;
-    if (!attr_set) {
-        cudaError_t e =
-            cudaFuncSetAttribute(k_shell_fixed<SMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static PerDevice once;
+    const cudaError_t e = allow_smem(once, k_shell_fixed<SMAX>, smem);
+    if (e != cudaSuccess) return e;
     const Grid &g = A.g;
     const int tiles = (g.nx + 31) / 32 * ((g.ny + FX_TY - 1) / FX_TY);
     A.lz = march_planes((long long)tiles * A.M, g.nz, SMAX, fixed_per_sm(SMAX), 1.0, 0.9, A.M > 1, 65535 / A.M);

@@ -314,14 +314,10 @@ __global__ void __launch_bounds__(32 * SM_TY, shell_march_per_sm(SMAX))
 
 template <int SMAX>
 cudaError_t launch_shell_march_t(const ShellMarchMaps &maps, ShellMarchArgs &A, cudaStream_t st) {
-    static bool attr_set = false;
     constexpr int smem = ShellMarchSmem<SMAX>::BYTES;
-    if (!attr_set) {
-        cudaError_t e =
-            cudaFuncSetAttribute(k_shell_march<SMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static PerDevice once;
+    const cudaError_t e = allow_smem(once, k_shell_march<SMAX>, smem);
+    if (e != cudaSuccess) return e;
     const Grid &g = A.g;
     const int tiles = (g.nx + 31) / 32 * ((g.ny + SM_TY - 1) / SM_TY);
     constexpr int per_sm = shell_march_per_sm(SMAX);
