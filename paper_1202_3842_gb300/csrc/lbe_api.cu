@@ -71,8 +71,11 @@ struct lbe_ctx {
     Buf npad2;  // FP32 direct shell force: padded deviations n_b - ref_n [M][P]; gnpad then holds g_ab n_b - ref_g
     double ref_n[MAXS] = {0}, ref_g[MAXS][MAXS] = {{0}};
     bool ref_dirty = true;
-    Buf fix, top;  // FP64 direct shell force: fixed-point images of n_b and g_ab n_b [M + M^2][P], maxima's high words
-    ShellMarchMaps *march_maps = nullptr;
+    // FP64 direct shell force: fixed-point images of n_b and g_ab n_b [M + M^2][P], maxima's high words and the word
+    // that says whether a field's values lie too far apart for them
+    Buf fix, top;
+    bool shell_wide = false;  // k_shell_wide takes such fields (wide_maps: the padded fields themselves)
+    ShellMarchMaps *march_maps = nullptr, *wide_maps = nullptr;
     Buf flux_buf, flux_acc, flux_last;
     Buf err;
     Buf scratch64;  // FP64 scratch for getters: n [M][N] + J [M][3][N] (+ more)
@@ -683,17 +686,22 @@ lbe_status prepare(lbe_ctx *c) {
         if (!c->spectral && !f64) TRY(dev_alloc(c, c->npad2, rb * c->M * g.P));
         if (!c->spectral && f64) {
             TRY(dev_alloc(c, c->fix, 8 * (c->M + c->M * c->M) * g.P));
-            TRY(dev_alloc(c, c->top, 4 * (c->M + c->M * c->M)));
+            TRY(dev_alloc(c, c->top, 4 * (c->M + c->M * c->M + 1)));
         }
         c->ref_dirty = true;
         TRY(dev_alloc(c, c->gab, rb * c->M * c->M * g.N));
         TRY(dev_alloc(c, c->C, rb * c->M * 3 * g.N));
         CK(cudaMemsetAsync(c->npad.p, 0, rb * c->M * g.P, c->stream), "memset npad");
         if (!c->spectral && f64) CK(cudaMemsetAsync(c->gnpad.p, 0, gnb, c->stream), "memset gnpad");
-        if (!c->march_maps) {
-            c->march_maps = new (std::nothrow) ShellMarchMaps;
-            if (!c->march_maps) return fail(c, LBE_ERR_OOM, "host allocation failed");
+        for (ShellMarchMaps **m : {&c->march_maps, &c->wide_maps}) {
+            if (!*m) *m = new (std::nothrow) ShellMarchMaps;
+            if (!*m) return fail(c, LBE_ERR_OOM, "host allocation failed");
         }
+        // The fixed-point sums round relative to a field's largest value.  So do the FFTs; pairs that would not be
+        // theirs under the cost rule, or that the caller asked a stencil for, keep sums that round like the values.
+        c->shell_wide = f64 && !c->spectral && (c->shell_method == LBE_SHELL_DIRECT || !spectral_cheaper(c, f64));
+        int Smax = 0;
+        for (auto &ps : c->pairs) Smax = std::max(Smax, ps.S);
         CK(cudaMemsetAsync(c->C.p, 0, rb * c->M * 3 * g.N, c->stream), "memset C");
         for (auto &ps : c->pairs) {
             if (c->spectral) break;
@@ -704,6 +712,11 @@ lbe_status prepare(lbe_ctx *c) {
             shell_box(f64, ps.S, &bx, &by);
             TRY(make_map(c, &c->march_maps->n[ab], nb, bx, by));
             TRY(make_map(c, &c->march_maps->gn[ab], gn, bx, by));
+            if (c->shell_wide) {
+                shell_wide_box(Smax, ps.S, &bx, &by);
+                TRY(make_map(c, &c->wide_maps->n[ab], (char *)c->npad.p + rb * ps.b * g.P, bx, by));
+                TRY(make_map(c, &c->wide_maps->gn[ab], (char *)c->gnpad.p + rb * ab * g.P, bx, by));
+            }
         }
         {
             int bx = 0, by = 0;
@@ -817,7 +830,7 @@ lbe_status force_stage_core(lbe_ctx *c, const void *pop, void *Pbase, void *xiba
         std::memcpy(L.refg, c->ref_g, sizeof(L.refg));
         L.xi = xibase;
         L.top = (unsigned *)c->top.p;
-        if (f64) CK(cudaMemsetAsync(c->top.p, 0, 4 * (c->M + c->M * c->M), c->stream), "memset maxima");
+        if (f64) CK(cudaMemsetAsync(c->top.p, 0, 4 * (c->M + c->M * c->M + 1), c->stream), "memset maxima");
         L.err = (int *)c->err.p;
         LAUNCH(launch_contact_tma(f64, L, c->stream), "contact kernel");
     }
@@ -850,11 +863,14 @@ lbe_status force_stage_core(lbe_ctx *c, const void *pop, void *Pbase, void *xiba
     if (f64) {
         FixedArgs A{};
         fill(A, 0.0);
-        A.top = (const unsigned *)c->top.p;
-        LAUNCH(launch_to_fixed(Smax, (const double *)c->npad.p, (const double *)c->gnpad.p, c->g.P, c->M, A.top,
+        unsigned *top = (unsigned *)c->top.p;
+        A.top = top;
+        A.wide = c->shell_wide ? top + c->M + c->M * c->M : nullptr;
+        LAUNCH(launch_to_fixed(Smax, (const double *)c->npad.p, (const double *)c->gnpad.p, c->g.P, c->M, top,
                                (long long *)c->fix.p, c->stream),
                "fixed-point fields");
         LAUNCH(launch_shell_fixed(Smax, *c->march_maps, A, c->stream), "shell force kernel");
+        if (A.wide) LAUNCH(launch_shell_wide(Smax, *c->wide_maps, A, c->stream), "shell force of far-apart values");
     } else {
         ShellMarchArgs A{};
         fill(A, 0.f);
@@ -1087,6 +1103,7 @@ void lbe_destroy(lbe_ctx *c) {
     for (Buf *b : all) dev_free(c, *b);
     cudaStreamSynchronize(c->stream);
     delete c->march_maps;
+    delete c->wide_maps;
     delete c;
 }
 

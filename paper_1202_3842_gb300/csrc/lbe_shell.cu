@@ -53,10 +53,17 @@ __device__ __forceinline__ long long to_fixed(double v, int top, int bits) {
     const long long r = d <= 0 ? m << -d : (d > 54 ? 0 : (m + (1ll << (d - 1))) >> d);
     return b < 0 ? -r : r;
 }
+// Whether a value lies so far below the field's largest (a factor of 8 to 16) that the image may drop some of its bits.
+__device__ __forceinline__ bool far_below(double v, int top) {
+    const long long b = __double_as_longlong(v);
+    const int e = (int)((b >> 52) & 0x7ff);
+    return (b << 1) != 0 && (e + 3 < top || e == 0);
+}
 __global__ void __launch_bounds__(256) k_to_fixed(const double *__restrict__ npad, const double *__restrict__ gnpad,
-                                                 long long P, int M, int bits,
-                                                 const unsigned *__restrict__ top, long long *__restrict__ out) {
+                                                 long long P, int M, int bits, const unsigned *__restrict__ top,
+                                                 unsigned *__restrict__ wide, long long *__restrict__ out) {
     pdl_wait();
+    bool low = false;
     const int f = blockIdx.y;  // n_b, then g_ab n_b
     const double *src = f < M ? npad + f * P : gnpad + (long long)(f - M) * P;
     const int e = fx_exponent(top[f]);
@@ -66,13 +73,15 @@ __global__ void __launch_bounds__(256) k_to_fixed(const double *__restrict__ npa
          i += (long long)gridDim.x * blockDim.x) {
         const double2 v = s2[i];
         dst[i] = make_longlong2(to_fixed(v.x, e, bits), to_fixed(v.y, e, bits));
+        low = low || far_below(v.x, e) || far_below(v.y, e);
     }
+    if (low) *wide = 1u;
 }
 cudaError_t launch_to_fixed(int Smax, const double *npad, const double *gnpad, long long P, int M,
-                            const unsigned *top, long long *out, cudaStream_t st) {
+                            unsigned *top, long long *out, cudaStream_t st) {
     const long long nb = (P / 2 + 255) / 256;
     return launch_pdl(k_to_fixed, dim3((unsigned)(nb < 2048 ? nb : 2048), M + M * M), 256, 0, st, npad, gnpad, P, M,
-                      fx_bits(Smax), top, out);
+                      fx_bits(Smax), (const unsigned *)top, top + M + M * M, out);
 }
 
 bool shell_supported(bool fp64, int S) { return S >= 1 && S <= (fp64 ? 7 : 8); }

@@ -13,7 +13,9 @@
 //     that keep the product to about one unit of the fixed point.
 // Everything after that is exact again (adds and the factor Z), until the sums of an output become doubles.  The
 // result is the sum of the definition to a few 2^-55 of the field's largest value, where FP64 sums (and more so
-// the FFTs) round at every addition.
+// the FFTs) round at every addition.  FP64 sums round relative to the values at hand, though: where a field's
+// values lie more than a factor of 8 to 16 apart, k_shell_wide takes the launch (lbe_shell_wide.cu), except for
+// pairs whose general form are the FFTs, which round relative to the whole field, ten times as much.
 // Error of C against sums in extended precision, rms over max |C| (300 nodes; this kernel, the FP64 stencil it
 // replaces, the FFTs that were the default from diameter 4 on): 24^3 with 1% noise, diameter 3 9.0e-16, 9.2e-16,
 // 8.4e-15; diameter 6 1.15e-15, 1.08e-15, 1.3e-14; diameter 7 1.5e-15, 1.3e-15, 1.2e-14; 48^3 well of diameter 6
@@ -214,6 +216,7 @@ struct FixedArgs {
     int S[MAXS * MAXS], q[MAXS * MAXS];
     double coef[MAXS * MAXS];
     const unsigned *top;  // high words of the fields' largest values: n_b [M], g_ab n_b [M][M]
+    const unsigned *wide; // NULL, or not 0 where a field's values lie too far apart: k_shell_wide takes the pairs
     const double *npad, *gab;
     double *C, *Pout;
     int *err;
@@ -359,7 +362,7 @@ __global__ void __launch_bounds__(64 * FX_TY, fixed_per_sm(SMAX))
     }
     __syncthreads();
     pdl_wait();
-    if (nout <= 0) return;
+    if (nout <= 0 || (A.wide && *A.wide)) return;
     int it = 0;
     bool accumulate = false;
     for (int b = 0; b < A.M; ++b) {
