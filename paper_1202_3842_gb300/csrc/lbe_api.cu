@@ -863,14 +863,14 @@ lbe_status force_stage_core(lbe_ctx *c, const void *pop, void *Pbase, void *xiba
     if (f64) {
         FixedArgs A{};
         fill(A, 0.0);
-        unsigned *top = (unsigned *)c->top.p;
-        A.top = top;
-        A.wide = c->shell_wide ? top + c->M + c->M * c->M : nullptr;
-        LAUNCH(launch_to_fixed(Smax, (const double *)c->npad.p, (const double *)c->gnpad.p, c->g.P, c->M, top,
+        unsigned *wide = c->shell_wide ? (unsigned *)c->top.p + c->M + c->M * c->M : nullptr;
+        A.top = (const unsigned *)c->top.p;
+        A.wide = wide;
+        LAUNCH(launch_to_fixed(Smax, (const double *)c->npad.p, (const double *)c->gnpad.p, c->g.P, c->M, A.top, wide,
                                (long long *)c->fix.p, c->stream),
                "fixed-point fields");
         LAUNCH(launch_shell_fixed(Smax, *c->march_maps, A, c->stream), "shell force kernel");
-        if (A.wide) LAUNCH(launch_shell_wide(Smax, *c->wide_maps, A, c->stream), "shell force of far-apart values");
+        if (wide) LAUNCH(launch_shell_wide(Smax, *c->wide_maps, A, c->stream), "shell force of far-apart values");
     } else {
         ShellMarchArgs A{};
         fill(A, 0.f);

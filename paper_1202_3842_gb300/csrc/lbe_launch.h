@@ -178,13 +178,13 @@ void contact_box(bool fp64, int M, int RB, int *bx, int *by);
 cudaError_t launch_shell_march(int Smax, const ShellMarchMaps &maps, ShellMarchArgs &A, cudaStream_t st);
 cudaError_t launch_fill(float *p, long long n, float v, cudaStream_t st);
 // K3 in FP64, diameters 1..7, and the fixed-point images [M + M^2][P] of its fields; top: high words of the
-// largest values of n_b [M] and g_ab n_b [M][M], from K2, then the word that k_to_fixed sets where a field's values
-// lie far apart.  launch_shell_wide: the same sums in FP64 on the padded fields themselves, where that word is set.
+// largest values of n_b [M] and g_ab n_b [M][M], from K2; wide: NULL, or a word that k_to_fixed sets (from 0) where a
+// field's values lie far apart.  launch_shell_wide: the same sums in FP64 on the padded fields themselves, where that word is set.
 cudaError_t launch_shell_fixed(int Smax, const ShellMarchMaps &maps, FixedArgs &A, cudaStream_t st);
 cudaError_t launch_shell_wide(int Smax, const ShellMarchMaps &maps, FixedArgs &A, cudaStream_t st);
 void shell_wide_box(int Smax, int S, int *bx, int *by);
 cudaError_t launch_to_fixed(int Smax, const double *npad, const double *gnpad, long long P, int M,
-                            unsigned *top, long long *out, cudaStream_t st);
+                            const unsigned *top, unsigned *wide, long long *out, cudaStream_t st);
 bool shell_supported(bool fp64, int S);
 void shell_box(bool fp64, int S, int *bx, int *by);      // forward kernels
 void adj_shell_box(bool fp64, int S, int *bx, int *by);  // shell transpose: boxes of its own tiles

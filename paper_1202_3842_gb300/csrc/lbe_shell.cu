@@ -75,13 +75,14 @@ __global__ void __launch_bounds__(256) k_to_fixed(const double *__restrict__ npa
         dst[i] = make_longlong2(to_fixed(v.x, e, bits), to_fixed(v.y, e, bits));
         low = low || far_below(v.x, e) || far_below(v.y, e);
     }
-    if (low) *wide = 1u;
+    // (wide: NULL where nothing asks; most warps find the word set already)
+    if (wide && __any_sync(0xffffffffu, low) && (threadIdx.x & 31) == 0 && *(volatile unsigned *)wide == 0u) *wide = 1u;
 }
 cudaError_t launch_to_fixed(int Smax, const double *npad, const double *gnpad, long long P, int M,
-                            unsigned *top, long long *out, cudaStream_t st) {
+                            const unsigned *top, unsigned *wide, long long *out, cudaStream_t st) {
     const long long nb = (P / 2 + 255) / 256;
     return launch_pdl(k_to_fixed, dim3((unsigned)(nb < 2048 ? nb : 2048), M + M * M), 256, 0, st, npad, gnpad, P, M,
-                      fx_bits(Smax), (const unsigned *)top, top + M + M * M, out);
+                      fx_bits(Smax), top, wide, out);
 }
 
 bool shell_supported(bool fp64, int S) { return S >= 1 && S <= (fp64 ? 7 : 8); }
