@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(collide_threads(M), collide_ctas(M, sizeof(T) 
         return;
     }
     Collision<T, UNIT> col;
-    col.set(n, DEV ? dn : n, Pi, ua, u, Cv, nF, sc_omega<S, T>(sc), sc_inv<S, T>(sc),
+    col.set(n, DEV ? dn : n, Pi, J, ua, u, Cv, nF, sc_omega<S, T>(sc), sc_inv<S, T>(sc),
             UNIT ? sc_in0<S, T>(sc) : (T)0);
     col.rest(f[0], gq[0]);
     put(std::integral_constant<int, 0>{}, f[0], gq[0]);

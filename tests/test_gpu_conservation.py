@@ -2,7 +2,7 @@
 import numpy as np
 import pytest
 
-from lbe_cases import setup_gpu
+from lbe_cases import rel_err, setup_gpu, setup_oracle
 
 pytestmark = pytest.mark.gpu
 
@@ -33,3 +33,27 @@ def test_fp32_momentum_of_a_periodic_gas(M, tau):
     mass, mom, _ = g.totals()
     assert np.abs(mom - mom0).max() <= 1e-5 * np.abs(mom0).max()
     assert np.abs(mass - mass0).max() <= 1e-6 * mass0.max()
+
+
+@pytest.mark.parametrize("prec,tol", [("fp32", 1e-5), ("fp64", 1e-12)])
+@pytest.mark.parametrize("M", [1, 2, 3])
+def test_nodes_without_density(M, prec, tol):
+    """Populations after a collision where f sums to 0 and g does not: velocity and equilibrium are 0 there."""
+    shape, N = (9, 5, 4), 180
+    rng = np.random.default_rng(8)
+    arr = dict(solid=np.zeros(N, np.uint8), V=np.zeros((M, N)), phi=np.zeros(N), amp=np.zeros(N),
+               n=np.zeros((M, N)))  # deviations from 0: such a node sums to 0 exactly
+    w = dict(shape=shape, periodic=(1, 1, 1), sigma=[0.0] * M, tau=[0.8] * M, body=[(1e-3, 0.0, 0.0)] * M)
+    g, o = setup_gpu(w, arr, prec), setup_oracle(w, arr)
+    empty = rng.random(N) < 0.3
+    for a in range(M):
+        f = W[:, None] * 0.05 * (1.0 + 0.1 * rng.random((19, N)))
+        q = W[:, None] * 0.05 * (1.0 + 0.1 * rng.random((19, N)))
+        f[:, empty] = 0.0
+        g.set_populations(a, f, q)
+        o.set_populations(a, f, q)
+    g.step(1)
+    o.step(1)
+    for a in range(M):
+        for got, ref in zip(g.populations(a), o.get_populations(a)):
+            assert rel_err(np.asarray(got).reshape(-1), np.asarray(ref).reshape(-1)) <= tol
