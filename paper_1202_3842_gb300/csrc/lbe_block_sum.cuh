@@ -31,6 +31,14 @@ __host__ __device__ __forceinline__ double bits_double(long long b) {
 #endif
 }
 
+// 2 v by its exponent; zero, subnormal and the largest values, whose exponents do not tell, by an addition.
+__host__ __device__ __forceinline__ double twice(double v) {
+    const long long b = double_bits(v);
+    const unsigned e = (unsigned)(b >> 52) & 0x7ffu;
+    if (e - 1u < 0x7fdu) return bits_double(b + (1ll << 52));
+    return v + v;
+}
+
 // Largest biased exponent of the populations, or 0 where they cannot be summed as integers.
 __host__ __device__ __forceinline__ int block_exponent(const double *v) {
     unsigned m = 0;

@@ -210,12 +210,6 @@ struct Collision64 {
             r[e] += d[i] * ua[j] + d[j] * ua[i];
         }
     }
-    // 2 v by its exponent (zero, subnormal and non-finite values as they are)
-    static __device__ __forceinline__ double twice(double v) {
-        const int h = __double2hiint(v);
-        const unsigned e = (unsigned)h >> 20 & 0x7ffu;
-        return __hiloint2double(e - 1u < 0x7fdu ? h + 0x100000 : h, __double2loint(v));
-    }
     __device__ __forceinline__ void rest(double &f) const { f = omc * f + 12.0 * k; }
     template <int P>
     __device__ __forceinline__ void pair(double &fp, double &fm) const {
