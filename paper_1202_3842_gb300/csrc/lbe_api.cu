@@ -512,7 +512,7 @@ lbe_status spectral_force(lbe_ctx *c, void *Pbase, void *xibase) {
     const int M = c->M, np = c->specPairs.npairs;
     const long long Nr = c->specNr, Nc = c->specNc;
     char *R = (char *)c->specR.p, *Z = (char *)c->specZ.p, *W = (char *)c->specW.p;
-    const double scale = 1.0 / (double)Nr;
+    const double scale = 1.0 / ((double)c->specL[0] * c->specL[1] * c->specL[2]);
     {
         StageTimer t(c, LBE_STAGE_CONTACT);
         LAUNCH(launch_spec_embed_n(f64, c->g, c->specL, Nr, M, c->npad.p, R, c->stream), "spectral embed");
@@ -1772,7 +1772,7 @@ lbe_status lbe_adjoint_flux_gradient(lbe_ctx *c, int T, int K, int axis, int pla
             return fail(c, LBE_ERR_UNSUPPORTED, "spectral shell transpose: " + why);
         }
         c->aspec = sp_new;
-        c->aNr = (long long)c->aL[0] * c->aL[1] * c->aL[2];
+        c->aNr = spectral_stride(c->aL);
         c->aNc = (long long)(c->aL[0] / 2 + 1) * c->aL[1] * c->aL[2];
         lbe_status st = LBE_OK;
         if (st == LBE_OK) st = dev_alloc(c, c->aR, rb * (size_t)std::max(nf, 3) * c->aNr);
@@ -1910,7 +1910,8 @@ lbe_status lbe_adjoint_flux_gradient(lbe_ctx *c, int T, int K, int axis, int pla
                     release();
                     return fail(c, LBE_ERR_CUDA, "spectral shell transpose: cuFFT forward transform failed");
                 }
-                LAUNCH(launch_adjspec_multiply(f64, aZ.p, aTab.p, aW.p, aNc, asp, 1.0 / (double)aNr, c->stream),
+                LAUNCH(launch_adjspec_multiply(f64, aZ.p, aTab.p, aW.p, aNc, asp,
+                                               1.0 / ((double)aL[0] * aL[1] * aL[2]), c->stream),
                        "adjoint spectral multiply");
                 if (spectral_inverse(aspec, 1, aW.p, aR.p) != 0) {
                     release();

@@ -301,6 +301,9 @@ struct SpecPairs {
     double half_coef[MAXS * MAXS];       // coef_ab / 2
 };
 struct SpectralShell;  // cuFFT plans of one lattice
+// Elements from one real grid field to the next: the grid's points, and one more where they are odd in number (cuFFT
+// wants every array aligned for its complex type).
+long long spectral_stride(const int L[3]);
 bool spectral_available(std::string *why);
 // Plans for the grid L (x fastest): forward of the M densities (0), inverse of ninv force spectra (1),
 // forward of three table fields (2), forward of the npairs fields g n (3), inverse of the M ball

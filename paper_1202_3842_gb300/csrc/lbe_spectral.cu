@@ -24,10 +24,12 @@
 // libcufft.so.12 so that the library still needs only libcuda to load; without it the spectral
 // method reports LBE_ERR_UNSUPPORTED.
 #include <cufft.h>
+#include <climits>
 #include <dlfcn.h>
 
 #include <mutex>
 #include <type_traits>
+#include <climits>
 #include <string>
 
 #include "lbe_device.cuh"
@@ -115,6 +117,11 @@ void spectral_destroy(SpectralShell *s) {
     delete s;
 }
 
+long long spectral_stride(const int L[3]) {
+    const long long n = (long long)L[0] * L[1] * L[2];
+    return n + (n & 1);
+}
+
 int spectral_create(SpectralShell **out, bool fp64, const int L[3], int M, int npairs, int ninv, size_t *work_bytes,
                     std::string *why) {
     const int batch[SpectralShell::NPLAN] = {M, ninv, 3, npairs, M};
@@ -132,9 +139,17 @@ int spectral_create_plans(SpectralShell **out, bool fp64, const int L[3], int np
     s->api = api;
     s->fp64 = fp64;
     for (int k = 0; k < 3; ++k) s->L[k] = L[k];
-    s->Nr = (long long)L[0] * L[1] * L[2];
+    const long long count = (long long)L[0] * L[1] * L[2];
+    s->Nr = spectral_stride(L);
     s->Nc = (long long)(L[0] / 2 + 1) * L[1] * L[2];
     int n[3] = {L[2], L[1], L[0]};  // row-major: x is the fastest (and the halved) dimension
+    int nc[3] = {L[2], L[1], L[0] / 2 + 1};
+    const bool padded = s->Nr != count;  // fields apart by more than their size: the layout in full
+    if (padded && (s->Nr > INT_MAX || s->Nc > INT_MAX)) {
+        if (why) *why = "an odd grid of 2^31 points or more";
+        spectral_destroy(s);
+        return -1;
+    }
     const cufftType fwd = fp64 ? CUFFT_D2Z : CUFFT_R2C, inv = fp64 ? CUFFT_Z2D : CUFFT_C2R;
     size_t wmax = 0;
     for (int k = 0; k < nplans; ++k) {
@@ -147,7 +162,10 @@ int spectral_create_plans(SpectralShell **out, bool fp64, const int L[3], int np
         s->made[k] = true;
         api->set_auto(s->plan[k], 0);
         size_t ws = 0;
-        r = api->make_many(s->plan[k], 3, n, nullptr, 1, 0, nullptr, 1, 0, forward[k] ? fwd : inv, batch[k], &ws);
+        const int dr = padded ? (int)s->Nr : 0, dc = padded ? (int)s->Nc : 0;
+        int *const er = padded ? n : nullptr, *const ec = padded ? nc : nullptr;
+        r = forward[k] ? api->make_many(s->plan[k], 3, n, er, 1, dr, ec, 1, dc, fwd, batch[k], &ws)
+                       : api->make_many(s->plan[k], 3, n, ec, 1, dc, er, 1, dr, inv, batch[k], &ws);
         if (r != CUFFT_SUCCESS) {
             if (why) *why = "cufftMakePlanMany failed (" + std::to_string((int)r) + ")";
             spectral_destroy(s);

@@ -102,3 +102,31 @@ def test_automatic_choice_and_errors():
     Phi, dA, dG = g.adjoint_flux_gradient(2, 1, 0, 10)
     assert np.isfinite(Phi) and np.isfinite(dA).all() and np.isfinite(dG).all()
     assert abs(dG[0]) > 0  # the flux responds to the body force (no wall potential here, so dA = 0)
+
+
+@pytest.mark.parametrize("prec,tol", [("fp64", 1e-12), ("fp32", 1e-5)])
+@pytest.mark.parametrize("shape,periodic,sig", [
+    ((15, 13, 11), (1, 1, 1), (3.0,)),       # an odd number of grid points: fields at odd distances
+    ((15, 13, 11), (1, 1, 1), (4.0, 6.0)),
+    ((21, 10, 9), (1, 0, 1), (4.0,)),        # odd rows; y is extended to 14
+    ((17, 9, 13), (1, 0, 0), (6.0, 6.0)),    # y and z are extended to 15 and 20
+    ((9, 9, 9), (0, 0, 0), (6.0,)),          # all three to 15
+])
+def test_odd_grids(shape, periodic, sig, prec, tol):
+    N, M = int(np.prod(shape)), len(sig)
+    rng = np.random.default_rng(23)
+    solid = (rng.random(N) < 0.05).astype(np.uint8)
+    n0 = 6.0 * 0.12 / (np.pi * sum(s ** 3 for s in sig))
+    arr = dict(solid=solid, V=np.zeros((M, N)), phi=np.zeros(N), amp=np.zeros(N),
+               n=n0 * (1.0 + 0.3 * (rng.random((M, N)) - 0.5)) * (solid == 0)[None, :])
+    w = dict(shape=shape, periodic=periodic, sigma=list(sig), tau=[1.0] * M, body=[(1e-4, 0.0, 0.0)] * M)
+    g, obs = setup_gpu(w, arr, prec, shell="spectral"), setup_oracle(w, arr).observe()
+    for a in range(M):
+        for b in range(M):
+            assert rel_err(g.contact(a, b), obs["g"][a, b]) <= tol
+        assert rel_err(g.force(a), obs["C"][a]) <= tol
+    if prec == "fp64":  # the transpose, against the stencil's
+        d = setup_gpu(w, arr, prec, shell="direct")
+        for x, y in zip(g.adjoint_flux_gradient(3, 2, 0, 7), d.adjoint_flux_gradient(3, 2, 0, 7)):
+            x, y = np.asarray(x), np.asarray(y)
+            assert np.abs(x - y).max() <= 1e-10 * max(np.abs(y).max(), 1e-30)
