@@ -485,7 +485,7 @@ lbe_status spectral_setup(lbe_ctx *c) {
     size_t ws = 0;
     if (spectral_create(&c->spec, f64, L, M, sp.npairs, ninv, &ws, &why) != 0)
         return fail(c, LBE_ERR_UNSUPPORTED, "spectral shell force: " + why);
-    const long long Nr = (long long)L[0] * L[1] * L[2], Nc = (long long)(L[0] / 2 + 1) * L[1] * L[2];
+    const long long Nr = spectral_stride(L), Nc = (long long)(L[0] / 2 + 1) * L[1] * L[2];
     // real fields: the densities, the pairs' g n and the ball averages, later the ninv force fields
     TRY(dev_alloc(c, c->specR, rb * (size_t)std::max(ninv, std::max(nfwd + M, 3)) * Nr));
     TRY(dev_alloc(c, c->specZ, 2 * rb * (size_t)std::max(nfwd, 3) * Nc));
@@ -516,24 +516,24 @@ lbe_status spectral_force(lbe_ctx *c, void *Pbase, void *xibase) {
     {
         StageTimer t(c, LBE_STAGE_CONTACT);
         LAUNCH(launch_spec_embed_n(f64, c->g, c->specL, Nr, M, c->npad.p, R, c->stream), "spectral embed");
-        if (spectral_forward(c->spec, 0, R, Z) != 0)
-            return fail(c, LBE_ERR_CUDA, "spectral contact values: cuFFT forward transform failed");
+        if (const int r = spectral_forward(c->spec, 0, R, Z))
+            return fail(c, LBE_ERR_CUDA, "spectral contact values: cuFFT forward transform failed (" + std::to_string(r) + ")");
         LAUNCH(launch_spec_ball_mul(f64, Z, (const char *)c->specTab.p + rb * 3 * (size_t)c->specNS * Nc, W, Nc, M,
                                     scale, c->stream),
                "spectral ball average");
         char *nbar = R + rb * (size_t)(M + np) * Nr;
-        if (spectral_inverse(c->spec, 4, W, nbar) != 0)
-            return fail(c, LBE_ERR_CUDA, "spectral contact values: cuFFT inverse transform failed");
+        if (const int r = spectral_inverse(c->spec, 4, W, nbar))
+            return fail(c, LBE_ERR_CUDA, "spectral contact values: cuFFT inverse transform failed (" + std::to_string(r) + ")");
         LAUNCH(launch_spec_contact(f64, c->g, c->specL, Nr, c->cparams, c->specPairs, c->npad.p, nbar, c->gab.p,
                                    xibase, R + rb * (size_t)M * Nr, (int *)c->err.p, c->stream),
                "spectral contact values");
     }
     StageTimer t(c, LBE_STAGE_SHELL);
-    if (spectral_forward(c->spec, 3, R + rb * (size_t)M * Nr, Z + 2 * rb * (size_t)M * Nc) != 0)
-        return fail(c, LBE_ERR_CUDA, "spectral shell force: cuFFT forward transform failed");
+    if (const int r = spectral_forward(c->spec, 3, R + rb * (size_t)M * Nr, Z + 2 * rb * (size_t)M * Nc))
+        return fail(c, LBE_ERR_CUDA, "spectral shell force: cuFFT forward transform failed (" + std::to_string(r) + ")");
     LAUNCH(launch_spec_multiply(f64, Z, c->specTab.p, W, Nc, c->specPairs, scale, c->stream), "spectral multiply");
-    if (spectral_inverse(c->spec, 1, W, R) != 0)
-        return fail(c, LBE_ERR_CUDA, "spectral shell force: cuFFT inverse transform failed");
+    if (const int r = spectral_inverse(c->spec, 1, W, R))
+        return fail(c, LBE_ERR_CUDA, "spectral shell force: cuFFT inverse transform failed (" + std::to_string(r) + ")");
     LAUNCH(launch_spec_combine(f64, c->g, c->specL, Nr, R, c->npad.p, c->gab.p, c->specPairs, c->C.p, Pbase,
                                c->stream),
            "spectral combine");
