@@ -410,23 +410,35 @@ __global__ void __launch_bounds__(CT_THREADS)
                             q[0] = pv[f][0];
                         }
                     }
-                    // the periodic images inside the halo: one offset for all fields
+                    // the periodic images inside the halo: one offset for all fields; along y and z a pair stays one
+                    // store (two stores of every other value: 330 instead of 203 us on 1024x1024x1, two species)
                     const Images iz = images(z, g.nz, g.H, g.per[2]);
                     if (edge || (iz.k0 | iz.k1) != 0) {
+                        for (int kz = iz.k0; kz <= iz.k1; ++kz)
+                            for (int ky = iy.k0; ky <= iy.k1; ++ky) {
+                                const long long d =
+                                    pc + (long long)g.px * (ky * g.ny + (long long)g.py * (kz * g.nz));
+                                if ((ky | kz) != 0) {
 #pragma unroll
-                        for (int o = 0; o < NX; ++o) {
-                            if (o == 1 && !both) continue;
-                            const Images ix = o ? ix1 : ix0;
-                            for (int kz = iz.k0; kz <= iz.k1; ++kz)
-                                for (int ky = iy.k0; ky <= iy.k1; ++ky)
-                                    for (int kx = ix.k0; kx <= ix.k1; ++kx) {
-                                        if ((kx | ky | kz) == 0) continue;
-                                        const long long d = pc + o + kx * g.nx +
-                                                            g.px * (ky * g.ny + (long long)g.py * (kz * g.nz));
-#pragma unroll
-                                        for (int f = 0; f < ND + M * M; ++f) field(f)[d] = pv[f][o];
+                                    for (int f = 0; f < ND + M * M; ++f) {
+                                        T *q = field(f) + d;
+                                        if (NX == 2 && both)
+                                            *reinterpret_cast<float2 *>(q) = make_float2(pv[f][0], pv[f][NX - 1]);
+                                        else
+                                            q[0] = pv[f][0];
                                     }
-                        }
+                                }
+#pragma unroll
+                                for (int o = 0; o < NX; ++o) {
+                                    if (o == 1 && !both) continue;
+                                    const Images ix = o ? ix1 : ix0;
+                                    for (int kx = ix.k0; kx <= ix.k1; ++kx) {
+                                        if (kx == 0) continue;
+#pragma unroll
+                                        for (int f = 0; f < ND + M * M; ++f) field(f)[d + o + kx * g.nx] = pv[f][o];
+                                    }
+                                }
+                            }
                     }
                     if (bad) atomicOr(err, ERR_PACKING);
                 }
