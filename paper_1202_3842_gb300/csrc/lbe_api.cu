@@ -74,6 +74,7 @@ struct lbe_ctx {
     // FP64 direct shell force: fixed-point images of n_b and g_ab n_b [M + M^2][P], maxima's high words and the word
     // that says whether a field's values lie too far apart for them
     Buf fix, top;
+    bool march_swap = false;  // the shell march goes along y, its tiles' rows along z
     bool shell_wide = false;  // k_shell_wide takes such fields (wide_maps: the padded fields themselves)
     ShellMarchMaps *march_maps = nullptr, *wide_maps = nullptr;
     Buf flux_buf, flux_acc, flux_last;
@@ -261,7 +262,7 @@ PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
 
 // 3-D map over a padded field of the compute type, or (pair = true, FP32) over the interleaved
 // (n_b, g_ab n_b) field as 8-byte elements.
-lbe_status make_map(lbe_ctx *c, CUtensorMap *map, void *base, int bx, int by, bool pair = false) {
+lbe_status make_map(lbe_ctx *c, CUtensorMap *map, void *base, int bx, int by, bool pair = false, int bz = 1) {
     auto enc = get_encode();
     if (!enc) return fail(c, LBE_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
     const bool f64 = prec_fp64(c->prec);
@@ -269,7 +270,7 @@ lbe_status make_map(lbe_ctx *c, CUtensorMap *map, void *base, int bx, int by, bo
     const size_t es = e8 ? 8 : 4;
     cuuint64_t dims[3] = {(cuuint64_t)c->g.px, (cuuint64_t)c->g.py, (cuuint64_t)c->g.pz};
     cuuint64_t strides[2] = {(cuuint64_t)c->g.px * es, (cuuint64_t)c->g.px * c->g.py * es};
-    cuuint32_t box[3] = {(cuuint32_t)bx, (cuuint32_t)by, 1};
+    cuuint32_t box[3] = {(cuuint32_t)bx, (cuuint32_t)by, (cuuint32_t)bz};
     cuuint32_t estr[3] = {1, 1, 1};
     const CUtensorMapDataType dt = f64 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64
                                        : (pair ? CU_TENSOR_MAP_DATA_TYPE_UINT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32);
@@ -702,6 +703,11 @@ lbe_status prepare(lbe_ctx *c) {
         c->shell_wide = f64 && !c->spectral && (c->shell_method == LBE_SHELL_DIRECT || !spectral_cheaper(c, f64));
         int Smax = 0;
         for (auto &ps : c->pairs) Smax = std::max(Smax, ps.S);
+        // The shell march goes along z unless y is clearly the better way: each cut of the march reads 2S planes again,
+        // so few nodes along z cost many times their share (1024x1024x1, diameter 6: 400 us along z, 220 for the
+        // half-shell kernel before it).
+        c->march_swap = Smax > 0 && shell_march_cost(f64, g, c->M, Smax, true) <
+                                        0.8 * shell_march_cost(f64, g, c->M, Smax, false);
         CK(cudaMemsetAsync(c->C.p, 0, rb * c->M * 3 * g.N, c->stream), "memset C");
         for (auto &ps : c->pairs) {
             if (c->spectral) break;
@@ -710,8 +716,9 @@ lbe_status prepare(lbe_ctx *c) {
             char *gn = f64 ? (char *)c->fix.p + rb * (c->M + ab) * g.P : (char *)c->gnpad.p + rb * ab * g.P;
             int bx = 0, by = 0;
             shell_box(f64, ps.S, &bx, &by);
-            TRY(make_map(c, &c->march_maps->n[ab], nb, bx, by));
-            TRY(make_map(c, &c->march_maps->gn[ab], gn, bx, by));
+            const int mby = c->march_swap ? 1 : by, mbz = c->march_swap ? by : 1;
+            TRY(make_map(c, &c->march_maps->n[ab], nb, bx, mby, false, mbz));
+            TRY(make_map(c, &c->march_maps->gn[ab], gn, bx, mby, false, mbz));
             if (c->shell_wide) {
                 shell_wide_box(Smax, ps.S, &bx, &by);
                 TRY(make_map(c, &c->wide_maps->n[ab], (char *)c->npad.p + rb * ps.b * g.P, bx, by));
@@ -841,6 +848,7 @@ lbe_status force_stage_core(lbe_ctx *c, const void *pop, void *Pbase, void *xiba
     auto fill = [&](auto &A, auto zero) {  // the launch's arguments, in the precision of `zero`
         using T = decltype(zero);
         A.g = c->g;
+        A.dir = march_axes(c->g, c->march_swap);
         A.M = c->M;
         for (size_t q = 0; q < c->pairs.size(); ++q) {
             const PairShell &ps = c->pairs[q];

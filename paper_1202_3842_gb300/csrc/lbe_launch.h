@@ -186,7 +186,9 @@ void shell_wide_box(int Smax, int S, int *bx, int *by);
 cudaError_t launch_to_fixed(int Smax, const double *npad, const double *gnpad, long long P, int M,
                             const unsigned *top, unsigned *wide, long long *out, cudaStream_t st);
 bool shell_supported(bool fp64, int S);
-void shell_box(bool fp64, int S, int *bx, int *by);      // forward kernels
+void shell_box(bool fp64, int S, int *bx, int *by);      // forward kernels: extent along x and along the tile's rows
+// Time of the forward march of M species, in planes of one block per SM (march_planes), with rows along y or z.
+double shell_march_cost(bool fp64, const Grid &g, int M, int Smax, bool swap);
 void adj_shell_box(bool fp64, int S, int *bx, int *by);  // shell transpose: boxes of its own tiles
 // K4: fused moments + DD-TR collision + pull streaming.
 cudaError_t launch_collide(Prec p, const Grid &g, const void *src, void *dst, const uint32_t *mask, bool solid,

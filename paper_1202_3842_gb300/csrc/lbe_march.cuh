@@ -87,7 +87,9 @@ __device__ __forceinline__ void store_pair(float *p, f2 v, bool vec, bool both) 
 // 10% of the measured times).
 // Where blocks differ in length (`mixed`), a round of resident blocks takes less than its longest.
 // At most `most` parts (a grid has 65535 blocks along z).
-inline int march_planes(long long tiles, int nz, int r, int per_sm, double halo, double lat, bool mixed, int most) {
+// `cost`: the product itself, in planes of one block per SM.
+inline int march_planes(long long tiles, int nz, int r, int per_sm, double halo, double lat, bool mixed, int most,
+                        double *cost_out = nullptr) {
     int best = 0;
     double cost = 0.0;
     for (int lz = (nz + most - 1) / most;;) {  // the shortest march of every number of parts
@@ -100,9 +102,34 @@ inline int march_planes(long long tiles, int nz, int r, int per_sm, double halo,
             cost = t;
             best = lz;
         }
-        if (parts == 1) return best;
+        if (parts == 1) break;
         lz = (nz + parts - 2) / (parts - 1);
     }
+    if (cost_out) *cost_out = cost;
+    return best;
+}
+
+// Which way a shell march goes.  Its tiles have rows along `row` (1: y, 2: z) and it advances along the other axis; a
+// plane of the tile is a box of one node along that axis, so one tensor serves both (the shell is symmetric).
+struct MarchAxes {
+    int swap;        // 0: rows along y, march along z; 1: rows along z, march along y
+    int rows, planes;  // the lattice's extents along them
+    unsigned srow, splane;  // a node's distance to the next row and plane, in nodes
+    long long prow, pplane;  // the same in the padded field
+};
+inline MarchAxes march_axes(const Grid &g, bool swap) {
+    const long long pxy = (long long)g.px * g.py;
+    const unsigned xy = (unsigned)g.nx * (unsigned)g.ny;
+    return swap ? MarchAxes{1, g.nz, g.ny, xy, (unsigned)g.nx, pxy, g.px}
+                : MarchAxes{0, g.ny, g.nz, (unsigned)g.nx, xy, g.px, pxy};
+}
+
+__device__ __forceinline__ long long march_pidx(const Grid &g, const MarchAxes &dir, int x, int y, int z) {
+    return x + g.H + dir.prow * (y + g.H) + dir.pplane * (z + g.H);
+}
+// Offset of the force's component that the tile knows as c (0: x, 1: along its rows, 2: along the march).
+__device__ __forceinline__ long long march_component(const Grid &g, const MarchAxes &dir, int c) {
+    return g.N * (c == 0 ? 0 : (c == 1 ? 1 + dir.swap : 2 - dir.swap));
 }
 
 // Tensor maps of the shell fields of every ordered pair [a][b]: n_b and g_ab n_b (FP32: their deviations), boxes

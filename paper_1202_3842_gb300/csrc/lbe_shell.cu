@@ -100,6 +100,17 @@ void adj_shell_box(bool fp64, int S, int *bx, int *by) {
     *by = (S >= 5 ? 4 : 8) + 2 * S;
 }
 
+double shell_march_cost(bool fp64, const Grid &g, int M, int Smax, bool swap) {
+    const MarchAxes dir = march_axes(g, swap);
+    const int ty = fp64 ? FX_TY : SM_TY;
+    const int smax = Smax <= 4 ? 4 : (Smax <= 6 ? 6 : (fp64 ? 7 : 8));
+    const int per_sm = fp64 ? fixed_per_sm(smax) : shell_march_per_sm(smax);
+    const long long tiles = (long long)((g.nx + 31) / 32) * ((dir.rows + ty - 1) / ty);
+    double cost = 0.0;
+    march_planes(tiles * M, dir.planes, smax, per_sm, 1.0, 0.9, M > 1, 65535 / M, &cost);
+    return cost;
+}
+
 void shell_box(bool fp64, int S, int *bx, int *by) {
     if (!fp64) {  // ShellMarchTile
         *bx = 32 + 2 * ((S + 3) / 4 * 4);

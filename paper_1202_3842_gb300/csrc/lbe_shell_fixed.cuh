@@ -211,6 +211,7 @@ __device__ __forceinline__ void fixed_plane(const i64 *c, FixedSum *Bx, FixedSum
 
 struct FixedArgs {
     Grid g;
+    MarchAxes dir;
     int M, lz, nzb;
     int order[MAXS];
     int S[MAXS * MAXS], q[MAXS * MAXS];
@@ -237,6 +238,7 @@ __device__ __forceinline__ bool fixed_march(const ShellMarchMaps &maps, const Fi
     using Tl = FixedTile<S>;
     using Sm = FixedSmem<SMAX>;
     const Grid &g = A.g;
+    const MarchAxes &dir = A.dir;
     const int tid = threadIdx.x;
     const int fld = tid / (32 * FX_TY);  // 0: P (n_b), 1: Q (g_ab n_b)
     const int ot = tid - fld * (32 * FX_TY);
@@ -250,13 +252,13 @@ __device__ __forceinline__ bool fixed_march(const ShellMarchMaps &maps, const Fi
     const int first_it = it;
     double *xch = reinterpret_cast<double *>(base + Sm::XCH);
 
-    auto issue = [&](int j) {  // plane j holds interior z = z0 - S + j
+    auto issue = [&](int j) {  // plane j holds interior z = z0 - S + j (z: along the march, y: along the rows)
         const int k = first_it + j, slot = k % FX_R;
         unsigned char *dst = base + slot * Sm::SLOT;
         const int bx = x0 + g.H - Tl::S2, by = y0 + g.H - S, zp = z0 - S + j + g.H;
         mbar_arrive_expect_tx(&bars[slot], 2u * Tl::PLANE * 8u);
-        tma_load_3d(dst, &maps.n[pair], bx, by, zp, &bars[slot]);
-        tma_load_3d(dst + Tl::PLANE_BYTES, &maps.gn[pair], bx, by, zp, &bars[slot]);
+        tma_load_3d(dst, &maps.n[pair], bx, dir.swap ? zp : by, dir.swap ? by : zp, &bars[slot]);
+        tma_load_3d(dst + Tl::PLANE_BYTES, &maps.gn[pair], bx, dir.swap ? zp : by, dir.swap ? by : zp, &bars[slot]);
     };
     if (leader) {
         if (first_it > 0) fence_proxy_async_smem();  // the ring was read for the pair before
@@ -266,28 +268,29 @@ __device__ __forceinline__ bool fixed_march(const ShellMarchMaps &maps, const Fi
     i64 ax[2 * S], ay[2 * S], az[2 * S];
 #pragma unroll
     for (int k = 0; k < 2 * S; ++k) ax[k] = ay[k] = az[k] = 0;
-    const bool act = x < g.nx && y < g.ny;
-    unsigned i = (unsigned)x + (unsigned)g.nx * ((unsigned)y + (unsigned)g.ny * (unsigned)z0);
+    const bool act = x < g.nx && y < dir.rows;
+    unsigned i = (unsigned)x + dir.srow * (unsigned)y + dir.splane * (unsigned)z0;
     // fixed point to double: the field's scale, and the unit of the products
     const int top = fx_exponent(A.top[fld == 0 ? b : A.M + pair]);
     const double unit = fx_pow2(top - 1023 - (fx_bits(SMAX) - 1) + fx_unit(S));
     const double half_coef = 0.5 * A.coef[pair];
-    double *Cb = A.C + 3 * (long long)a * g.N;
+    double *const Ca = A.C + 3 * (long long)a * g.N, *const Pa = A.Pout ? A.Pout + 3 * (long long)A.q[pair] * g.N : nullptr;
+    const long long comp[3] = {0, march_component(g, dir, 1), march_component(g, dir, 2)};
     const double *gb = A.gab + (long long)pair * g.N;
-    double *Pb = A.Pout ? A.Pout + 3 * (long long)A.q[pair] * g.N : nullptr;
+    const double *np = A.npad + (long long)a * g.P + march_pidx(g, dir, x, y, z0);
     const int coff = (row + S) * Tl::BX + tx + Tl::S2;
 
     double na = 0.0, gr = 0.0, old[3] = {0.0, 0.0, 0.0};  // the epilogue's reads, one plane ahead
-    auto load_epilogue = [&](int z) {
-        na = A.npad[(long long)a * g.P + pidx(g, x, y, z)];
+    auto load_epilogue = [&] {
+        na = *np;
         if (fld == 0) {
             gr = gb[i];
         } else if (accumulate) {
 #pragma unroll
-            for (int c = 0; c < 3; ++c) old[c] = Cb[c * g.N + i];
+            for (int c = 0; c < 3; ++c) old[c] = Ca[comp[c] + i];
         }
     };
-    if (act) load_epilogue(z0);
+    if (act) load_epilogue();
 
     for (int j = 0; j < nplanes; ++j) {
         const int k = first_it + j, slot = k % FX_R;
@@ -325,7 +328,7 @@ __device__ __forceinline__ bool fixed_march(const ShellMarchMaps &maps, const Fi
             for (int cc = 0; cc < 3; ++cc) {
                 const double p = unit * (double)v[cc];
                 xo[cc * (32 * FX_TY)] = gp * p;
-                if (Pb) Pb[cc * g.N + i] = p;
+                if (Pa) Pa[comp[cc] + i] = p;
             }
         }
         __syncthreads();
@@ -336,11 +339,12 @@ __device__ __forceinline__ bool fixed_march(const ShellMarchMaps &maps, const Fi
         if (fld == 1 && out) {
 #pragma unroll
             for (int cc = 0; cc < 3; ++cc)
-                Cb[cc * g.N + i] = old[cc] + fma(pre, unit * (double)v[cc], xo[cc * (32 * FX_TY)]);
+                Ca[comp[cc] + i] = old[cc] + fma(pre, unit * (double)v[cc], xo[cc * (32 * FX_TY)]);
         }
         if (j >= 2 * S) {
-            i += (unsigned)(g.nx * g.ny);
-            if (act && j + 1 < nplanes) load_epilogue(z0 + j + 1 - 2 * S);
+            i += dir.splane;
+            np += dir.pplane;
+            if (act && j + 1 < nplanes) load_epilogue();
         }
     }
     it = first_it + nplanes;
@@ -355,7 +359,7 @@ __global__ void __launch_bounds__(64 * FX_TY, fixed_per_sm(SMAX))
     uint64_t *bars = reinterpret_cast<uint64_t *>(base + FixedSmem<SMAX>::BARS);
     const int k = blockIdx.z / A.nzb, a = A.order[k];
     const int z0 = (blockIdx.z - k * A.nzb) * A.lz;
-    const int nout = min(A.lz, A.g.nz - z0);
+    const int nout = min(A.lz, A.dir.planes - z0);
     if (threadIdx.x == 0) {
         for (int r = 0; r < FX_R; ++r) mbar_init(&bars[r], 1);
         fence_mbar_init();
@@ -389,9 +393,9 @@ cudaError_t launch_shell_fixed_t(const ShellMarchMaps &maps, FixedArgs &A, cudaS
     const cudaError_t e = allow_smem(once, k_shell_fixed<SMAX>, smem);
     if (e != cudaSuccess) return e;
     const Grid &g = A.g;
-    const int tiles = (g.nx + 31) / 32 * ((g.ny + FX_TY - 1) / FX_TY);
-    A.lz = march_planes((long long)tiles * A.M, g.nz, SMAX, fixed_per_sm(SMAX), 1.0, 0.9, A.M > 1, 65535 / A.M);
-    A.nzb = (g.nz + A.lz - 1) / A.lz;
+    const int tiles = (g.nx + 31) / 32 * ((A.dir.rows + FX_TY - 1) / FX_TY);
+    A.lz = march_planes((long long)tiles * A.M, A.dir.planes, SMAX, fixed_per_sm(SMAX), 1.0, 0.9, A.M > 1, 65535 / A.M);
+    A.nzb = (A.dir.planes + A.lz - 1) / A.lz;
     march_order(A, (long long)tiles * A.M * A.nzb, fixed_per_sm(SMAX));
     return launch_pdl(k_shell_fixed<SMAX>, dim3(tiles, 1, A.M * A.nzb), 64 * FX_TY, smem, st, maps, A);
 }

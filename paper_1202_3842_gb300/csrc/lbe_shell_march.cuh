@@ -153,6 +153,7 @@ __device__ __forceinline__ void march_plane(const float *c, f2 *Bx, f2 *By, f2 *
 
 struct ShellMarchArgs {
     Grid g;
+    MarchAxes dir;
     int M, lz, nzb;              // planes per block, blocks along z
     int order[MAXS];             // species in the order their blocks start
     int S[MAXS * MAXS];          // pair diameter of [a][b], 0: no pair
@@ -171,6 +172,7 @@ __device__ __forceinline__ bool shell_march(const ShellMarchMaps &maps, const Sh
     using Tl = ShellMarchTile<S>;
     using Sm = ShellMarchSmem<SMAX>;
     const Grid &g = A.g;
+    const MarchAxes &dir = A.dir;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int fld = warp / (SM_TY / 2);  // 0: P (n_b), 1: Q (g_ab n_b)
     const int ot = tid - fld * (16 * SM_TY);
@@ -185,13 +187,13 @@ __device__ __forceinline__ bool shell_march(const ShellMarchMaps &maps, const Sh
     const int first_it = it;
     f2 *xch = reinterpret_cast<f2 *>(base + Sm::XCH);
 
-    auto issue = [&](int j) {  // plane j holds interior z = z0 - S + j
+    auto issue = [&](int j) {  // plane j holds interior z = z0 - S + j (z: along the march, y: along the rows)
         const int k = first_it + j, slot = k % SM_R;
         unsigned char *dst = base + slot * Sm::SLOT;
         const int bx = x0 + g.H - Tl::S4, by = y0 + g.H - S, zp = z0 - S + j + g.H;
         mbar_arrive_expect_tx(&bars[slot], 2u * Tl::PLANE * 4u);
-        tma_load_3d(dst, &maps.n[pair], bx, by, zp, &bars[slot]);
-        tma_load_3d(dst + Tl::PLANE_BYTES, &maps.gn[pair], bx, by, zp, &bars[slot]);
+        tma_load_3d(dst, &maps.n[pair], bx, dir.swap ? zp : by, dir.swap ? by : zp, &bars[slot]);
+        tma_load_3d(dst + Tl::PLANE_BYTES, &maps.gn[pair], bx, dir.swap ? zp : by, dir.swap ? by : zp, &bars[slot]);
     };
     if (leader) {
         if (first_it > 0) fence_proxy_async_smem();  // the ring was read for the pair before
@@ -201,30 +203,31 @@ __device__ __forceinline__ bool shell_march(const ShellMarchMaps &maps, const Sh
     f2 ax[2 * S], ay[2 * S], az[2 * S];
 #pragma unroll
     for (int k = 0; k < 2 * S; ++k) ax[k] = ay[k] = az[k] = 0ull;
-    const bool act0 = x < g.nx && y < g.ny, act1 = act0 && x + 1 < g.nx;
+    const bool act0 = x < g.nx && y < dir.rows, act1 = act0 && x + 1 < g.nx;
     const bool vec = (g.nx & 1) == 0;  // rows start on 8-byte boundaries
     // node index of the output at hand (lattices hold fewer than 2^31 nodes); one 32-bit offset per thread from
     // the pair's base pointers, which are the same for the whole block
-    unsigned i = (unsigned)x + (unsigned)g.nx * ((unsigned)y + (unsigned)g.ny * (unsigned)z0);
+    unsigned i = (unsigned)x + dir.srow * (unsigned)y + dir.splane * (unsigned)z0;
     const f2 half_coef = f2splat(0.5f * A.coef[pair]);
     const int coff = (row + S) * Tl::BX + tx + Tl::S4;
-    float *Cb = A.C + 3 * (long long)a * g.N;
+    float *const Ca = A.C + 3 * (long long)a * g.N, *const Pa = A.Pout ? A.Pout + 3 * (long long)A.q[pair] * g.N : nullptr;
+    const long long comp[3] = {0, march_component(g, dir, 1), march_component(g, dir, 2)};
     const float *gb = A.gab + (long long)pair * g.N;
-    float *Pb = A.Pout ? A.Pout + 3 * (long long)A.q[pair] * g.N : nullptr;
+    const float *np = A.npad + (long long)a * g.P + march_pidx(g, dir, x, y, z0);
 
     // what the epilogue reads from global memory, loaded one plane ahead; rows of the padded field start on
     // 8-byte boundaries and x is even, so its two outputs are one load (within the row)
     f2 na = 0, gr = 0, old[3] = {0, 0, 0};
-    auto load_epilogue = [&](int z) {
-        na = *reinterpret_cast<const f2 *>(A.npad + (long long)a * g.P + pidx(g, x, y, z));
+    auto load_epilogue = [&] {
+        na = *reinterpret_cast<const f2 *>(np);
         if (fld == 0) {
             gr = load_pair(gb + i, vec, act1);
         } else if (accumulate) {
 #pragma unroll
-            for (int c = 0; c < 3; ++c) old[c] = load_pair(Cb + c * g.N + i, vec, act1);
+            for (int c = 0; c < 3; ++c) old[c] = load_pair(Ca + comp[c] + i, vec, act1);
         }
     };
-    if (act0) load_epilogue(z0);
+    if (act0) load_epilogue();
 
     for (int j = 0; j < nplanes; ++j) {
         const int k = first_it + j, slot = k % SM_R;
@@ -255,7 +258,7 @@ __device__ __forceinline__ bool shell_march(const ShellMarchMaps &maps, const Sh
 #pragma unroll
             for (int cc = 0; cc < 3; ++cc) {
                 xo[cc * (16 * SM_TY)] = f2mul(gp, v[cc]);
-                if (Pb) store_pair(Pb + cc * g.N + i, v[cc], vec, act1);
+                if (Pa) store_pair(Pa + comp[cc] + i, v[cc], vec, act1);
             }
         }
         __syncthreads();
@@ -266,11 +269,12 @@ __device__ __forceinline__ bool shell_march(const ShellMarchMaps &maps, const Sh
         if (fld == 1 && out) {
 #pragma unroll
             for (int cc = 0; cc < 3; ++cc)
-                store_pair(Cb + cc * g.N + i, f2add(old[cc], f2fma(pre, v[cc], xo[cc * (16 * SM_TY)])), vec, act1);
+                store_pair(Ca + comp[cc] + i, f2add(old[cc], f2fma(pre, v[cc], xo[cc * (16 * SM_TY)])), vec, act1);
         }
         if (j >= 2 * S) {
-            i += (unsigned)(g.nx * g.ny);
-            if (act0 && j + 1 < nplanes) load_epilogue(z0 + j + 1 - 2 * S);
+            i += dir.splane;
+            np += dir.pplane;
+            if (act0 && j + 1 < nplanes) load_epilogue();
         }
     }
     it = first_it + nplanes;
@@ -285,7 +289,7 @@ __global__ void __launch_bounds__(32 * SM_TY, shell_march_per_sm(SMAX))
     uint64_t *bars = reinterpret_cast<uint64_t *>(base + ShellMarchSmem<SMAX>::BARS);
     const int k = blockIdx.z / A.nzb, a = A.order[k];
     const int z0 = (blockIdx.z - k * A.nzb) * A.lz;
-    const int nout = min(A.lz, A.g.nz - z0);
+    const int nout = min(A.lz, A.dir.planes - z0);
     if (threadIdx.x == 0) {
         for (int r = 0; r < SM_R; ++r) mbar_init(&bars[r], 1);
         fence_mbar_init();
@@ -319,10 +323,10 @@ cudaError_t launch_shell_march_t(const ShellMarchMaps &maps, ShellMarchArgs &A, 
     const cudaError_t e = allow_smem(once, k_shell_march<SMAX>, smem);
     if (e != cudaSuccess) return e;
     const Grid &g = A.g;
-    const int tiles = (g.nx + 31) / 32 * ((g.ny + SM_TY - 1) / SM_TY);
+    const int tiles = (g.nx + 31) / 32 * ((A.dir.rows + SM_TY - 1) / SM_TY);
     constexpr int per_sm = shell_march_per_sm(SMAX);
-    A.lz = march_planes((long long)tiles * A.M, g.nz, SMAX, per_sm, 1.0, 0.9, A.M > 1, 65535 / A.M);
-    A.nzb = (g.nz + A.lz - 1) / A.lz;
+    A.lz = march_planes((long long)tiles * A.M, A.dir.planes, SMAX, per_sm, 1.0, 0.9, A.M > 1, 65535 / A.M);
+    A.nzb = (A.dir.planes + A.lz - 1) / A.lz;
     march_order(A, (long long)tiles * A.M * A.nzb, per_sm);
     return launch_pdl(k_shell_march<SMAX>, dim3(tiles, 1, A.M * A.nzb), 32 * SM_TY, smem, st, maps, A);
 }

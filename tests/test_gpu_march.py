@@ -101,3 +101,27 @@ def test_long_axes(prec, tol, shape, sig):
     order = [1, 0, 2] if swap else [2, 1, 0]
     assert rel_err(d, np.swapaxes(e, swap, 2)) <= tol
     assert rel_err(c, np.swapaxes(f, swap + 1, 3)[order]) <= tol
+
+
+@pytest.mark.parametrize("prec,tol", [("fp32", 1e-5), ("fp64", 1e-12)])
+@pytest.mark.parametrize("shape,periodic,sig", [
+    ((37, 97, 1), (1, 1, 1), (6.0,)),            # one node along z: the march goes along y
+    ((37, 97, 1), (0, 1, 0), (5.0,)),
+    ((66, 301, 2), (1, 0, 1), (4.0, 6.0)),
+    ((33, 150, 3), (1, 1, 0), (2.0, 4.0, 6.0)),
+    ((5, 1030, 5), (1, 1, 1), (7.0,)),
+    ((35, 1, 90), (1, 1, 1), (4.0,)),            # one along y: it stays along z
+])
+def test_march_along_the_longer_axis(shape, periodic, sig, prec, tol):
+    test_march_edges(shape, periodic, sig, prec, tol)
+    # the adjoint keeps P of every pair: the transposed and the spectral form on the same lattice
+    if prec == "fp64" and len(sig) < 3:
+        N, M = int(np.prod(shape)), len(sig)
+        rng = np.random.default_rng(2)
+        n0 = 6.0 * 0.12 / (np.pi * sum(s ** 3 for s in sig))
+        arr = dict(solid=np.zeros(N, np.uint8), V=np.zeros((M, N)), phi=np.zeros(N), amp=np.zeros(N),
+                   n=n0 * (1.0 + 0.3 * (rng.random((M, N)) - 0.5)))
+        w = dict(shape=shape, periodic=periodic, sigma=list(sig), tau=[1.0] * M, body=[(1e-4, 0.0, 0.0)] * M)
+        x, y = (np.asarray(setup_gpu(w, arr, prec, shell=m).adjoint_flux_gradient(2, 1, 0, 3)[2])
+                for m in ("direct", "spectral"))
+        assert np.abs(x - y).max() <= 1e-10 * np.abs(y).max()
