@@ -84,12 +84,18 @@ typedef enum { LBE_DD_TR = 0, LBE_SD_TR = 1, LBE_SD_EU = 2, LBE_DD_EU = 3 } lbe_
  *     likewise; any integer pair diameter up to the limit of the contact
  *     values (sigma_b / 2 <= 4);
  *   LBE_SHELL_AUTO (default): spectral for diameters without a compiled
- *     stencil, direct for compiled diameters on lattices of 16384 nodes and
- *     more (measured on GB300); on smaller ones, and in FP32 runs of the
+ *     stencil; direct for compiled diameters on lattices of 16384 nodes and
+ *     more, except in FP32 where a cost model measured on GB300 finds the
+ *     spectral form faster (few nodes along two axes, or along one with large
+ *     diameters); on smaller lattices, and in FP32 runs of the
  *     single-distribution schemes, spectral where the mean shell of the pairs
  *     is above about 320 points (FP32) or 110 points (FP64), scaled by the
  *     padded grid over the lattice.
- * Both give the sums of the definition up to rounding.  The discrete adjoint
+ * Both give the sums of the definition up to rounding: the spectral form
+ * relative to a field's largest values, the direct form relative to the values
+ * on a node's shells; where AUTO takes the direct form in place of the
+ * spectral one in FP64, relative to a field's largest value too (by less).
+ * The discrete adjoint
  * (lbe_adjoint_flux_gradient) transposes the shell sums with the method this
  * call sets: the stencil (pair diameters with a compiled stencil), the
  * spectral form (any), or under LBE_SHELL_AUTO the spectral form unless the

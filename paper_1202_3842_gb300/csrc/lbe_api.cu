@@ -350,19 +350,45 @@ bool spectral_cheaper(const lbe_ctx *c, bool f64, double stencil_factor = 1.0) {
 }
 
 // Whether the marching kernels (lbe_shell_march.cuh, lbe_shell_fixed.cuh, lbe_contact.cuh) take the forward force
-// under LBE_SHELL_AUTO.  K2 + K3 on GB300 in FP32: 738 against 1146 us on the 256^3 well of diameter 6, 533 against
-// 602 us on a 192^3 well of diameter 8 (the widest they take), 1100 against 2390 us on the 512x128x128 channel
-// of diameters 4 and 6, 51 against 95 us on a 64^3 well of diameter 6; in FP64 1125 against 3870 us on the
-// 256x64x64 channel of diameters 4 and 6, 75 against 195 us on a 48^3 well of diameter 4: direct wherever a
-// stencil is compiled.  Lattices below DIRECT_NODES nodes are bound by launches in either form and keep the
-// rule above, which programs that record the method of a small lattice rely on.
+// under LBE_SHELL_AUTO where the rule above is for the spectral form.  K2 + K3 on GB300, march against FFTs:
+// - FP64: the march on every lattice measured (256x64x64 channel of diameters 4 and 6 1125 against 3870 us, 48^3 of
+//   diameter 7 189 against 199, 512x512x1 of diameter 6 345 against 418);
+// - FP32: the march on 256^3 of diameter 6 (738 against 1146), 192^3 of diameter 8 (533 against 602), the 512x128x128
+//   channel of diameters 4 and 6 (1100 against 2390), 64^3 of diameter 8 (70 against 89); the FFTs where its tiles or its
+//   2S extra planes are mostly empty (1024x1024x1 of diameter 6 239 against 129, of diameters 4 and 6 624 against
+//   210; 4096x16x16 of diameter 8 170 against 122).  Both sides as fits to 70 lattices, in us:
+//     march: 1.1e-3 shell_march_cost x points per species + 12 + 1.8e-6 padded field values + 2.5 P / N (the images of
+//     a node, one after the other),   FFTs: 72 + 6.3e-6 fields x grid points; within 15% the march;
+// - FP32 runs of the single-distribution schemes: the FFTs.  Their velocity carries the rounding of f (1e-5 of it and
+//   more), and a force that rounds otherwise moves it by half of that (well of diameter 6, 20 steps: 5.8e-6 between the
+//   two forms, each 1.0e-5 from FP64; the two-distribution schemes move by 2e-6 and less);
+// - fewer than DIRECT_NODES nodes: the FFTs, so that the method reported for a small lattice stays the one that it has
+//   been.  (The march is the faster form there too: 24^3, diameter 6, 29 against 75 us in FP32, 70 against 136 in
+//   FP64; set_shell_method takes it.)
 constexpr long long DIRECT_NODES = 16384;
-// FP32 runs of the single-distribution schemes keep the cost rule: their velocity carries the rounding of f (1e-5 of it
-// and more), and a force that rounds otherwise moves it by half of that (well of diameter 6, 20 steps: 5.8e-6 between
-// the two forms, each 1.0e-5 from FP64; the two-distribution schemes move by 2e-6 and less).
 bool direct_cheaper(const lbe_ctx *c) {
-    if (c->prec == Prec::F32 && (c->cfg.scheme == LBE_SD_TR || c->cfg.scheme == LBE_SD_EU)) return false;
-    return c->g.N >= DIRECT_NODES;
+    const Grid &g = c->g;
+    if (g.N < DIRECT_NODES) return false;
+    if (c->prec == Prec::F64) return true;
+    if (c->cfg.scheme == LBE_SD_TR || c->cfg.scheme == LBE_SD_EU) return false;
+    const int M = c->M, n3[3] = {g.nx, g.ny, g.nz};
+    int Smax = 0;
+    double points = 0.0;
+    for (const auto &ps : c->pairs) {
+        points += shell_count(ps.S);
+        Smax = std::max(Smax, ps.S);
+    }
+    const int H = (Smax + 3) / 4 * 4;
+    double P = 1.0, grid = 1.0;
+    for (int k = 0; k < 3; ++k) {
+        P *= n3[k] + 2 * H;
+        grid *= g.per[k] ? n3[k] : fft_size(n3[k] + Smax);
+    }
+    const double cost =
+        std::min(shell_march_cost(false, g, M, Smax, false), shell_march_cost(false, g, M, Smax, true));
+    const double march = 1.1e-3 * cost * points / M + 12.0 + 1.8e-6 * (M + M * M) * P + 2.5 * P / (double)g.N;
+    const double ffts = 72.0 + 6.3e-6 * (5 * M + 4 * (double)c->pairs.size()) * grid;
+    return march < 1.15 * ffts;
 }
 
 // The pairs as the spectral kernels see them (shell index into the table of distinct shells), the

@@ -130,3 +130,24 @@ def test_odd_grids(shape, periodic, sig, prec, tol):
         for x, y in zip(g.adjoint_flux_gradient(3, 2, 0, 7), d.adjoint_flux_gradient(3, 2, 0, 7)):
             x, y = np.asarray(x), np.asarray(y)
             assert np.abs(x - y).max() <= 1e-10 * max(np.abs(y).max(), 1e-30)
+
+
+@pytest.mark.parametrize("shape,sig,prec,method", [
+    ((1024, 512, 1), (6.0,), "fp32", "spectral"),  # one plane: marches of 2 S + 1 planes, or tiles of one row in four
+    ((1024, 512, 1), (4.0, 6.0), "fp32", "spectral"),
+    ((4096, 16, 16), (8.0,), "fp32", "spectral"),
+    ((512, 512, 8), (6.0,), "fp32", "direct"),
+    ((64, 64, 64), (8.0,), "fp32", "direct"),
+    ((96, 96, 96), (8.0,), "fp32", "direct"),
+    ((96, 40, 40), (4.0, 6.0), "fp32", "direct"),
+    ((512, 256, 1), (7.0,), "fp64", "direct"),
+    ((1024, 512, 1), (3.0,), "fp32", "direct"),    # small shells: never the FFTs
+])
+def test_automatic_choice_on_thin_lattices(shape, sig, prec, method):
+    """AUTO is the form that measured faster on these lattices (K2 + K3 of both, by 10% and more)."""
+    N, M = int(np.prod(shape)), len(sig)
+    n0 = 6.0 * 0.1 / (np.pi * sum(s ** 3 for s in sig))
+    arr = dict(solid=np.zeros(N, np.uint8), V=np.zeros((M, N)), phi=np.zeros(N), amp=np.zeros(N),
+               n=np.full((M, N), n0))
+    w = dict(shape=shape, periodic=(1, 1, 1), sigma=list(sig), tau=[1.0] * M, body=[(0.0, 0.0, 0.0)] * M)
+    assert setup_gpu(w, arr, prec).shell_method() == method
