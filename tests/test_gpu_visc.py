@@ -98,3 +98,22 @@ def test_shifted_16bit_storage_with_viscous_force(prec, tol):
     obs = o.observe()
     for a in range(2):
         assert rel_err(g.density(a), obs["n"][a]) <= tol
+
+
+@pytest.mark.parametrize("prec,tol", [("fp64", 1e-12), ("fp32", 1e-5)])
+@pytest.mark.parametrize("shape,periodic,sig", [((19, 11, 9), (1, 1, 1), (3.0,)), ((5, 3, 2), (1, 0, 1), (2.0, 4.0))])
+def test_blocks_that_the_lattice_does_not_fill(shape, periodic, sig, prec, tol):
+    """A gather's block takes 32 nodes: lattices of 1881 and of 30, with solid nodes."""
+    N, M = int(np.prod(shape)), len(sig)
+    rng = np.random.default_rng(29)
+    solid = (rng.random(N) < 0.1).astype(np.uint8)
+    n0 = 6.0 * 0.1 / (np.pi * sum(s ** 3 for s in sig))
+    arr = dict(solid=solid, V=np.zeros((M, N)), phi=np.zeros(N), amp=np.zeros(N),
+               n=n0 * (1.0 + 0.2 * (rng.random((M, N)) - 0.5)) * (solid == 0)[None, :])
+    w = dict(shape=shape, periodic=periodic, sigma=list(sig), tau=[1.0] * M, body=[(1e-4, 0.0, 0.0)] * M)
+    g, o = setup_gpu(w, arr, prec, visc=True), setup_oracle(w, arr, visc=True)
+    g.step(3)
+    o.step(3)
+    for a in range(M):
+        for got, ref in zip(g.populations(a), o.get_populations(a)):
+            assert rel_err(np.asarray(got).reshape(-1), np.asarray(ref).reshape(-1)) <= tol
