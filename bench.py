@@ -49,6 +49,9 @@ QPOP = 19
 # change to g's 18, and of f and g together the rest populations 6, the axis pairs 42 and the edge pairs 108.  The
 # 57 additions of the moments run on the integer pipe (lbe_block_sum.cuh).  (Each population by itself took 864.)
 K4_FLOPS_PER_NODE_SPECIES = 31 + 81 + 18 + 6 + 42 + 108
+# FP32-pipe operations (add, multiply, multiply-add) of the FP32 collide (Collision in lbe_collide.cuh): moments 57,
+# recovery and velocities 25, constants 61, rest populations 6, three axis pairs of 22 and six edge pairs of 24.
+K4_FP32_OPS_PER_NODE_SPECIES = 57 + 25 + 61 + 6 + 3 * 22 + 6 * 24
 STAGE_STEPS = 20  # steps of the instrumented pass that gives the per-stage times
 
 WORKLOAD_TEXT = {
@@ -181,6 +184,20 @@ def shell_flops_per_node(S):
     for e in half_shell(S):
         f += 2 + 4 * sum(1 for v in e if v != 0)
     return f + 3 * 4 + 2
+
+
+def march_ops(S):
+    """FP32-pipe operations (add, multiply, multiply-add) that the marching shell kernel executes per output and field:
+    the points (+-X, +-Y) of a plane combined once, one operation per component and height |Z| that they reach,
+    and the running sums.  Halo planes are not counted."""
+    n = 0
+    for Y in range(S + 1):
+        for X in range(S + 1):
+            Z = [z for z in range(S + 1) if S * S - S + 1 <= X * X + Y * Y + z * z <= S * S + S]
+            if Z:
+                n += (0 if X == 0 and Y == 0 else 2 if X == 0 or Y == 0 else 7)
+                n += sum((X > 0) + (Y > 0) + (z > 0) for z in Z)
+    return n + 3 + 2 * (2 * S - 1) + (2 * S - 2) + 1
 
 
 def ball_count(radius):
@@ -502,8 +519,11 @@ def step_roofline(w, prec, N, M, sb, ms_step, stage_ms, kernels, hbm, fp_peak_tf
       populations (76 per node and species) alone and with C, F and n (7 words per node and species) and
       the link mask (4 B per node).  Flops: the shell sums (shell_flops_per_node per ordered pair), the
       collision (K4_FLOPS_PER_NODE_SPECIES per node and species) and the ball sums of the contact values
-      (one add per ball point).  Computed for the direct shell form; the spectral form's transforms are
-      not counted here.
+      (one add per ball point).  FP64: without the shell sums, which run on the integer pipe.  Computed for
+      the direct shell form; the spectral form's transforms are not counted here.
+    - roof_executed_ms (FP32 arithmetic): the same with the operations that the shell and collide kernels execute
+      (march_ops, K4_FP32_OPS_PER_NODE_SPECIES; the definition's count above is larger), a multiply-add as
+      one of the FP32 pipe's operations; the ball sums are left out.
     - stage_roof_sum_ms: the sum over stages of each stage's own bound (stage time x its roofline
       fraction), since the stages run one after another; the stages without a fraction (the flux
       reduction) are left out."""
@@ -515,13 +535,19 @@ def step_roofline(w, prec, N, M, sb, ms_step, stage_ms, kernels, hbm, fp_peak_tf
            "full_frac_of_measured_hbm": full_bytes / (ms_step * 1e-3) / 1e9 / hbm}
     if shell_method == "direct" and fp_peak_tflops:
         S_list = [int(round(0.5 * (w["sigma"][a] + w["sigma"][b]))) for a in range(M) for b in range(M)]
-        flops = N * (sum(shell_flops_per_node(S) for S in S_list) + M * K4_FLOPS_PER_NODE_SPECIES
+        flops = N * ((sum(shell_flops_per_node(S) for S in S_list) if prec != "fp64" else 0)
+                     + M * K4_FLOPS_PER_NODE_SPECIES
                      + sum(ball_count(0.5 * s_) for s_ in w["sigma"] if s_ > 0))
         t_b = full_bytes / (hbm * 1e9) * 1e3
         t_f = flops / (fp_peak_tflops * 1e12) * 1e3
         out.update({"flops_per_step": flops, "roof_bytes_ms": t_b, "roof_flops_ms": t_f,
                     "roof_max_ms": max(t_b, t_f), "frac_of_roof_max": max(t_b, t_f) / ms_step,
                     "bound": "flops" if t_f >= t_b else "bytes"})
+        if prec != "fp64":
+            ops = N * (2 * sum(march_ops(S) for S in S_list) + M * K4_FP32_OPS_PER_NODE_SPECIES)
+            t_e = max(t_b, ops / (0.5 * fp_peak_tflops * 1e12) * 1e3)
+            out.update({"executed_ops_per_step": ops, "roof_executed_ms": t_e,
+                        "frac_of_roof_executed": t_e / ms_step})
     parts = {k: stage_ms[k] * kernels[k]["frac"] for k in ("density", "contact", "shell", "collide")
              if k in stage_ms and k in kernels and kernels[k].get("frac")}
     if parts:
@@ -588,15 +614,22 @@ def shell_roofline(w, prec, N, M, stage, peaks, peaks_kind, sms, wname, shell_me
         achieved = per_launch_flops / (per_launch_ms * 1e-3) / 1e12
         clk = float(peaks.get("sm_max_mhz", 2070.0))
         peak = sms * FP32_LANES_PER_SM * 2 * clk * 1e6 / 1e12 if prec != "fp64" else None
-        # flops by the definition's half shell; the kernel shares work between outputs and executes fewer
+        # achieved: flops by the definition's half shell; the kernel shares work between outputs and executes fewer,
+        # and the fraction is that of the operations it executes (a multiply-add is one) in the FP32 pipe's
         name = "k_shell_fixed (K3 mean-field shell force, fixed point)" if prec == "fp64" else \
             "k_shell_march (K3 mean-field shell force)"
         roof = {"kernel": name, "bound": "alu", "achieved": achieved,
-                "peak": peak, "unit": "TFLOP/s", "frac": (achieved / peak) if peak else None,
+                "peak": peak, "unit": "TFLOP/s", "frac": None,
                 "traffic": traffic_for("shell", wname, prec), "algorithmic_flops_per_launch": per_launch_flops,
                 "launches": dom_n, "avg_launch_ms": per_launch_ms,
                 "peak_source": "FP32 FMA: %d SMs (the device's multiprocessor count) x 128 lanes x 2 flop x "
                                "%.0f MHz (max SM clock)" % (sms, clk)}
+        if peak:
+            ops = 2 * sum(march_ops(S) for S in S_list) * N / len(S_list)
+            roof.update({"executed_ops_per_launch": ops, "frac_by_definition": achieved / peak,
+                         "frac": ops / (per_launch_ms * 1e-3) / (0.5e12 * peak),
+                         "frac_is": "executed FP32-pipe operations over 128 lanes x SMs x clock; achieved / peak by the "
+                                    "definition's flops is frac_by_definition"})
     return roof
 
 

@@ -117,3 +117,22 @@ def test_shell_roofline_in_both_forms_and_its_kernels_entry():
         assert out["shell"]["frac"] == roof["frac"] and key in out["shell"]
     c = bench.collide_roofline(N, M, 4, (4.0, 4), peaks, "measured", "x", "fp32")
     assert c["algorithmic_bytes_per_launch"] == N * M * 304 and abs(c["avg_launch_ms"] - 1.0) < 1e-12
+
+
+def test_shell_fraction_counts_what_the_kernel_executes():
+    """At most 1 whatever the time a kernel could take: operations over the pipe's rate, and the FP64 step's flops
+    without the shell sums that run on integers."""
+    # diameter 1: the points (+-1, 0, 0), (0, +-1, 0), (0, 0, +-1), (+-1, +-1, 0) ...: counted by hand
+    assert bench.march_ops(1) == 26
+    assert bench.march_ops(6) == 439
+    N, M = 1000, 1
+    w = {"sigma": [6.0], "shape": (10, 10, 10), "periodic": (1, 1, 1)}
+    peaks = {"hbm_gbs": 1000.0, "sm_max_mhz": 2070.0}
+    t = 2 * 439 * N / (152 * 128 * 2070e6)  # the pipe's own time for these operations
+    r = bench.shell_roofline(w, "fp32", N, M, (t * 1e3, 1), peaks, "measured", 152, "x", "direct")
+    assert abs(r["frac"] - 1.0) < 1e-9 and r["frac_by_definition"] > 1.5
+    s = bench.step_roofline(w, "fp64", N, M, 8, 1.0, {}, {}, 1000.0, 1.25, "direct")
+    assert s["flops_per_step"] == N * (bench.K4_FLOPS_PER_NODE_SPECIES + bench.ball_count(3.0))
+    e = bench.step_roofline(w, "fp32", N, M, 4, 1.0, {}, {}, 1e9, 80.0, "direct")
+    assert e["executed_ops_per_step"] == N * (2 * 439 + bench.K4_FP32_OPS_PER_NODE_SPECIES)
+    assert abs(e["roof_executed_ms"] - e["executed_ops_per_step"] / 40e12 * 1e3) < 1e-15
