@@ -207,6 +207,17 @@ def ball_count(radius):
                if x * x + y * y + z * z <= radius * radius)
 
 
+def contact_smem_bytes(sigma, prec):
+    """Bytes of shared memory that the contact kernel reads per node for the ball of one species: of a plane the rows of
+    the ball's widest section, FP32 as 8-byte loads that serve two nodes."""
+    d2 = int(sigma * sigma / 4 + 1e-9)
+    total = 0.0
+    for dy in range(-math.isqrt(d2), math.isqrt(d2) + 1):
+        e = math.isqrt(d2 - dy * dy)
+        total += (2 * e + 1) * 8 if prec == "fp64" else ((e + 1) // 2 * 2 + 1) * 8 / 2
+    return total
+
+
 def source_hash(files):
     h = hashlib.sha256()
     for f in files:
@@ -443,10 +454,11 @@ def kernel_rooflines(stages, w, prec, N, M, sb, hbm, roof, sms, clk, shell_metho
     K4: reads and writes f~ and g~ (76 populations) per node and species; HBM bound with 32- and 16-bit
     storage; with FP64 storage it is bound by GB300's FP64 rate, so it also carries the FP64-rate roofline
     of K4_FLOPS_PER_NODE_SPECIES flops per node and species against the nominal FP64 rate.
-    K2, stencil form: the sum_b |B_b| ball points per node as shared-memory loads of the padded densities (the
-    kernel shares sums between heights and reads fewer), against the shared-memory load bandwidth (32 banks x 4 B per clock per SM); in spectral form its fields through
-    HBM.  K3: the shell stage's roofline in the form in use (stencil: algorithmic flops against the FP32
-    FMA peak; spectral: its fields through HBM, or FP64 transform flops)."""
+    K2, stencil form: the sum_b |B_b| ball points per node as shared-memory loads of the padded densities, against
+    the shared-memory load bandwidth (32 banks x 4 B per clock per SM); the kernel shares sums between heights
+    and reads fewer: frac_executed.  In spectral form its fields through HBM.  K3: the shell stage's roofline
+    in the form in use (stencil: executed operations against the FP32 pipe; spectral: its fields through HBM, or
+    FP64 transform flops)."""
     rb = 8 if prec == "fp64" else 4
     out = {}
     name = w.get("name", "")
@@ -486,7 +498,10 @@ def kernel_rooflines(stages, w, prec, N, M, sb, hbm, roof, sms, clk, shell_metho
             out["contact"] = {"bound": "smem", "algorithmic_smem_bytes_per_launch": b, "avg_launch_ms": t * 1e3,
                               "achieved_gbs": b / t / 1e9, "peak_gbs": peak, "frac": b / t / 1e9 / peak,
                               "peak_source": "shared-memory loads: %d SMs x 128 B/clock x %.0f MHz" % (sms, clk),
-                              "note": "%d points per node by the definition; the kernel reads a plane's discs" % loads,
+                              "note": "%d points per node by the definition; the kernel reads a plane's discs, which "
+                                      "is what frac_executed counts (no unit's limit)" % loads,
+                              "frac_executed": N * sum(contact_smem_bytes(s, prec) for s in w["sigma"] if s > 0)
+                              / t / 1e9 / peak,
                               "traffic": traffic_for("contact", name, prec)}
         else:
             # spectral contact stage: M densities embedded and transformed forward, ball spectra applied,
@@ -548,7 +563,7 @@ def step_roofline(w, prec, N, M, sb, ms_step, stage_ms, kernels, hbm, fp_peak_tf
             t_e = max(t_b, ops / (0.5 * fp_peak_tflops * 1e12) * 1e3)
             out.update({"executed_ops_per_step": ops, "roof_executed_ms": t_e,
                         "frac_of_roof_executed": t_e / ms_step})
-    parts = {k: stage_ms[k] * kernels[k]["frac"] for k in ("density", "contact", "shell", "collide")
+    parts = {k: stage_ms[k] * kernels[k].get("frac_executed", kernels[k]["frac"]) for k in ("density", "contact", "shell", "collide")
              if k in stage_ms and k in kernels and kernels[k].get("frac")}
     if parts:
         out["stage_roof_ms"] = parts

@@ -9,10 +9,10 @@
 // state per thread shrinks to one species', so more warps share an SM, and nothing is pulled twice.
 // One species: one thread per node, 32 consecutive nodes per warp, u = J/n.
 //
-// Bounds: HBM with FP32 storage (783 us for the 512x128x128 channel's 5.1 GB, 96% of the measured copy bandwidth; 886
+// Bounds: HBM with FP32 storage (785 us for the 512x128x128 channel's 5.1 GB, 96% of the measured copy bandwidth; 886
 // before the collision's pairs shared their parts); the FP64 pipe in FP64 (256x64x64 channel 2.55 -> 0.81 ms: 1.20
 // with shared pairs and two CTAs, 0.99 with the moments on the integer pipe, the rest by Collision64); issue with 16-bit storage
-// (channel 887 -> 701 us, half of them integer instructions for addresses and conversions).  Three species: the
+// (channel 887 -> 695 us, half of them integer instructions for addresses and conversions).  Three species: the
 // kernel with one thread per node for all of them pulled every population twice (90x75x66 166 -> 86 us).
 #include <math.h>
 

@@ -24,8 +24,8 @@
 // sum over the ball's points read 123 values for one.  The halo's periodic images are written by their own node,
 // one offset for all fields (an address per field and image doubled the time of the tiles at the edges).
 // Contact stage on GB300, before (sum over the ball's points from a ring of 2R + 2 planes; spectral on the wells)
-// and now: 512x128x128 channel of diameters 4 and 6 251 -> 91 us, 256^3 well of diameter 6 373 -> 127 us, 64^3
-// well 50 -> 14 us, 90x75x66 with diameters 2, 4 and 6 129 -> 34 us.
+// and now: 512x128x128 channel of diameters 4 and 6 251 -> 96 us, 256^3 well of diameter 6 373 -> 122 us, 64^3
+// well 50 -> 14 us, 90x75x66 with diameters 2, 4 and 6 129 -> 31 us, 1024x1024x1 of diameters 4 and 6 158 -> 103 us.
 #pragma once
 #include <algorithm>
 #include <atomic>
@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(CT_THREADS)
                         }
                     }
                     // the periodic images inside the halo: one offset for all fields; along y and z a pair stays one
-                    // store (two stores of every other value: 330 instead of 203 us on 1024x1024x1, two species)
+                    // store (two stores of every other value: 310 instead of 103 us on 1024x1024x1, two species)
                     const Images iz = images(z, g.nz, g.H, g.per[2]);
                     if (edge || (iz.k0 | iz.k1) != 0) {
                         for (int kz = iz.k0; kz <= iz.k1; ++kz)

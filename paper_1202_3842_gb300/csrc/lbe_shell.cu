@@ -1,6 +1,6 @@
 // Dispatch of the shell-force kernels by precision and pair diameter, and the host-side shell helpers.
 // FP32: every pair in one launch of the marching kernel (lbe_shell_march.cuh), instantiated for the largest
-// pair diameter 4, 6 or 8 (the registers of a thread grow with it: 128, 166, 222, so four, three and two
+// pair diameter 4, 6 or 8 (the registers of a thread grow with it: 128, 162, 206, so four, three and two
 // blocks of 128 threads per SM).  FP64: the same march in fixed point (lbe_shell_fixed.cuh) on the integer images
 // of the padded fields that k_to_fixed writes.
 #include "lbe_device.cuh"

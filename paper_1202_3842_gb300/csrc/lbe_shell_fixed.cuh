@@ -21,12 +21,15 @@
 // 8.4e-15; diameter 6 1.15e-15, 1.08e-15, 1.3e-14; diameter 7 1.5e-15, 1.3e-15, 1.2e-14; 48^3 well of diameter 6
 // after 50 steps 2.65e-16, 2.61e-16, 3.3e-16; 48x24x24 channel of diameters 4 and 6 6.5e-16, 6.6e-16, 6.8e-16.
 //
-// Shell stage on GB300: 256x64x64 channel of diameters 4 and 6 12.2 ms (stencil) and 3.12 ms (FFTs) -> 0.85 ms;
-// 48^3 well of diameter 4 114 us (FFTs) -> 46; 24^3 well of diameter 3 429 us (stencil, six blocks) -> 17.
+// Shell stage on GB300: 256x64x64 channel of diameters 4 and 6 12.2 ms (stencil) and 3.12 ms (FFTs) -> 0.86 ms;
+// 48^3 well of diameter 4 114 us (FFTs) -> 46; 24^3 well of diameter 3 429 us (stencil, six blocks) -> 16;
+// 512x512x1 of diameter 6 265 us (FFTs) -> 190, along y.
 // At diameter 6 a warp takes 1400 instructions for 32 outputs of one field and plane; the integer pipe is busy
 // half of the cycles at 2.6 warps per scheduler, the rest is latency of the multiply chains.
 //
-// One output and one field per thread: the running sums take 12 S registers, the plane's B about 60 at S = 6.
+// One output and one field per thread: the running sums take 12 S registers, the plane's B about 60 at S = 6.  Where the
+// largest diameter is 5 or 6, the 168 registers of three blocks per SM do not hold them all (288 bytes of spill stores and
+// 148 of loads in the code); up to 4 and at 7 nothing spills.
 #pragma once
 #include "lbe_launch.h"
 #include "lbe_march.cuh"

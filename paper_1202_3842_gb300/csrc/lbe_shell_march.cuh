@@ -23,13 +23,23 @@
 // S = 6), and odd X take their operands from the halves of two loads (scalar adds, same pipe time).
 // The two fields of a pair run in separate warps of a block; P reaches the warps that finish C through
 // shared memory.  What C's epilogue reads from global memory is loaded one plane ahead (read in the plane's
-// own pass, its latency showed: 1190 instead of 1010 us below).
+// own pass, its latency showed: 1190 instead of 1010 us on the 512x128x128 channel).
+//
+// The march goes along z with tiles of 32 x 4 nodes in x and y, or along y with tiles in x and z where few nodes lie
+// along z (march_axes): each cut of a march reads 2S planes again.
 //
 // Shell stage on GB300, against the half-shell stencils it replaces (y-blocked for diameters 4 to 6, z-blocked
-// else; spectral on the wells): 512x128x128 channel of diameters 4 and 6 1566 -> 1010 us, 256^3 well of diameter
-// 6 776 -> 640 us, 64^3 well 50 -> 36 us, 128x32x32 channel 184 -> 46 us, 90x75x66 with diameters 2, 4 and 6
-// 311 -> 166 us.  On the 160^3 well the FP32 pipe is busy 64% of the active cycles at 2.2 warps per scheduler
-// (164 registers); the rest is dependent issue ("wait" 0.9 cycles per instruction).
+// else; spectral on the wells): 512x128x128 channel of diameters 4 and 6 1566 -> 996 us, 256^3 well of diameter
+// 6 776 -> 638 us, 64^3 well 50 -> 35 us, 128x32x32 channel 184 -> 45 us, 90x75x66 with diameters 2, 4 and 6
+// 311 -> 163 us, 1024x1024x1 of diameter 6 220 -> 177 us, of diameter 8 250 -> 289 us.  The channel's operations
+// (439 per output and field at diameter 6, without the halo planes) take the FP32 pipe 55% of that time.  On the 160^3 well the pipe is busy 64% of the active cycles at 2.2 warps per scheduler
+// (162 registers); the rest is dependent issue ("wait" 0.9 cycles per instruction).
+//
+// Error of C in FP32 against FP64, rms over the root of the sum of squares on the shell (half-shell stencils in
+// brackets): 1% noise, diameter 6, 3.5e-8 (8.1e-8); density over one decade along x 4.8e-7 1.2e-7 2.3e-7 in x, y, z
+// (6.1e-7 1.4e-7 1.4e-7), over three, where it is 1e-3 to 1e-2 of its largest, 4.1e-5 6.9e-7 2.0e-6 (4.1e-5 6.9e-7
+// 6.6e-7: there the densities themselves, stored as deviations from n0, are off by 6e-5).  z sums like values that
+// cancel between planes.
 #pragma once
 #include "lbe_launch.h"
 #include "lbe_march.cuh"

@@ -136,3 +136,14 @@ def test_shell_fraction_counts_what_the_kernel_executes():
     e = bench.step_roofline(w, "fp32", N, M, 4, 1.0, {}, {}, 1e9, 80.0, "direct")
     assert e["executed_ops_per_step"] == N * (2 * 439 + bench.K4_FP32_OPS_PER_NODE_SPECIES)
     assert abs(e["roof_executed_ms"] - e["executed_ops_per_step"] / 40e12 * 1e3) < 1e-15
+
+
+def test_contact_fraction_counts_what_the_kernel_reads():
+    # diameter 6: 19 loads of 8 bytes for two nodes; diameter 4: 11; FP64 one value of 8 bytes per point of the disc
+    assert bench.contact_smem_bytes(6.0, "fp32") == 19 * 8 / 2 and bench.contact_smem_bytes(4.0, "fp32") == 11 * 8 / 2
+    assert bench.contact_smem_bytes(6.0, "fp64") == (7 + 2 * (5 + 5 + 1)) * 8
+    w = {"sigma": [4.0, 6.0], "shape": (10, 10, 10), "periodic": (1, 0, 0)}
+    k = bench.kernel_rooflines({"contact": (1.0, 4)}, w, "fp32", 1000, 2, 4, 1000.0, None, 152, 2070.0, "direct")
+    assert k["contact"]["frac_executed"] < k["contact"]["frac"]
+    s = bench.step_roofline(w, "fp32", 1000, 2, 4, 3.0, {"contact": 0.25}, k, 1000.0, 80.0, "direct")
+    assert abs(s["stage_roof_ms"]["contact"] - 0.25 * k["contact"]["frac_executed"]) < 1e-15
