@@ -351,10 +351,10 @@ bool spectral_cheaper(const lbe_ctx *c, bool f64, double stencil_factor = 1.0) {
 
 // Whether the marching kernels (lbe_shell_march.cuh, lbe_shell_fixed.cuh, lbe_contact.cuh) take the forward force
 // under LBE_SHELL_AUTO where the rule above is for the spectral form.  K2 + K3 on GB300, march against FFTs:
-// - FP64: the march on every lattice measured (256x64x64 channel of diameters 4 and 6 1125 against 3870 us, 48^3 of
+// - FP64: the march on every lattice measured (256x64x64 channel of diameters 4 and 6 1128 against 3870 us, 48^3 of
 //   diameter 7 189 against 199, 512x512x1 of diameter 6 345 against 418);
-// - FP32: the march on 256^3 of diameter 6 (738 against 1146), 192^3 of diameter 8 (533 against 602), the 512x128x128
-//   channel of diameters 4 and 6 (1100 against 2390), 64^3 of diameter 8 (70 against 89); the FFTs where its tiles or its
+// - FP32: the march on 256^3 of diameter 6 (760 against 1145), 192^3 of diameter 8 (560 against 602), the 512x128x128
+//   channel of diameters 4 and 6 (1092 against 2395), 64^3 of diameter 8 (70 against 89); the FFTs where its tiles or its
 //   2S extra planes are mostly empty (1024x1024x1 of diameter 6 239 against 129, of diameters 4 and 6 624 against
 //   210; 4096x16x16 of diameter 8 170 against 122).  Both sides as fits to 70 lattices, in us:
 //     march: 1.1e-3 shell_march_cost x points per species + 12 + 1.8e-6 padded field values + 2.5 P / N (the images of
