@@ -154,34 +154,6 @@ lbe_status cuda_fail(lbe_ctx *c, cudaError_t e, const char *where) {
         if (_e != cudaSuccess) return cuda_fail(c, _e, where); \
     } while (0)
 
-lbe_status dev_alloc(lbe_ctx *c, Buf &b, size_t bytes) {
-    if (b.p && b.bytes >= bytes) return LBE_OK;
-    if (b.p) {
-        if (c->have_alloc)
-            c->alloc.free(b.p, b.bytes, c->stream, c->alloc.user);
-        else
-            cudaFreeAsync(b.p, c->stream);
-        b.p = nullptr;
-        b.bytes = 0;
-    }
-    if (bytes == 0) bytes = 16;
-    bytes = (bytes + 255) / 256 * 256;
-    void *p = nullptr;
-    if (c->have_alloc) {
-        p = c->alloc.alloc(bytes, c->stream, c->alloc.user);
-        if (!p) return fail(c, LBE_ERR_OOM, "device allocation of " + std::to_string(bytes) + " bytes failed");
-    } else {
-        cudaError_t e = cudaMallocAsync(&p, bytes, c->stream);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            return fail(c, LBE_ERR_OOM, std::string("cudaMallocAsync: ") + cudaGetErrorString(e));
-        }
-    }
-    b.p = p;
-    b.bytes = bytes;
-    return LBE_OK;
-}
-
 void dev_free(lbe_ctx *c, Buf &b) {
     if (!b.p) return;
     if (c->have_alloc)
@@ -190,6 +162,36 @@ void dev_free(lbe_ctx *c, Buf &b) {
         cudaFreeAsync(b.p, c->stream);
     b.p = nullptr;
     b.bytes = 0;
+}
+
+// Memory of at least `bytes` in b.  Where none is left, the fixed-point images make room: the FP64 shell sums do
+// without them (k_shell_wide), so that they never keep a call from running.
+lbe_status dev_alloc(lbe_ctx *c, Buf &b, size_t bytes) {
+    if (b.p && b.bytes >= bytes) return LBE_OK;
+    dev_free(c, b);
+    if (bytes == 0) bytes = 16;
+    bytes = (bytes + 255) / 256 * 256;
+    for (;;) {
+        void *p = nullptr;
+        cudaError_t e = cudaSuccess;
+        if (c->have_alloc) {
+            p = c->alloc.alloc(bytes, c->stream, c->alloc.user);
+        } else if ((e = cudaMallocAsync(&p, bytes, c->stream)) != cudaSuccess) {
+            cudaGetLastError();
+            p = nullptr;
+        }
+        if (p) {
+            b.p = p;
+            b.bytes = bytes;
+            return LBE_OK;
+        }
+        if (!c->fix.p) {
+            return fail(c, LBE_ERR_OOM,
+                        c->have_alloc ? "device allocation of " + std::to_string(bytes) + " bytes failed"
+                                      : std::string("cudaMallocAsync: ") + cudaGetErrorString(e));
+        }
+        dev_free(c, c->fix);
+    }
 }
 
 #define TRY(x)                          \
@@ -712,7 +714,8 @@ lbe_status prepare(lbe_ctx *c) {
         if (!c->spectral) TRY(dev_alloc(c, c->gnpad, gnb));
         if (!c->spectral && !f64) TRY(dev_alloc(c, c->npad2, rb * c->M * g.P));
         if (!c->spectral && f64) {
-            TRY(dev_alloc(c, c->fix, 8 * (c->M + c->M * c->M) * g.P));
+            const lbe_status st = dev_alloc(c, c->fix, 8 * (c->M + c->M * c->M) * g.P);
+            if (st != LBE_OK && st != LBE_ERR_OOM) return st;
             TRY(dev_alloc(c, c->top, 4 * (c->M + c->M * c->M + 1)));
         }
         c->ref_dirty = true;
@@ -743,9 +746,11 @@ lbe_status prepare(lbe_ctx *c) {
             int bx = 0, by = 0;
             shell_box(f64, ps.S, &bx, &by);
             const int mby = c->march_swap ? 1 : by, mbz = c->march_swap ? by : 1;
-            TRY(make_map(c, &c->march_maps->n[ab], nb, bx, mby, false, mbz));
-            TRY(make_map(c, &c->march_maps->gn[ab], gn, bx, mby, false, mbz));
-            if (c->shell_wide) {
+            if (!f64 || c->fix.p) {
+                TRY(make_map(c, &c->march_maps->n[ab], nb, bx, mby, false, mbz));
+                TRY(make_map(c, &c->march_maps->gn[ab], gn, bx, mby, false, mbz));
+            }
+            if (f64) {
                 shell_wide_box(Smax, ps.S, &bx, &by);
                 TRY(make_map(c, &c->wide_maps->n[ab], (char *)c->npad.p + rb * ps.b * g.P, bx, by));
                 TRY(make_map(c, &c->wide_maps->gn[ab], (char *)c->gnpad.p + rb * ab * g.P, bx, by));
@@ -897,13 +902,17 @@ lbe_status force_stage_core(lbe_ctx *c, const void *pop, void *Pbase, void *xiba
     if (f64) {
         FixedArgs A{};
         fill(A, 0.0);
-        unsigned *wide = c->shell_wide ? (unsigned *)c->top.p + c->M + c->M * c->M : nullptr;
+        unsigned *wide = c->shell_wide || !c->fix.p ? (unsigned *)c->top.p + c->M + c->M * c->M : nullptr;
         A.top = (const unsigned *)c->top.p;
         A.wide = wide;
-        LAUNCH(launch_to_fixed(Smax, (const double *)c->npad.p, (const double *)c->gnpad.p, c->g.P, c->M, A.top, wide,
-                               (long long *)c->fix.p, c->stream),
-               "fixed-point fields");
-        LAUNCH(launch_shell_fixed(Smax, *c->march_maps, A, c->stream), "shell force kernel");
+        if (c->fix.p) {
+            LAUNCH(launch_to_fixed(Smax, (const double *)c->npad.p, (const double *)c->gnpad.p, c->g.P, c->M, A.top, wide,
+                                   (long long *)c->fix.p, c->stream),
+                   "fixed-point fields");
+            LAUNCH(launch_shell_fixed(Smax, *c->march_maps, A, c->stream), "shell force kernel");
+        } else {
+            CK(cudaMemsetAsync(wide, 1, 4, c->stream), "set the far-apart word");
+        }
         if (wide) LAUNCH(launch_shell_wide(Smax, *c->wide_maps, A, c->stream), "shell force of far-apart values");
     } else {
         ShellMarchArgs A{};

@@ -48,3 +48,48 @@ def test_fp64_force_is_exact_locally(kind, sig, shell):
     for a in range(M):
         scale = shell_scale(shape, sig, n.reshape(M, N), obs["g"], a)
         assert (np.abs(g.force(a) - obs["C"][a]) <= 1e-12 * scale).all()
+
+
+@pytest.mark.parametrize("short_of", ["images", "scratch"])
+@pytest.mark.parametrize("sig", [(3.0,), (2.0, 4.0)])
+def test_no_room_for_the_images(sig, short_of, monkeypatch):
+    """A device without room for the fixed-point images, or for a getter's scratch beside them: the stencil needs none."""
+    from paper_1202_3842_gb300 import lbe
+    shape, N, M = (20, 18, 16), 5760, len(sig)
+    H = (int(max(sig)) + 3) // 4 * 4
+    P = (shape[0] + 2 * H + 7) // 8 * 8 * (shape[1] + 2 * H) * (shape[2] + 2 * H)
+    size = {"images": 8 * (M + M * M) * P, "scratch": 8 * (4 * M * N + 4 * N)}[short_of]
+    refused = []
+
+    class Full(lbe.TorchAllocator):
+        def __init__(self, *args, **kw):
+            super().__init__(*args, **kw)
+            alloc = self._a
+
+            def _alloc(nbytes, stream, user):
+                if nbytes == (size + 255) // 256 * 256 and (short_of == "images" or not refused):
+                    refused.append(nbytes)
+                    return None
+                return alloc(nbytes, stream, user)
+
+            self._full = lbe._ALLOC_FN(_alloc)
+            self.struct = lbe.lbe_allocator(self._full, self._f, None)
+
+    rng = np.random.default_rng(4)
+    n0 = 6.0 * 0.12 / (np.pi * sum(s ** 3 for s in sig))
+    arr = dict(solid=np.zeros(N, np.uint8), V=np.zeros((M, N)), phi=np.zeros(N), amp=np.zeros(N),
+               n=n0 * (1.0 + 0.3 * (rng.random((M, N)) - 0.5)))
+    w = dict(shape=shape, periodic=(1, 1, 1), sigma=list(sig), tau=[1.0] * M, body=[(0.0, 0.0, 0.0)] * M)
+    o = setup_oracle(w, arr)
+    monkeypatch.setattr(lbe, "TorchAllocator", Full)
+    g = setup_gpu(w, arr, "fp64", shell="direct")
+    for _ in range(2):
+        obs = o.observe()
+        for a in range(M):
+            assert np.abs(g.force(a) - obs["C"][a]).max() <= 1e-12 * np.abs(obs["C"][a]).max()
+            assert np.abs(g.density(a) - obs["n"][a]).max() <= 1e-12 * n0
+            J = obs["J"][a].reshape(-1)
+            assert np.abs(np.asarray(g.momentum(a)).reshape(-1) - J).max() <= 1e-12 * np.abs(J).max()
+        g.step(3)
+        o.step(3)
+    assert refused
