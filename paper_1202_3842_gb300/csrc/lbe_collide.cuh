@@ -10,7 +10,8 @@
 //   even_f = kf + k2 (2s - t) t + (c.X9) s,  even_g = kg + k2 (2s - t) t + (c.G9) s,  s = c.u^a, t = c.u,
 //   odd_f  = c.Of,  odd_g = c.Og,
 // so a pair shares its dot products, and the constants carry om, inv and the edge links' weight 1/36 (or 1/n0,
-// below).  That is 14 flops per population where each population's own f_eq, S_f and update took 36.
+// below).  That is 24 operations for the four populations of an edge pair, f and g, where one population's own f_eq,
+// S_f and update took 36 flops.
 #pragma once
 #include <type_traits>
 #include <utility>
